@@ -5,9 +5,10 @@
 // one warp).  The tile's depth-ordered splat list is staged through shared
 // memory in batches of one splat per thread; a block-wide vote ends the walk
 // once every pixel has saturated.  The backward replays the same walk in
-// reverse from the stored final transmittance, recovering T_k by division,
-// and sums each splat's adjoint over the warp's pixels with shuffles before a
-// single vector atomic per warp and splat.
+// reverse from the stored final transmittance, recovering T_k by division, one
+// warp per group of pixels and piece of the list, two splats at a time.
+#include <climits>
+
 #include "tgs_common.cuh"
 
 namespace tgs {
@@ -57,14 +58,6 @@ __device__ __forceinline__ float splat_pow2(const float4& co, float dx, float dy
 
 // alpha of a splat at offset (dx, dy) from its centre; G receives exp(power).
 // Returns false when the splat is skipped (power > 0 or alpha < 1/255).
-__device__ __forceinline__ bool splat_alpha_p(const float4& co, float dx, float dy, float& alpha, float& G, float& p) {
-  p = splat_pow2(co, dx, dy);
-  if (p > 0.f) return false;
-  G = ex2_approx(p);
-  alpha = fminf(kAlphaMax, __fmul_rn(co.w, G));
-  return alpha >= kAlphaMin;
-}
-
 __device__ __forceinline__ bool splat_alpha(const float4& co, float dx, float dy, float& alpha, float& G) {
   const float p = splat_pow2(co, dx, dy);
   if (p > 0.f) return false;
@@ -805,72 +798,6 @@ size_t split_smem_bytes(int G) {
   return NW * 32 * sizeof(Splat) + (size_t)NW * G * (2 * sizeof(float4) + 2 * sizeof(int));
 }
 
-// The adjoints of a splat's centre and conic from the sums over its pixels of
-// dL/dpower times dx, dy, dx^2, dx dy, dy^2 (power = -(a dx^2 + c dy^2)/2 -
-// b dx dy, dx = px - x): dL/dx = a m1 + b m2, dL/dy = c m2 + b m1,
-// dL/da = -m3 / 2, dL/db = -m4, dL/dc = -m5 / 2 (co: the pre-scaled conic).
-__device__ __forceinline__ void power_moments_to_grad(const float4& co, float m1, float m2, float m3, float m4,
-                                                      float m5, float (&g)[5]) {
-  const float A = co.x * kInvA, Bc = co.y * kInvB, Cc = co.z * kInvA;
-  g[0] = A * m1 + Bc * m2;
-  g[1] = Cc * m2 + Bc * m1;
-  g[2] = -0.5f * m3;
-  g[3] = -m4;
-  g[4] = -0.5f * m5;
-}
-
-// Sum of v[0..7] over the warp, scattered: lane l ends with the total of
-// v[(l >> 2) & 7] (halving exchanges at distances 16, 8, 4, then a butterfly
-// over the last two bits): 9 shuffles instead of 40.
-__device__ __forceinline__ float warp_reduce_scatter8(const float (&v)[9], int lane) {
-  float a4[4], b2[2];
-  {
-    const bool up = lane & 16;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float send = up ? v[k] : v[4 + k];
-      const float keep = up ? v[4 + k] : v[k];
-      a4[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-  }
-  {
-    const bool up = lane & 8;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float send = up ? a4[k] : a4[2 + k];
-      const float keep = up ? a4[2 + k] : a4[k];
-      b2[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-  }
-  const bool up = lane & 4;
-  float c = (up ? b2[1] : b2[0]) + __shfl_xor_sync(0xffffffffu, up ? b2[0] : b2[1], 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
-  return c;
-}
-
-// Sum of v[0..3] over the warp, scattered: lane l ends with the total of
-// v[(l >> 3) & 3] (halving exchanges at distances 16 and 8, then a butterfly
-// over the last three bits): 6 shuffles.
-__device__ __forceinline__ float warp_reduce_scatter4(const float (&v)[4], int lane) {
-  float b2[2];
-  {
-    const bool up = lane & 16;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float send = up ? v[k] : v[2 + k];
-      const float keep = up ? v[2 + k] : v[k];
-      b2[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-  }
-  const bool up = lane & 8;
-  float c = (up ? b2[1] : b2[0]) + __shfl_xor_sync(0xffffffffu, up ? b2[0] : b2[1], 8);
-  c += __shfl_xor_sync(0xffffffffu, c, 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
-  return c;
-}
-
 // Where the backward also accumulates the error back-projection statistics of
 // Sec. 3.8 (Eq. 12): the per-pixel error e (from the loss) and the per-
 // Gaussian rows (E, W, D, 0) they are added to.
@@ -879,312 +806,493 @@ struct StatsK {
   float4* stats;
 };
 
-// Per-splat adjoints of a batch are summed over the block in shared memory
-// (acc, 9 floats per batch slot) and flushed once per block and splat with
-// vector atomics, instead of once per warp and splat.
-__device__ __forceinline__ void render_tile_bwd(const RasterArgs& a, int j, Splat* sm,
-                                                const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
-                                                const float* __restrict__ dL_drgb, float* __restrict__ grad2d) {
-  __shared__ int s_max_last;
-  float* acc = reinterpret_cast<float*>(sm + blockDim.x);
-  const int t = a.active_tiles ? a.active_tiles[j] : j;
-  const int p0 = a.pix_off[j], p1 = a.pix_off[j + 1];
-  const bool has_pix = p0 + (int)threadIdx.x < p1;
-  const int s = p0 + threadIdx.x;
-  float px = 0.f, py = 0.f, T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f;
-  int last = 0;
-  if (has_pix) {
-    const int l = a.pix_idx[s];
-    px = (float)((t % a.tiles_x) * TGS_TILE + (l & 15)) + 0.5f;
-    py = (float)((t / a.tiles_x) * TGS_TILE + (l >> 4)) + 0.5f;
-    T = T_final[s];
-    last = n_last[s];
-    g0 = dL_drgb[3 * s];
-    g1 = dL_drgb[3 * s + 1];
-    g2 = dL_drgb[3 * s + 2];
-  }
-  if (threadIdx.x == 0) s_max_last = 0;
-  __syncthreads();
-  if (last > 0) atomicMax(&s_max_last, last);
-  __syncthreads();
-  const int2 range = a.ranges[j];
-  const int end = range.x + s_max_last;  // no pixel blended anything past here
-  float S0 = a.bg[0], S1 = a.bg[1], S2 = a.bg[2];
-  const int B = blockDim.x;
-  const int lane = threadIdx.x & 31;
-  int warp_last = last;  // the warp skips splats none of its pixels blended
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) warp_last = max(warp_last, __shfl_xor_sync(0xffffffffu, warp_last, o));
-  const float2 band = warp_rows(last > 0, py);  // and splats that cannot reach its rows
-  // the next batch's records are fetched into registers while the current
-  // one is replayed, and the list entries (ids) of the batch after it
-  SplatRaw nxt;
-  int idn = 0;
-  {
-    const int k = end - B + (int)threadIdx.x;
-    if (end > range.x && k >= range.x) fetch_splat(a, a.vals[k], nxt);
-    if (end > range.x && k - B >= range.x) idn = a.vals[k - B];
-  }
-  for (int top = end; top > range.x; top -= B) {
-    const int lo = max(range.x, top - B);
-    const int cnt = top - lo;
-    __syncthreads();
-    // batch [top - B, top) was fetched into slot threadIdx.x - (B - cnt)
-    {
-      const int k = top - B + (int)threadIdx.x;
-      if (k >= range.x) finish_splat(nxt, sm[threadIdx.x - (B - cnt)]);
-#pragma unroll
-      for (int c = 0; c < 9; ++c) acc[9 * threadIdx.x + c] = 0.f;
-    }
-    __syncthreads();
-    {
-      const int k = top - 2 * B + (int)threadIdx.x;
-      if (k >= range.x) fetch_splat(a, idn, nxt);
-      if (k - B >= range.x) idn = a.vals[k - B];
-    }
-    const int qmax = min(cnt - 1, range.x + warp_last - 1 - lo);
-    for (int q = qmax; q >= 0; --q) {
-      const Splat sp = sm[q];
-      const int pos = lo + q - range.x;  // position in the tile list
-      float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      bool hit = false;
-      if (sp.yr.y < band.x || sp.yr.x > band.y) continue;  // warp-uniform: no pixel of the warp is reached
-      if (pos < last) {
-        const float dx = __fsub_rn(px, sp.xy.x), dy = __fsub_rn(py, sp.xy.y);
-        float alpha, G;
-        if (splat_alpha(sp.co, dx, dy, alpha, G)) {
-          hit = true;
-          T = __fdividef(T, 1.f - alpha);  // transmittance in front of this splat (1 - alpha >= 0.01)
-          const float wgt = alpha * T;
-          v[6] = wgt * g0;
-          v[7] = wgt * g1;
-          v[8] = wgt * g2;
-          const float e0 = sp.rgb.x - S0, e1 = sp.rgb.y - S1, e2 = sp.rgb.z - S2;
-          const float dalpha = T * (e0 * g0 + e1 * g1 + e2 * g2);
-          S0 += alpha * e0;  // the light seen behind the splat in front
-          S1 += alpha * e1;
-          S2 += alpha * e2;
-          if (alpha < kAlphaMax) {  // not clamped
-            v[5] = dalpha * G;
-            const float dpow = dalpha * alpha;
-            const float tx = dpow * dx, ty = dpow * dy;
-            v[0] = tx;  // the moments of dL/dpower; the conic is applied per splat
-            v[1] = ty;
-            v[2] = tx * dx;
-            v[3] = tx * dy;
-            v[4] = ty * dy;
-          }
-        }
-      }
-      if (__any_sync(0xffffffffu, hit)) {
-        const float r8 = warp_reduce_scatter8(v, lane);
-        const float r9 = warp_sum(v[8]);
-        if ((lane & 3) == 0) atomicAdd(acc + 9 * q + ((lane >> 2) & 7), r8);
-        else if (lane == 1) atomicAdd(acc + 9 * q + 8, r9);
-      }
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-      const float* r = acc + 9 * threadIdx.x;
-      if (r[0] != 0.f || r[1] != 0.f || r[2] != 0.f || r[3] != 0.f || r[4] != 0.f || r[5] != 0.f ||
-          r[6] != 0.f || r[7] != 0.f || r[8] != 0.f) {
-        const Splat& sq = sm[threadIdx.x];
-        float* gp = grad2d + 12 * (size_t)__float_as_int(sq.rgb.w);
-        float gc[5];
-        power_moments_to_grad(sq.co, r[0], r[1], r[2], r[3], r[4], gc);
-        red_add_v4(gp, gc[0], gc[1], gc[2], gc[3]);
-        red_add_v4(gp + 4, gc[4], r[5], r[6], r[7]);
-        atomicAdd(gp + 8, r[8]);
-      }
-    }
-  }
-}
-
-__global__ void k_render_bwd(RasterArgs a, const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
-                             const float* __restrict__ dL_drgb, float* __restrict__ grad2d) {
-  extern __shared__ Splat sm[];
-  const int j = blockIdx.x;
-  if (j >= *a.n_active) return;
-  render_tile_bwd(a, j, sm, T_final, n_last, dL_drgb, grad2d);
-}
-
-// Split backward, one warp per piece: piece c of tile j is list positions
-// [c E, (c + 1) E) (E = kCkptEvery), or from n_slots E to the end for
-// c = n_slots, replayed for every sampled pixel of the tile, PPL pixels per
-// lane (pixel p0 + lane + 32 u).  A pixel whose last blended splat lies in
-// the piece starts from (T_final, bg); one whose walk goes on past it starts
-// from the forward's checkpoint at the piece's back edge, with the light
-// from behind recovered as S = (out - C) / T (out = T-weighted colours +
-// T_final bg).  The lane first sums its pixels' adjoints of a splat in
-// registers, so one warp reduction serves 32 PPL pixels, and the warp's
-// totals go straight to the Gaussian's gradient row (two vector atomics and
-// one scalar).  Warps never wait on each other: each stages its splats, one
-// per lane, in its own slice of shared memory (sm, 32 entries).
+// ---------------------------------------------------------------------------
+// The compositing adjoint.  A warp takes one item: a group of at most 32 PPL
+// sampled pixels of a tile (PPL per lane) and a piece of the tile's list.  It
+// walks the piece from the back in chunks of 32 positions, keeps the splats
+// that can reach the group's rectangle, and replays them two at a time, in
+// packed fp32 arithmetic (the two splats of a pair in the halves of a
+// register pair, one issue slot per operation): only a pixel's transmittance
+// T and the light from behind it, R = sum_{j behind} w_j c_j . g + T_final
+// bg . g, go through the two one after the other:
+//   T_k = T / (1 - alpha),  dL/dalpha = T_k c . g - R / (1 - alpha),
+//   R += w c . g  (w = alpha T_k).
+// The lane sums a pair's adjoints over its pixels in registers; one warp
+// reduction then serves both splats (21 shuffles and two atomic instructions
+// a pair), so the work per splat and 32 pixels falls with PPL.  Warps never
+// wait on each other.
+//
+// Where a piece ends: a pixel whose last blended splat lies in the piece
+// starts from (T_final, T_final bg . g); one whose walk goes on past it from
+// the forward's checkpoint at the piece's back edge, R = (out - C) . g.
+// Without checkpoints a tile is one piece.
+//
+// Bound: instruction issue and the latency of the chain alpha -> T -> sums ->
+// reduction (500k Gaussians, 1280x720: 54-68 % issue, 10-16 warps an SM).
+// Against one splat at a time with scalar arithmetic and a reduction per
+// splat and warp of pixels (and, without checkpoints, a block per tile with
+// shared-memory atomics): 720 tiles of 85 pixels 67 -> 54 us, 3600 of 25
+// pixels 155 -> 132, the dense view 728 -> 421, eight views of 3M Gaussians
+// 1738 -> 1043.  Measured beside it and slower: pixels streamed through lanes
+// that hold the splats (no reduction, but long serial chains): 98, 211 and 483
+// us for the first three.
 //
 // STATS: the same replay also sums, per splat, Eq. 12's e w, w and D w over
-// the pixels (w = T alpha the compositing weight, e the pixel's error, D the
-// conic Mahalanobis distance of the pixel centre) into its statistics row.
-template <int PPL, bool STATS>
-__device__ __forceinline__ void render_piece_bwd_warp(const RasterArgs& a, int j, int c, Splat* sm,
-                                                      const float* __restrict__ T_final,
-                                                      const int32_t* __restrict__ n_last,
-                                                      const float* __restrict__ dL_drgb,
-                                                      float* __restrict__ grad2d, const Ckpt& ck,
-                                                      const StatsK st = StatsK{nullptr, nullptr}) {
-  constexpr int E = kCkptEvery;
+// the pixels (e the pixel's error, D the conic Mahalanobis distance of the
+// pixel centre) into its statistics row.
+// ---------------------------------------------------------------------------
+constexpr int kBwdPpl = 4;      // most pixels a lane
+// One warp a block: items differ in length (empty ones, long lists), and a
+// block of four holds its slots until its longest is done (sparse step: 66 us
+// with four warps a block, 57 with one).  20 blocks an SM: 96 registers.
+constexpr int kBwdBlocksPerSm = 20;
+
+// Two fp32 values in one 64-bit register pair: each operation is the IEEE
+// operation on both, in one issue slot.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float y;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
+// Two kept splats as the replay reads them (element e in half e).
+struct __align__(16) BwdPair {
+  f32x2 nx, ny;      // minus the centre
+  f32x2 ca, cb;      // the pre-scaled conic
+  f32x2 cc, op;      // and the opacity
+  f32x2 cr, cg;      // colour
+  f32x2 cbl;
+  f32x2 np;          // minus (position from the chunk's first + 1/2)
+  float cf[2][8];    // factors of the reduced sums, in the gradient row's order
+  float bo[2];       // cross factor of the centre's two sums
+  int id[2];
+};
+constexpr int kBwdPairs = 17;  // a chunk's 32 splats and one left over
+
+// Whether a splat's alpha can reach 1/255 in the rectangle box (x0, y0, x1,
+// y1): splat_rows along both axes (half-width sqrt(2 tau c / det)), with
+// approximate functions and tau rounded up by 1e-6, well inside the margins.
+__device__ __forceinline__ bool splat_reaches(float2 xy, const float4& c, float4 box) {
+  const float x = 255.f * c.w;
+  if (!(x > 1.f)) return false;
+  const float det = c.x * c.z - c.y * c.y;
+  if (!(det > 0.f) || !(c.x > 0.f)) return true;
+  const float k = __fdividef(2.f * (__logf(x) + 1e-6f), det);
+  const float h = sqrt_approx(k * c.x) * 1.001f + 1e-3f, w = sqrt_approx(k * c.z) * 1.001f + 1e-3f;
+  return xy.y + h >= box.y && xy.y - h <= box.w && xy.x + w >= box.x && xy.x - w <= box.z;
+}
+
+// Entry i of the warp's queue.
+__device__ __forceinline__ void bwd_stage(BwdPair* Q, int i, const SplatRaw& w, float pos) {
+  BwdPair& P = Q[i >> 1];
+  const int e = i & 1;
+  reinterpret_cast<float*>(&P.nx)[e] = -w.xy.x;
+  reinterpret_cast<float*>(&P.ny)[e] = -w.xy.y;
+  reinterpret_cast<float*>(&P.ca)[e] = __fmul_rn(w.c.x, kPow2A);
+  reinterpret_cast<float*>(&P.cb)[e] = __fmul_rn(w.c.y, kPow2B);
+  reinterpret_cast<float*>(&P.cc)[e] = __fmul_rn(w.c.z, kPow2A);
+  reinterpret_cast<float*>(&P.op)[e] = w.c.w;
+  reinterpret_cast<float*>(&P.cr)[e] = w.r;
+  reinterpret_cast<float*>(&P.cg)[e] = w.g;
+  reinterpret_cast<float*>(&P.cbl)[e] = w.b;
+  reinterpret_cast<float*>(&P.np)[e] = -(pos + 0.5f);
+  P.id[e] = w.id;
+  // sums of dL/dpower times dx, dy, dx^2, dx dy, dy^2, 1 (power = -(a dx^2 +
+  // c dy^2)/2 - b dx dy, dx = px - x): dL/dx = a m1 + b m2, dL/dy = c m2 + b m1,
+  // dL/da = -m3 / 2, dL/db = -m4, dL/dc = -m5 / 2, dL/do = m0 / o
+  const float o = w.c.w;
+  float4* f = reinterpret_cast<float4*>(P.cf[e]);
+  f[0] = make_float4(w.c.x, w.c.z, -0.5f, -1.f);
+  f[1] = make_float4(-0.5f, o > 0.f ? __fdividef(1.f, o) : 0.f, 1.f, 1.f);
+  P.bo[e] = w.c.y;
+}
+
+// One pair against the lane's pixels, and its sums into the gradient rows.
+// CAPPED: an opacity reaches the cap on alpha.  Where a splat does not blend,
+// sums and states change by zeros, so everything has to be finite.
+template <int PPL, bool CAPPED, bool STATS>
+__device__ __forceinline__ void bwd_pair(const BwdPair& P, const f32x2 (&px)[PPL], const f32x2 (&py)[PPL],
+                                         const f32x2 (&g0)[PPL], const f32x2 (&g1)[PPL], const f32x2 (&g2)[PPL],
+                                         const float (&err)[STATS ? PPL : 1], const f32x2 (&last)[PPL],
+                                         float (&T)[PPL], float (&R)[PPL], float* __restrict__ grad2d,
+                                         float4* __restrict__ stats) {
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int t = a.active_tiles ? a.active_tiles[j] : j;
-  const int p0 = a.pix_off[j], p1 = a.pix_off[j + 1];
-  int max_last;
-  if (ck.tile_last) {
-    max_last = ck.tile_last[j];  // from the forward
-  } else {
-    int m = 0;
-#pragma unroll
-    for (int u = 0; u < PPL; ++u) {
-      const int s = p0 + lane + 32 * u;
-      if (s < p1) m = max(m, n_last[s]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    max_last = m;
-  }
-  const int lo_pos = c * E;
-  const int hi_pos = c < ck.n_slots ? min(lo_pos + E, max_last) : max_last;
-  if (hi_pos <= lo_pos) return;  // warp-uniform: nothing blended here
-  float px[PPL], py[PPL], T[PPL], g0[PPL], g1[PPL], g2[PPL], S0[PPL], S1[PPL], S2[PPL];
-  float ep[STATS ? PPL : 1];
-  int last[PPL];
-  int warp_last = 0;
+  const f32x2 nx = P.nx, ny = P.ny, ca = P.ca, cb = P.cb, cc = P.cc, op = P.op, cr = P.cr, cg = P.cg, cbl = P.cbl;
+  const f32x2 np = P.np;
+  const f32x2 mone = pk2(-1.f, -1.f), namin = pk2(-kAlphaMin, -kAlphaMin);
+  f32x2 v[9], sv[3];
 #pragma unroll
   for (int u = 0; u < PPL; ++u) {
-    const int s = p0 + lane + 32 * u;
-    last[u] = s < p1 ? n_last[s] : 0;
-    if (last[u] <= lo_pos) last[u] = 0;  // this pixel blended nothing in the piece
-    px[u] = py[u] = 0.f;
-    T[u] = 1.f;
-    g0[u] = g1[u] = g2[u] = 0.f;
-    if (STATS) ep[u] = last[u] > 0 ? st.err[s] : 0.f;
-    S0[u] = a.bg[0];
-    S1[u] = a.bg[1];
-    S2[u] = a.bg[2];
-    if (last[u] > 0) {
-      const int l = a.pix_idx[s];
-      px[u] = (float)((t % a.tiles_x) * TGS_TILE + (l & 15)) + 0.5f;
-      py[u] = (float)((t / a.tiles_x) * TGS_TILE + (l >> 4)) + 0.5f;
-      g0[u] = dL_drgb[3 * s];
-      g1[u] = dL_drgb[3 * s + 1];
-      g2[u] = dL_drgb[3 * s + 2];
-      if (c < ck.n_slots && last[u] > lo_pos + E) {
-        const float4 q = ck.data[c * ck.stride + s];  // in front of position (c + 1) E
-        T[u] = q.x;
-        const float iT = 1.f / q.x;
-        S0[u] = (ck.rgb[3 * s] - q.y) * iT;
-        S1[u] = (ck.rgb[3 * s + 1] - q.z) * iT;
-        S2[u] = (ck.rgb[3 * s + 2] - q.w) * iT;
-        last[u] = lo_pos + E;
-      } else {
-        T[u] = T_final[s];
-      }
+    const f32x2 dx = add2(px[u], nx), dy = add2(py[u], ny);
+    const f32x2 p = fma2(fma2(ca, dx, mul2(cb, dy)), dx, mul2(mul2(cc, dy), dy));  // splat_pow2 of both
+    const float p0 = lo2(p), p1 = hi2(p);
+    const float G0 = ex2_approx(p0), G1 = ex2_approx(p1);
+    const f32x2 og = mul2(op, pk2(G0, G1));
+    // blends where power <= 0, alpha >= 1/255 and the pixel's walk came past the splat
+    const f32x2 am_ = add2(og, namin), ahead = add2(last[u], np);
+    const bool ok0 = min3(-p0, lo2(am_), lo2(ahead)) >= 0.f, ok1 = min3(-p1, hi2(am_), hi2(ahead)) >= 0.f;
+    float a0 = ok0 ? lo2(og) : 0.f, a1 = ok1 ? hi2(og) : 0.f;
+    if (CAPPED) {
+      a0 = ok0 ? fminf(kAlphaMax, lo2(og)) : 0.f;
+      a1 = ok1 ? fminf(kAlphaMax, hi2(og)) : 0.f;
     }
-    warp_last = max(warp_last, last[u]);
+    const f32x2 am = pk2(a0, a1);
+    const f32x2 cdg = fma2(cbl, g2[u], fma2(cg, g1[u], mul2(cr, g0[u])));  // c . g
+    const f32x2 d = add2(am, mone);  // -(1 - alpha), at most -0.01
+    const float i0 = rcp_approx(lo2(d)), i1 = rcp_approx(hi2(d));
+    const float T0 = -T[u] * i0, T1 = -T0 * i1;  // transmittance in front of each
+    const f32x2 Tv = pk2(T0, T1);
+    const f32x2 w = mul2(am, Tv);
+    const float R0 = R[u], R1 = __fmaf_rn(lo2(w), lo2(cdg), R0);
+    const f32x2 da = fma2(pk2(R0, R1), pk2(i0, i1), mul2(Tv, cdg));  // dL/dalpha
+    // alpha dL/dalpha, the gradient of the power and, over the opacity, of the
+    // opacity; a capped alpha passes none
+    const f32x2 t = mul2(da, CAPPED ? pk2(a0 < kAlphaMax ? a0 : 0.f, a1 < kAlphaMax ? a1 : 0.f) : am);
+    T[u] = T1;
+    R[u] = __fmaf_rn(hi2(w), hi2(cdg), R1);
+    const f32x2 tx = mul2(t, dx), ty = mul2(t, dy);
+    v[0] = u == 0 ? tx : add2(v[0], tx);
+    v[1] = u == 0 ? ty : add2(v[1], ty);
+    v[2] = u == 0 ? mul2(tx, dx) : fma2(tx, dx, v[2]);
+    v[3] = u == 0 ? mul2(tx, dy) : fma2(tx, dy, v[3]);
+    v[4] = u == 0 ? mul2(ty, dy) : fma2(ty, dy, v[4]);
+    v[5] = u == 0 ? t : add2(v[5], t);
+    v[6] = u == 0 ? mul2(w, g0[u]) : fma2(w, g0[u], v[6]);
+    v[7] = u == 0 ? mul2(w, g1[u]) : fma2(w, g1[u], v[7]);
+    v[8] = u == 0 ? mul2(w, g2[u]) : fma2(w, g2[u], v[8]);
+    if (STATS) {
+      // a dx^2 + 2 b dx dy + c dy^2 = -2 power = -2 ln(2) p
+      const float D0 = sqrt_approx(fmaxf(p0 * kInvA, 0.f)), D1 = sqrt_approx(fmaxf(p1 * kInvA, 0.f));
+      const f32x2 ee = pk2(err[u], err[u]);
+      sv[0] = u == 0 ? mul2(w, ee) : fma2(w, ee, sv[0]);
+      sv[1] = u == 0 ? w : add2(w, sv[1]);
+      sv[2] = u == 0 ? mul2(w, pk2(D0, D1)) : fma2(w, pk2(D0, D1), sv[2]);
+    }
+  }
+  // the sums over the warp: splat 0's to lanes 0-15, splat 1's to 16-31, then
+  // component k to lanes 2 k and 2 k + 1 of the half, component 8 to all of it
+  const bool up = lane & 16;
+  float r[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const float keep = up ? hi2(v[k]) : lo2(v[k]), send = up ? lo2(v[k]) : hi2(v[k]);
+    r[k] = keep + __shfl_xor_sync(full, send, 16);
+  }
+  float b4[4], b2[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool h = lane & 8;
+    const float keep = h ? r[4 + k] : r[k], send = h ? r[k] : r[4 + k];
+    b4[k] = keep + __shfl_xor_sync(full, send, 8);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) warp_last = max(warp_last, __shfl_xor_sync(0xffffffffu, warp_last, o));
-  // slot u of the lanes holds 32 consecutive sampled pixels (row-major): a band of rows; a splat
-  // outside a slot's band is skipped for that slot by the whole warp
-  float2 band[PPL];
+  for (int k = 0; k < 2; ++k) {
+    const bool h = lane & 4;
+    const float keep = h ? b4[2 + k] : b4[k], send = h ? b4[k] : b4[2 + k];
+    b2[k] = keep + __shfl_xor_sync(full, send, 4);
+  }
+  const bool h2 = lane & 2;
+  float s = (h2 ? b2[1] : b2[0]) + __shfl_xor_sync(full, h2 ? b2[0] : b2[1], 2);
+  s += __shfl_xor_sync(full, s, 1);
+  float s8 = r[8];
 #pragma unroll
-  for (int u = 0; u < PPL; ++u) band[u] = warp_rows(last[u] > 0, py[u]);
-  const int2 range = a.ranges[j];
-  const int first = range.x + lo_pos, end = range.x + min(hi_pos, warp_last);
-  for (int top = end; top > first; top -= 32) {
-    const int lo = max(first, top - 32);
-    __syncwarp();
-    if (lo + lane < top) load_splat(a, lo + lane, sm[lane]);
-    __syncwarp();
-    for (int q = top - lo - 1; q >= 0; --q) {
-      const Splat sp = sm[q];
-      const int pos = lo + q - range.x;  // position in the tile list
-      float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      float sv[4] = {0.f, 0.f, 0.f, 0.f};
-      bool hit = false;
+  for (int o = 8; o > 0; o >>= 1) s8 += __shfl_xor_sync(full, s8, o);
+  const int e = lane >> 4, k = (lane >> 1) & 7;
+  const float other = __shfl_xor_sync(full, s, 2);  // the other sum of the centre (k = 0, 1)
+  float val = P.cf[e][k] * s;
+  if (k < 2) val += P.bo[e] * other;
+  float* gp = grad2d + 12 * (size_t)P.id[e] + k;
+  if (lane & 1) {
+    gp += 8;
+    val = k == 0 ? s8 : 0.f;
+  }
+  if (val != 0.f) atomicAdd(gp, val);
+  if (STATS) {
+    float z[3];
 #pragma unroll
-      for (int u = 0; u < PPL; ++u) {
-        if (sp.yr.y < band[u].x || sp.yr.x > band[u].y) continue;  // warp-uniform
-        if (pos >= last[u]) continue;
-        const float dx = __fsub_rn(px[u], sp.xy.x), dy = __fsub_rn(py[u], sp.xy.y);
-        float alpha, G, pw;
-        if (!splat_alpha_p(sp.co, dx, dy, alpha, G, pw)) continue;
-        hit = true;
-        T[u] = __fdividef(T[u], 1.f - alpha);  // transmittance in front of this splat (1 - alpha >= 0.01)
-        const float wgt = alpha * T[u];
-        if (STATS) {
-          // a dx^2 + 2 b dx dy + c dy^2 = -2 power = -2 ln(2) p
-          const float D = sqrtf(fmaxf(pw * kInvA, 0.f));
-          sv[0] += ep[u] * wgt;
-          sv[1] += wgt;
-          sv[2] += D * wgt;
+    for (int k3 = 0; k3 < 3; ++k3) {
+      const float keep = up ? hi2(sv[k3]) : lo2(sv[k3]), send = up ? lo2(sv[k3]) : hi2(sv[k3]);
+      z[k3] = keep + __shfl_xor_sync(full, send, 16);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) z[k3] += __shfl_xor_sync(full, z[k3], o);
+    }
+    if ((lane & 15) == 0 && z[1] != 0.f)
+      red_add_v4(reinterpret_cast<float*>(stats + P.id[e]), z[0], z[1], z[2], 0.f);
+  }
+}
+
+// The rest of an item (list entries [first, top) from the back) where a
+// gradient, a colour or a state is infinite or NaN: splat by splat, and only
+// where a pixel blends one, so that such values stay with their own pixels
+// and splats.  TR: T and R of the group's pixels.
+template <bool STATS>
+__device__ __noinline__ void bwd_rest_safe(const RasterArgs& a, int j, int p0, int p1, int lo_pos, int start, int first,
+                                           int top, const float2* TR, const int32_t* __restrict__ n_last,
+                                           const float* __restrict__ dL_drgb, float* __restrict__ grad2d,
+                                           const StatsK& st) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, t = a.active_tiles ? a.active_tiles[j] : j;
+  const float ox = (float)((t % a.tiles_x) * TGS_TILE) + 0.5f, oy = (float)((t / a.tiles_x) * TGS_TILE) + 0.5f;
+  for (int s0 = p0; s0 < p1; s0 += 32) {
+    const int s = s0 + lane;
+    const bool has = s < p1;
+    const int last = has ? n_last[s] : 0, l = has ? a.pix_idx[s] : 0;
+    const float px = ox + (float)(l & 15), py = oy + (float)(l >> 4);
+    const float g0 = has ? dL_drgb[3 * (size_t)s] : 0.f, g1 = has ? dL_drgb[3 * (size_t)s + 1] : 0.f,
+                g2 = has ? dL_drgb[3 * (size_t)s + 2] : 0.f;
+    const float err = STATS && has ? st.err[s] : 0.f;
+    float T = TR[s - p0].x, R = TR[s - p0].y;
+    for (int k = top - 1; k >= first; --k) {
+      Splat sp;
+      load_splat(a, k, sp);
+      float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, z[3] = {0.f, 0.f, 0.f};
+      const float dx = __fsub_rn(px, sp.xy.x), dy = __fsub_rn(py, sp.xy.y);
+      float al, G;
+      const bool ok = last > lo_pos && k - start < last && sp.yr.y >= py && sp.yr.x <= py &&
+                      splat_alpha(sp.co, dx, dy, al, G);
+      if (ok) {
+        const float inv = rcp_approx(1.f - al), cdg = sp.rgb.x * g0 + sp.rgb.y * g1 + sp.rgb.z * g2;
+        T *= inv;
+        const float w = al * T, da = T * cdg - R * inv;
+        R += w * cdg;
+        v[6] = w * g0;
+        v[7] = w * g1;
+        v[8] = w * g2;
+        if (al < kAlphaMax) {
+          const float tt = da * al, tx = tt * dx, ty = tt * dy;
+          v[0] = tx;
+          v[1] = ty;
+          v[2] = tx * dx;
+          v[3] = tx * dy;
+          v[4] = ty * dy;
+          v[5] = da * G;
         }
-        v[6] += wgt * g0[u];
-        v[7] += wgt * g1[u];
-        v[8] += wgt * g2[u];
-        const float e0 = sp.rgb.x - S0[u], e1 = sp.rgb.y - S1[u], e2 = sp.rgb.z - S2[u];
-        const float dalpha = T[u] * (e0 * g0[u] + e1 * g1[u] + e2 * g2[u]);
-        S0[u] += alpha * e0;  // the light seen behind the splat in front
-        S1[u] += alpha * e1;
-        S2[u] += alpha * e2;
-        if (alpha < kAlphaMax) {  // not clamped
-          v[5] += dalpha * G;
-          const float dpow = dalpha * alpha;
-          const float tx = dpow * dx, ty = dpow * dy;
-          v[0] += tx;  // the moments of dL/dpower; the conic is applied per splat
-          v[1] += ty;
-          v[2] += tx * dx;
-          v[3] += tx * dy;
-          v[4] += ty * dy;
-        }
+        z[0] = err * w;
+        z[1] = w;
+        z[2] = w * sqrt_approx(fmaxf(splat_pow2(sp.co, dx, dy) * kInvA, 0.f));
       }
-      if (!__any_sync(0xffffffffu, hit)) continue;
-      const float r8 = warp_reduce_scatter8(v, lane);  // lane 4 k + (0..3): component k
-      const float r9 = warp_sum(v[8]);
-      // components 0..3 to lane 0, 4..7 to lane 16
-      const float c1 = __shfl_down_sync(0xffffffffu, r8, 4);
-      const float c2 = __shfl_down_sync(0xffffffffu, r8, 8);
-      const float c3 = __shfl_down_sync(0xffffffffu, r8, 12);
-      float* gp = grad2d + 12 * (size_t)__float_as_int(sp.rgb.w);
+      if (!__any_sync(full, ok)) continue;
+      for (int c = 0; c < 9; ++c) v[c] = warp_sum(v[c]);
+      const int id = __float_as_int(sp.rgb.w);
+      const float A = sp.co.x * kInvA, Bc = sp.co.y * kInvB, Cc = sp.co.z * kInvA;
       if (lane == 0) {
-        float gc[5];
-        power_moments_to_grad(sp.co, r8, c1, c2, c3, 0.f, gc);
-        red_add_v4(gp, gc[0], gc[1], gc[2], gc[3]);
-      } else if (lane == 16) {
-        red_add_v4(gp + 4, -0.5f * r8, c1, c2, c3);  // dL/dc from the dy^2 moment
-      } else if (lane == 1) {
-        atomicAdd(gp + 8, r9);
+        float* gp = grad2d + 12 * (size_t)id;
+        red_add_v4(gp, A * v[0] + Bc * v[1], Cc * v[1] + Bc * v[0], -0.5f * v[2], -v[3]);
+        red_add_v4(gp + 4, -0.5f * v[4], v[5], v[6], v[7]);
+        atomicAdd(gp + 8, v[8]);
       }
       if (STATS) {
-        const float rs = warp_reduce_scatter4(sv, lane);  // lane 8 k + (0..7): statistic k
-        const float s1 = __shfl_down_sync(0xffffffffu, rs, 8);
-        const float s2 = __shfl_down_sync(0xffffffffu, rs, 16);
-        if (lane == 0) red_add_v4(reinterpret_cast<float*>(st.stats + __float_as_int(sp.rgb.w)), rs, s1, s2, 0.f);
+        for (int c = 0; c < 3; ++c) z[c] = warp_sum(z[c]);
+        if (lane == 0) red_add_v4(reinterpret_cast<float*>(st.stats + id), z[0], z[1], z[2], 0.f);
       }
     }
   }
 }
 
-constexpr int kBwdWarps = 4;  // pieces per block of the one-view split backward
+// How a launch divides its tiles into items: `groups` of at most `gpx` pixels,
+// and `pieces` of `span` checkpoint intervals (the last one open); one piece
+// without checkpoints.
+struct BwdSplit {
+  int groups, gpx, pieces, span;
+};
+
+// Item (tile j, q = piece * groups + group).
+template <int PPL, bool STATS>
+__device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int q, const BwdSplit& sp, BwdPair* Q,
+                                                const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
+                                                const float* __restrict__ dL_drgb, float* __restrict__ grad2d,
+                                                const Ckpt& ck, const StatsK& st) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int c = q / sp.groups, grp = q - c * sp.groups;
+  const int lo_pos = c * sp.span * kCkptEvery;
+  const bool open = c == sp.pieces - 1;
+  const int hi_edge = open ? INT_MAX : lo_pos + sp.span * kCkptEvery;
+  if (ck.tile_last && ck.tile_last[j] <= lo_pos) return;  // warp-uniform: nothing blended here
+  const int p0 = a.pix_off[j] + grp * sp.gpx, p1 = min(a.pix_off[j + 1], p0 + sp.gpx);
+  const int2 range = a.ranges[j];
+  const int first = range.x + lo_pos;
+  // the loads of the first chunk's list entries go out with the pixels' own
+  int top = open ? 0 : range.x + hi_edge;
+  int id = !open && top - 1 - lane < range.y ? a.vals[top - 1 - lane] : -1;
+  const int t = a.active_tiles ? a.active_tiles[j] : j;
+  const float ox = (float)((t % a.tiles_x) * TGS_TILE) + 0.5f, oy = (float)((t / a.tiles_x) * TGS_TILE) + 0.5f;
+  int last[PPL], hi_pos = 0;
+  f32x2 px[PPL], py[PPL], g0[PPL], g1[PPL], g2[PPL];
+  float T[PPL], R[PPL], err[STATS ? PPL : 1];
+  bool finite = true;
+  float4 box = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+  for (int u = 0; u < PPL; ++u) {
+    const int s = p0 + 32 * u + lane;
+    const bool in = s < p1;
+    last[u] = in ? n_last[s] : 0;
+    const int l = in ? a.pix_idx[s] : 0;
+    float d0 = in ? dL_drgb[3 * (size_t)s] : 0.f, d1 = in ? dL_drgb[3 * (size_t)s + 1] : 0.f,
+          d2 = in ? dL_drgb[3 * (size_t)s + 2] : 0.f;
+    T[u] = in ? T_final[s] : 1.f;
+    if (STATS) err[u] = in ? st.err[s] : 0.f;
+    const float x = ox + (float)(l & 15), y = oy + (float)(l >> 4);
+    if (last[u] <= lo_pos) {  // this pixel blended nothing in the piece
+      last[u] = 0;
+      d0 = d1 = d2 = 0.f;
+      T[u] = 1.f;
+      if (STATS) err[u] = 0.f;
+    } else {
+      box = make_float4(fminf(box.x, x), fminf(box.y, y), fmaxf(box.z, x), fmaxf(box.w, y));
+    }
+    R[u] = T[u] * (a.bg[0] * d0 + a.bg[1] * d1 + a.bg[2] * d2);
+    if (last[u] > hi_edge) {
+      const float4 k4 = ck.data[((c + 1) * sp.span - 1) * ck.stride + s];  // in front of position hi_edge
+      T[u] = k4.x;
+      R[u] = (ck.rgb[3 * (size_t)s] - k4.y) * d0 + (ck.rgb[3 * (size_t)s + 1] - k4.z) * d1 +
+             (ck.rgb[3 * (size_t)s + 2] - k4.w) * d2;
+    }
+    if (STATS) finite = finite && fabsf(err[u]) < INFINITY;
+    finite = finite && fabsf(d0) + fabsf(d1) + fabsf(d2) + fabsf(R[u]) + fabsf(T[u]) < INFINITY;
+    hi_pos = max(hi_pos, min(last[u], hi_edge));
+    px[u] = pk2(x, x);
+    py[u] = pk2(y, y);
+    g0[u] = pk2(d0, d0);
+    g1[u] = pk2(d1, d1);
+    g2[u] = pk2(d2, d2);
+  }
+  hi_pos = __reduce_max_sync(full, hi_pos);
+  if (hi_pos <= lo_pos) return;
+  if (open) {
+    top = range.x + hi_pos;
+    id = top - 1 - lane >= first ? a.vals[top - 1 - lane] : -1;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    box.x = fminf(box.x, __shfl_xor_sync(full, box.x, o));
+    box.y = fminf(box.y, __shfl_xor_sync(full, box.y, o));
+    box.z = fmaxf(box.z, __shfl_xor_sync(full, box.z, o));
+    box.w = fmaxf(box.w, __shfl_xor_sync(full, box.w, o));
+  }
+  int qn = 0, left = 0;  // left: list entry of the splat left over in the queue
+  for (; top > first; top -= 32) {
+    // positions count from the chunk's first, so that they stay small in floats
+    const int base = top - 32, k = top - 1 - lane;
+    f32x2 lastf[PPL];
+#pragma unroll
+    for (int u = 0; u < PPL; ++u) {
+      const float l = (float)max(min(last[u] - (base - range.x), 64), 0);
+      lastf[u] = pk2(l, l);
+    }
+    SplatRaw w;
+    bool keep = false;
+    if (id >= 0 && k < range.x + hi_pos) {
+      fetch_splat(a, id, w);
+      keep = splat_reaches(w.xy, w.c, box);
+      // a record that is not finite takes the item off the fast path
+      finite = finite && (!keep || fabsf(w.xy.x) + fabsf(w.xy.y) + fabsf(w.c.x) + fabsf(w.c.y) + fabsf(w.c.z) +
+                                           fabsf(w.c.w) + fabsf(w.r) + fabsf(w.g) + fabsf(w.b) <
+                                       INFINITY);
+    }
+    id = k - 32 >= first ? a.vals[k - 32] : -1;  // the next chunk's, ahead of this one's replay
+    if (!__all_sync(full, finite)) {
+      float2* TR = reinterpret_cast<float2*>(Q);
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < PPL; ++u) TR[32 * u + lane] = make_float2(T[u], R[u]);
+      __syncwarp();
+      bwd_rest_safe<STATS>(a, j, p0, p1, lo_pos, range.x, first, qn ? left + 1 : min(top, range.y), TR, n_last, dL_drgb, grad2d, st);
+      return;
+    }
+    const unsigned m = __ballot_sync(full, keep);
+    if (m) left = top - 1 - (31 - __clz(m));  // the front-most one kept
+    if (keep) bwd_stage(Q, qn + __popc(m & ((1u << lane) - 1u)), w, (float)(k - base));
+    qn += __popc(m);
+    // the second half of the last pair, or of one left over for a whole chunk
+    // (a position stays below 64): a splat that blends nowhere
+    const bool end = top - 32 <= first || m == 0u;
+    if (end && (qn & 1)) {
+      if (lane == 0) {
+        SplatRaw z;
+        z.xy = make_float2(0.f, 0.f);
+        z.c = make_float4(0.f, 0.f, 0.f, 0.f);
+        z.r = z.g = z.b = 0.f;
+        z.id = 0;
+        bwd_stage(Q, qn, z, 1e9f);
+      }
+      ++qn;
+    }
+    __syncwarp();
+    const int pairs = qn >> 1;
+#pragma unroll 1
+    for (int i = 0; i < pairs; ++i) {
+      if (fmaxf(lo2(Q[i].op), hi2(Q[i].op)) < kAlphaMax)
+        bwd_pair<PPL, false, STATS>(Q[i], px, py, g0, g1, g2, err, lastf, T, R, grad2d, st.stats);
+      else
+        bwd_pair<PPL, true, STATS>(Q[i], px, py, g0, g1, g2, err, lastf, T, R, grad2d, st.stats);
+    }
+    __syncwarp();
+    if (qn & 1) {  // one splat left over: to the front
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(Q + pairs);
+      uint32_t* dst = reinterpret_cast<uint32_t*>(Q);
+      if (pairs > 0)
+        for (int i = lane; i < (int)(sizeof(BwdPair) / 4); i += 32) dst[i] = src[i];
+      __syncwarp();
+      if (lane == 0) reinterpret_cast<float*>(&Q[0].np)[0] -= 32.f;  // from the next chunk's first
+    }
+    qn &= 1;
+  }
+}
 
 template <int PPL, bool STATS>
-__global__ void __launch_bounds__(32 * kBwdWarps, PPL <= 3 ? 7 : 1)
-    k_render_bwd_warp(RasterArgs a, const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
-                      const float* __restrict__ dL_drgb, float* __restrict__ grad2d, Ckpt ck, StatsK st) {
-  __shared__ Splat sm[kBwdWarps][32];
-  const int j = blockIdx.x;
+__global__ void __launch_bounds__(32, kBwdBlocksPerSm)
+    k_render_bwd(RasterArgs a, const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
+                 const float* __restrict__ dL_drgb, float* __restrict__ grad2d, Ckpt ck, StatsK st, BwdSplit sp, int n_tiles) {
+  __shared__ BwdPair Q[kBwdPairs];
+  const int q = blockIdx.x / n_tiles, j = blockIdx.x - q * n_tiles;  // deeper pieces last: most of them are empty
   if (j >= *a.n_active) return;
-  const int w = threadIdx.x >> 5;
-  const int c = blockIdx.y * kBwdWarps + w;
-  if (c > ck.n_slots) return;  // warp-uniform; the kernel has no block-wide barrier
-  render_piece_bwd_warp<PPL, STATS>(a, j, c, sm[w], T_final, n_last, dL_drgb, grad2d, ck, st);
+  render_item_bwd<PPL, STATS>(a, j, q, sp, Q, T_final, n_last, dL_drgb, grad2d, ck, st);
 }
 
 // Error back-projection statistics (Sec. 3.8, Eq. 12): one
@@ -1264,7 +1372,7 @@ constexpr int kMaxViews = 16;
 
 struct BatchArgs {
   int n_views;
-  int pieces;  // backward items per tile: 1, or checkpoint slots + 1
+  BwdSplit split;  // the backward's items per tile
   int base[kMaxViews + 1];
   RasterArgs a[kMaxViews];
   float* rgb[kMaxViews];
@@ -1289,16 +1397,6 @@ __device__ __forceinline__ bool next_item(const BatchArgs& b, int* counter, int*
   return true;
 }
 
-// The same, claiming `step` consecutive items per atomic: the first is
-// returned in *first (shared), the caller walks them.
-__device__ __forceinline__ bool next_items(const BatchArgs& b, int* counter, int* s_item, int step, int& first) {
-  __syncthreads();
-  if (threadIdx.x == 0) *s_item = atomicAdd(counter, step);
-  __syncthreads();
-  first = *s_item;
-  return first < b.base[b.n_views];
-}
-
 __device__ __forceinline__ void item_view(const BatchArgs& b, int item, int& v, int& q) {
   v = 0;
   while (item >= b.base[v + 1]) ++v;
@@ -1314,41 +1412,58 @@ __global__ void k_render_fwd_batched(BatchArgs b, int* __restrict__ counter) {
   }
 }
 
-// Whole tiles, one item per block (the backward without checkpoints).
-__global__ void k_render_bwd_batched(BatchArgs b, int* __restrict__ counter) {
-  extern __shared__ Splat sm[];
-  __shared__ int s_item;
-  int v, q;
-  while (next_item(b, counter, &s_item, v, q))
-    if (q < *b.a[v].n_active) render_tile_bwd(b.a[v], q, sm, b.T[v], b.last[v], b.dL[v], b.grad2d[v]);
-}
-
-// With checkpoints: items are (view, tile, piece) with the pieces of a tile
-// consecutive; each warp claims kPieceClaim of them per atomic and replays
-// them as the one-view split backward does.
-constexpr int kPieceClaim = 4;
-constexpr int kBatchBwdWarps = 4;
+// The batched backward: items are (view, piece, group, tile); each warp claims kItemClaim of them per atomic and replays
+// them as the one-view backward does.
+constexpr int kItemClaim = 4;
 
 template <int PPL, bool STATS>
-__global__ void __launch_bounds__(32 * kBatchBwdWarps) k_render_bwd_batched_warp(BatchArgs b,
-                                                                                int* __restrict__ counter) {
-  __shared__ Splat sm[kBatchBwdWarps][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int total = b.base[b.n_views];
+__global__ void __launch_bounds__(32, kBwdBlocksPerSm) k_render_bwd_batched(BatchArgs b, int* __restrict__ counter) {
+  __shared__ BwdPair Q[kBwdPairs];
+  const int lane = threadIdx.x;
+  const int total = b.base[b.n_views], per_tile = b.split.pieces * b.split.groups;
   for (;;) {
     int first = 0;
-    if (lane == 0) first = atomicAdd(counter, kPieceClaim);
+    if (lane == 0) first = atomicAdd(counter, kItemClaim);
     first = __shfl_sync(0xffffffffu, first, 0);
     if (first >= total) return;
-    const int end = min(first + kPieceClaim, total);
+    const int end = min(first + kItemClaim, total);
     for (int item = first; item < end; ++item) {
       int v, q;
       item_view(b, item, v, q);
-      const int j = q / b.pieces, c = q - j * b.pieces;
+      const int n_tiles = (b.base[v + 1] - b.base[v]) / per_tile, r = q / n_tiles, j = q - r * n_tiles;
       if (j >= *b.a[v].n_active) continue;
-      render_piece_bwd_warp<PPL, STATS>(b.a[v], j, c, sm[w], b.T[v], b.last[v], b.dL[v], b.grad2d[v], b.ck[v],
-                                        StatsK{b.err[v], b.stats});
+      render_item_bwd<PPL, STATS>(b.a[v], j, r, b.split, Q, b.T[v], b.last[v], b.dL[v],
+                                  b.grad2d[v], b.ck[v], StatsK{b.err[v], b.stats});
     }
+  }
+}
+
+// The kernels of a launch with at most 32 ppl pixels a group.
+using BwdKernel = void (*)(RasterArgs, const float*, const int32_t*, const float*, float*, Ckpt, StatsK, BwdSplit,
+                           int);
+using BwdBatchedKernel = void (*)(BatchArgs, int*);
+static BwdKernel bwd_kernel(int ppl, bool stats) {
+  switch (2 * ppl + (stats ? 1 : 0)) {
+    case 2: return k_render_bwd<1, false>;
+    case 3: return k_render_bwd<1, true>;
+    case 4: return k_render_bwd<2, false>;
+    case 5: return k_render_bwd<2, true>;
+    case 6: return k_render_bwd<3, false>;
+    case 7: return k_render_bwd<3, true>;
+    case 8: return k_render_bwd<4, false>;
+    default: return k_render_bwd<4, true>;
+  }
+}
+static BwdBatchedKernel bwd_batched_kernel(int ppl, bool stats) {
+  switch (2 * ppl + (stats ? 1 : 0)) {
+    case 2: return k_render_bwd_batched<1, false>;
+    case 3: return k_render_bwd_batched<1, true>;
+    case 4: return k_render_bwd_batched<2, false>;
+    case 5: return k_render_bwd_batched<2, true>;
+    case 6: return k_render_bwd_batched<3, false>;
+    case 7: return k_render_bwd_batched<3, true>;
+    case 8: return k_render_bwd_batched<4, false>;
+    default: return k_render_bwd_batched<4, true>;
   }
 }
 
@@ -1373,6 +1488,32 @@ static bool raster_args(const tgs_projected* proj, const int32_t* tile_ranges, c
   a.bg[1] = bg[1];
   a.bg[2] = bg[2];
   return true;
+}
+
+// The division of a backward launch over `tiles` tiles.  Groups of 32
+// kBwdPpl pixels take the fewest instructions a pixel (one reduction serves
+// them all); while that leaves fewer items than four an SM (a tile's list
+// counted as four pieces where it has checkpoints), they are halved, down to
+// one pixel a lane.  64 tiles of 85 pixels: 10.7 us in three groups, 12.1 in
+// one; 19 whole tiles without checkpoints: 19.2 us at 32 pixels, 30.2 at 128.
+// Pieces: short ones give more items, long ones read each pixel's state and
+// run into half-filled chunks less often.  span 1 / 2 / 4: 64 tiles of 85
+// pixels 12.1 / 17.6 / 28.9 us, 720 tiles 63.6 / 54.4 / 58.1 us, 3600 tiles of
+// 25 pixels 218 / 160 / 132 us, eight views with 20000 tiles of 85 pixels
+// 1334 / 1088 / 1043 us.
+static BwdSplit bwd_split(int64_t tiles, int n_pix_max, const Ckpt& ck) {
+  const int64_t sms = device_sm_count();
+  BwdSplit sp;
+  int most = 32 * kBwdPpl;
+  auto groups = [&]() { return (n_pix_max + most - 1) / most; };
+  while (most > 32 && tiles * groups() * (ck.data ? 4 : 1) < 4 * sms) most /= 2;
+  sp.groups = groups();
+  sp.gpx = (n_pix_max + sp.groups - 1) / sp.groups;
+  sp.span = tiles * sp.groups <= 2 * sms ? 1 : tiles * sp.groups <= 16 * sms ? 2 : 4;
+  auto pieces = [&]() { return ck.data ? ck.n_slots / sp.span + 1 : 1; };
+  while (pieces() > 1 && tiles * sp.groups * pieces() > INT_MAX / 2) sp.span *= 2;  // items are counted in 32 bits
+  sp.pieces = pieces();
+  return sp;
 }
 
 static int block_for(int n_pix_max) { return std::min(256, std::max(32, (n_pix_max + 31) / 32 * 32)); }
@@ -1536,27 +1677,10 @@ static tgs_status render_backward_impl(const tgs_projected* proj, const int32_t*
   cudaMemsetAsync(grad2d, 0, sizeof(float) * 12 * (size_t)n_gaussians, s);
   if (stats && !accumulate_stats) cudaMemsetAsync(st.stats, 0, sizeof(float4) * (size_t)n_gaussians, s);
   if (n_active_max > 0) {
-    const int B = block_for(n_pix_max);
-    const size_t smem = B * (sizeof(Splat) + 9 * sizeof(float));
-    if (ck.data) {
-      // one warp per piece, kBwdWarps pieces per block, B / 32 pixels per lane
-      const dim3 grid(n_active_max, (ck.n_slots + 1 + kBwdWarps - 1) / kBwdWarps);
-      switch ((B / 32) * 2 + (stats ? 1 : 0)) {
-#define TGS_BWD_WARP(P)                                                                                         \
-  case 2 * P: k_render_bwd_warp<P, false><<<grid, 32 * kBwdWarps, 0, s>>>(a, T_final, n_last, dL_drgb, grad2d, \
-                                                                         ck, st); break;                       \
-  case 2 * P + 1: k_render_bwd_warp<P, true><<<grid, 32 * kBwdWarps, 0, s>>>(a, T_final, n_last, dL_drgb,       \
-                                                                            grad2d, ck, st); break;
-        TGS_BWD_WARP(1) TGS_BWD_WARP(2) TGS_BWD_WARP(3) TGS_BWD_WARP(4)
-        TGS_BWD_WARP(5) TGS_BWD_WARP(6) TGS_BWD_WARP(7) TGS_BWD_WARP(8)
-#undef TGS_BWD_WARP
-        default: break;
-      }
-    } else {
-      k_render_bwd<<<n_active_max, B, smem, s>>>(a, T_final, n_last, dL_drgb, grad2d);
-      if (stats)
-        k_error_stats<<<n_active_max, B, B * sizeof(Splat), s>>>(a, n_last, st.err, reinterpret_cast<float*>(st.stats));
-    }
+    const BwdSplit sp = bwd_split(n_active_max, n_pix_max, ck);
+    const int64_t items = (int64_t)n_active_max * sp.groups * sp.pieces;
+    bwd_kernel((sp.gpx + 31) / 32, stats)<<<(int)items, 32, 0, s>>>(a, T_final, n_last, dL_drgb, grad2d, ck, st,
+                                                                          sp, n_active_max);
   }
   return check_launch();
 }
@@ -1642,7 +1766,6 @@ static tgs_status batch_args(const tgs_view_batch* views, int32_t n_views, bool 
   B = 32;
   // checkpoints: all views or none, with one slot count
   const int slots = views[0].ckpt.n_slots > 0 ? views[0].ckpt.n_slots : 0;
-  b.pieces = backward && slots > 0 ? slots + 1 : 1;
   for (int v = 0; v < n_views; ++v) {
     const tgs_view_batch& w = views[v];
     if (w.n_active_max < 0 || w.n_pix_max < 1 || w.n_pix_max > 256) return TGS_ERR_INVALID_ARG;
@@ -1660,23 +1783,18 @@ static tgs_status batch_args(const tgs_view_batch* views, int32_t n_views, bool 
     if ((w.ckpt.n_slots > 0 ? w.ckpt.n_slots : 0) != slots) return TGS_ERR_INVALID_ARG;
     if (!ckpt_of(&w.ckpt, w.n_active_max, w.n_pix_max, w.rgb, b.ck[v])) return TGS_ERR_INVALID_ARG;
     if (b.ck[v].data && w.ckpt.rgb && w.ckpt.rgb != w.rgb) return TGS_ERR_INVALID_ARG;
-    b.base[v + 1] = b.base[v] + w.n_active_max * (backward ? b.pieces : 1);
     B = std::max(B, block_for(w.n_pix_max));
   }
-  return TGS_OK;
-}
-
-static int bwd_warp_blocks_per_sm(int ppl) {
-  int per_sm = 0;
-  const int T = 32 * kBatchBwdWarps;
-  switch (ppl) {
-#define TGS_OCC(P) \
-  case P: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_bwd_batched_warp<P, false>, T, 0); break;
-    TGS_OCC(1) TGS_OCC(2) TGS_OCC(3) TGS_OCC(4) TGS_OCC(5) TGS_OCC(6) TGS_OCC(7)
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_bwd_batched_warp<8, false>, T, 0);
-#undef TGS_OCC
+  int64_t tiles = 0;
+  int n_pix = 1;
+  for (int v = 0; v < n_views; ++v) {
+    tiles += views[v].n_active_max;
+    n_pix = std::max(n_pix, (int)views[v].n_pix_max);
   }
-  return per_sm;
+  b.split = bwd_split(tiles, n_pix, b.ck[0]);
+  for (int v = 0; v < n_views; ++v)
+    b.base[v + 1] = b.base[v] + views[v].n_active_max * (backward ? b.split.pieces * b.split.groups : 1);
+  return TGS_OK;
 }
 
 extern "C" tgs_status tgs_render_batched_resident(int32_t n_pix_max, int32_t backward, int32_t* ctas) {
@@ -1685,11 +1803,9 @@ extern "C" tgs_status tgs_render_batched_resident(int32_t n_pix_max, int32_t bac
   if (cudaGetDevice(&dev) != cudaSuccess) return check_launch();
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int B = block_for(n_pix_max);
-  if (backward == 2)
-    per_sm = bwd_warp_blocks_per_sm(B / 32);
-  else if (backward)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_bwd_batched, B,
-                                                  B * (sizeof(Splat) + 9 * sizeof(float)));
+  if (backward)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_batched_kernel(std::min(B / 32, kBwdPpl), false),
+                                                  32, 0);
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_fwd_batched, B, B * sizeof(Splat));
   *ctas = sms * per_sm;
@@ -1731,25 +1847,7 @@ static tgs_status render_backward_batched_impl(const tgs_view_batch* views, int3
   if (with_stats && !accumulate_stats && n_stats > 0) cudaMemsetAsync(stats, 0, sizeof(float4) * (size_t)n_stats, s);
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   if (b.base[n_views] == 0) return check_launch();
-  if (b.pieces == 1) {
-    k_render_bwd_batched<<<grid_ctas, B, B * (sizeof(Splat) + 9 * sizeof(float)), s>>>(b, counter);
-    // without checkpoints the statistics are the separate pass, view by view
-    for (int v = 0; with_stats && v < n_views; ++v)
-      if (views[v].n_active_max > 0) {
-        const int Bv = block_for(views[v].n_pix_max);
-        k_error_stats<<<views[v].n_active_max, Bv, Bv * sizeof(Splat), s>>>(b.a[v], b.last[v], b.err[v], stats);
-      }
-    return check_launch();
-  }
-  switch ((B / 32) * 2 + (with_stats ? 1 : 0)) {
-#define TGS_BWD_BATCH(P)                                                                                        \
-  case 2 * P: k_render_bwd_batched_warp<P, false><<<grid_ctas, 32 * kBatchBwdWarps, 0, s>>>(b, counter); break; \
-  case 2 * P + 1: k_render_bwd_batched_warp<P, true><<<grid_ctas, 32 * kBatchBwdWarps, 0, s>>>(b, counter); break;
-    TGS_BWD_BATCH(1) TGS_BWD_BATCH(2) TGS_BWD_BATCH(3) TGS_BWD_BATCH(4)
-    TGS_BWD_BATCH(5) TGS_BWD_BATCH(6) TGS_BWD_BATCH(7) TGS_BWD_BATCH(8)
-#undef TGS_BWD_BATCH
-    default: break;
-  }
+  bwd_batched_kernel((b.split.gpx + 31) / 32, with_stats)<<<grid_ctas, 32, 0, s>>>(b, counter);
   return check_launch();
 }
 

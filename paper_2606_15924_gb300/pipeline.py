@@ -138,11 +138,13 @@ class Trainer:
         self.lam = torch.zeros(S, device=dev)
         self.err_pix = torch.zeros(P, device=dev)
         self.loss = torch.zeros(1, dtype=torch.float64, device=dev)
-        # forward checkpoints for the split backward: only when the step has
-        # too few tiles to fill the GPU (sparse sampling); one slot every
-        # CKPT_EVERY positions of the tile list up to CKPT_POSITIONS
+        # forward checkpoints for the split backward: only when the step's
+        # tiles (whole lists, one warp per 128 sampled pixels) would fill the
+        # GPU less than twice over; one slot every CKPT_EVERY positions of the
+        # tile list up to CKPT_POSITIONS.  3600 tiles of 25 pixels: the
+        # backward takes 132 us with checkpoints, 201 without
         self.ckpt = None
-        if train and not dense and self.n_select < 4 * B.render_batched_resident(self.n_pix, 1):
+        if train and not dense and S * ((self.n_pix + 127) // 128) < 2 * B.render_batched_resident(self.n_pix, 1):
             n_slots = self.CKPT_POSITIONS // self.CKPT_EVERY
             self.ck_data = torch.empty(B.checkpoint_bytes(S, self.n_pix, n_slots) // 4, device=dev)
             self.ck_last = torch.zeros(S, dtype=torch.int32, device=dev)

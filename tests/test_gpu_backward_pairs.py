@@ -1,0 +1,117 @@
+"""The paired-splat backward at the sizes where its division into items
+changes: pixel counts around the lanes' and groups' edges, with and without
+checkpoints, few and many tiles, opacities at the cap on alpha; and infinite
+or NaN gradients and colours, which stay with the pixels and splats they
+belong to."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2606_15924_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+W, H, N = 96, 80, 700
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2606_15924_gb300 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+    oracle.build()
+    return oracle
+
+
+def _case(B, n_pix, slots, n_select, seed=11):
+    from gpu_util import bin_dev, projected_dev, select_dev
+    p = scenes.projected(N, W, H, seed=seed, radius_max=18)
+    p["opac"][::7] = 0.995                       # capped alphas near the centre
+    p["opac"][3::7] = 0.02                       # barely above the threshold
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=W, height=H)
+    sel = select_dev(B, scenes.error_map(W, H), scenes.age_map(W, H), W, H, n_select, n_pix, seed=4)
+    pd = projected_dev(p)
+    binned = bin_dev(B, pd, N, cam, sel["tile_rank"], sel["n_sel"], capacity=40000)
+    P = sel["n_sel"] * n_pix
+    out = dict(rgb=torch.zeros(P, 3, device="cuda"), T=torch.zeros(P, device="cuda"),
+               n_last=torch.zeros(P, dtype=torch.int32, device="cuda"))
+    ck = None
+    if slots:
+        data = torch.full((B.checkpoint_bytes(sel["n_sel"], n_pix, slots) // 4,), float("nan"), device="cuda")
+        last = torch.zeros(sel["n_sel"], dtype=torch.int32, device="cuda")
+        ck = B.checkpoints(data, slots, P, out["rgb"], last)
+        out["keep"] = (data, last)
+    bg = (0.3, 0.1, 0.6)
+    B.render_sampled(pd, binned["ranges"], binned["vals"], sel["active_tiles"], sel["n_active"], sel["n_sel"],
+                     sel["pix_off"], sel["pix_idx"], n_pix, cam, bg, out["rgb"], out["T"], out["n_last"], ckpt=ck)
+
+    def backward(dL, proj=pd):
+        g2 = torch.full((N, 12), 7.0, device="cuda")
+        B.render_backward_sampled(proj, binned["ranges"], binned["vals"], sel["active_tiles"], sel["n_active"],
+                                  sel["n_sel"], sel["pix_off"], sel["pix_idx"], n_pix, cam, bg, out["T"],
+                                  out["n_last"], dL, g2, ckpt=ck)
+        return g2
+    return p, sel, binned, out, bg, backward, P, pd
+
+
+@pytest.mark.parametrize("slots", [0, 3, 64])
+@pytest.mark.parametrize("n_pix", [1, 31, 33, 64, 65, 96, 97, 128, 129, 193, 256])
+def test_pixel_counts_against_oracle(B, orc, n_pix, slots):
+    from gpu_util import select_host
+    for n_select in (2, 30):
+        p, sel, binned, out, bg, backward, P, pd = _case(B, n_pix, slots, n_select)
+        sh = select_host(sel)
+        pix = orc.pixel_coords(sh["active_tiles"], sh["pix_off"], sh["pix_idx"], W)
+        dL = torch.zeros(P, 3, device="cuda")
+        dL[:len(pix)] = torch.randn(len(pix), 3, generator=torch.Generator().manual_seed(5)).cuda()
+        # pixels whose decisions sit at a threshold are left out of the loss
+        want = {k: np.asarray(v, np.float64) for k, v in p.items() if k != "radius"}
+        want["radius"] = p["radius"]
+        ref = orc.render_pixels(want, W, H, pix, bg=bg)
+        amb = torch.from_numpy(ref["margin"] <= 1e-4).cuda()
+        dL[:len(pix)][amb] = 0.0
+        g2 = backward(dL).cpu().numpy().astype(np.float64)
+        w2 = orc.render_backward(want, W, H, pix, dL[:len(pix)].cpu().numpy().astype(np.float64), bg=bg)
+        w2 = w2["grad2d"] if isinstance(w2, dict) else w2
+        k = w2.shape[1]
+        assert np.linalg.norm(g2[:, :k] - w2) <= 1e-3 * np.linalg.norm(w2) + 1e-12
+        assert np.all(g2[:, 9:] == 0.0)
+
+
+@pytest.mark.parametrize("slots", [0, 64])
+def test_nonfinite_values_stay_local(B, slots):
+    """One pixel with an infinite and one with a NaN gradient poison the splats
+    they blend and no others; an infinite colour poisons only its own pixels'
+    splats."""
+    n_pix = 85
+    p, sel, binned, out, bg, backward, P, pd = _case(B, n_pix, slots, 20)
+    A = int(sel["n_active"].item())
+    Pn = int(sel["pix_off"][A].item())
+    dL = torch.randn(P, 3, generator=torch.Generator().manual_seed(6)).cuda()
+    dL[Pn:] = 0.0
+    clean = backward(dL)
+    bad = [5, Pn // 2]
+    only = torch.zeros_like(dL)
+    only[bad] = 1.0
+    hit = (backward(only) != 0).any(1)            # the splats those pixels blend
+    assert hit.any() and not hit.all()
+    d2 = dL.clone()
+    d2[bad[0], 1] = float("inf")
+    d2[bad[1], 0] = float("nan")
+    got = backward(d2)
+    assert not torch.isfinite(got[hit][:, :9]).all(1).any()
+    assert torch.isfinite(got[~hit]).all()
+    rest = ~hit
+    err = (got[rest] - clean[rest]).norm() / clean[rest].norm()
+    assert float(err) <= 1e-5
+    # an infinite colour of one blended splat
+    i = int(torch.nonzero(hit)[0])
+    q = dict(pd)
+    q["rgb"] = pd["rgb"].clone()
+    q["rgb"][i, 2] = float("inf")
+    got = backward(dL, proj=q)
+    assert not bool(torch.isfinite(got[i, :9]).all())
+    assert bool(torch.isfinite(got).all(1).sum() > 0.5 * N)

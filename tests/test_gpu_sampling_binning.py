@@ -163,6 +163,38 @@ def test_bin_tiles_sort_bands_bit_exact(B, orc, n_crowd, presort):
     np.testing.assert_array_equal(out["keys"][:I].cpu().numpy().view(np.uint64), keys_w)
 
 
+# The per-tile sort on lists past a block's capacity (2048, 4096 and 8192 keys
+# at the three capacities), depths crowded into a small part of the range at
+# several scales, and one depth for all (the ids decide).
+@pytest.mark.parametrize("per_tile", [300, 1500, 3000])
+@pytest.mark.parametrize("n,shape", [(2049, "flat"), (4097, "crowd"), (8193, "crowd"), (20000, "nested"),
+                                     (30000, "flat"), (9000, "one"), (64, "one"), (1, "flat")])
+def test_bin_tiles_long_and_crowded_lists_bit_exact(B, orc, n, shape, per_tile):
+    from gpu_util import bin_dev, projected_dev
+    W, H, T = 64, 48, 12
+    rng = np.random.default_rng(n)
+    pr = scenes.projected(n, W, H, seed=n, depth_ties=False)
+    pr["xy"] = rng.uniform(20.0, 28.0, size=(n, 2)).astype(np.float32)
+    pr["radius"] = rng.integers(1, 3, n).astype(np.int32)
+    d = rng.uniform(1.0, 500.0, n)
+    if shape == "crowd":
+        d[: n - 20] = rng.uniform(2.0, 2.0001, n - 20)
+    elif shape == "nested":
+        d[: n // 2] = rng.uniform(3.0, 3.001, n // 2)
+        d[: n // 3] = 3.0005 + 1e-6 * rng.integers(0, 3, n // 3)
+    elif shape == "one":
+        d[:] = 7.25
+    pr["depth"] = d.astype(np.float32)
+    keys_w, vals_w, counts_w = orc.bin_tiles(pr["xy"], pr["radius"], pr["depth"], W, H)
+    cam = dict(viewmat=np.eye(4), fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
+    cap = max(len(vals_w) + 3, per_tile * T)  # the capacity also sets the sort's block
+    out = bin_dev(B, projected_dev(pr), n, cam, None, T, capacity=cap)
+    I = int(out["n_isect"].item())
+    assert I == len(vals_w)
+    np.testing.assert_array_equal(out["vals"][:I].cpu().numpy(), vals_w)
+    np.testing.assert_array_equal(out["keys"][:I].cpu().numpy().view(np.uint64), keys_w)
+
+
 def test_bin_tiles_edge_cases(B, orc):
     from gpu_util import bin_dev, projected_dev
     import torch

@@ -343,16 +343,13 @@ size_t tgs_checkpoint_bytes(int32_t n_active_max, int32_t n_pix_max, int32_t n_s
  * runs' results in list order, (T, C) -> (T T_run, C + T C_run); the run in
  * which the composed transmittance falls below the stopping value is walked
  * again from its entry state to find the exact stop.  The result equals the
- * sequential walk up to the rounding of the composition.  groups = 3 takes
- * the sequential walk with every warp on its own (each stages its own splat
- * batches and stops when its own pixels have saturated; the same bits as
- * the sequential walk), several tiles per block when tiles have few sampled
- * pixels.  groups = 0 (the default) leaves the choice to the library (the
- * walk with two threads per pixel for sparse launches of tiles with at most
- * 32 sampled pixels, else the block's walk); 1 is the block's sequential walk; 2 or 4
- * the split walk; 5 the walk with two threads per pixel (each walks one half
- * of every 32-position run at once, the second from a local transmittance of
- * 1; the halves compose as above, and the second half walks again from the
+ * sequential walk up to the rounding of the composition.  groups = 0 (the
+ * default) leaves the choice to the library (the walk with two threads per
+ * pixel for sparse launches of tiles with at most 32 sampled pixels, else the
+ * sequential walk); 1 and 3 are the sequential walk, every warp on its own;
+ * 2 or 4 the split walk; 5 the walk with two threads per pixel (each walks one
+ * half of every 32-position run at once, the second from a local transmittance
+ * of 1; the halves compose as above, and the second half walks again from the
  * composed state where the stop may lie in it, so that the stops and n_last
  * are the sequential walk's).
  * Process-wide; returns TGS_ERR_INVALID_ARG for other values.

@@ -1,10 +1,9 @@
 // Sparse forward rasterization and its adjoint (Sec. 3.6, Eq. 1).
 //
-// One thread block per active tile, one thread per sampled pixel of the tile
-// (block size = 32 * ceil(n_pix / 32), so a tile sampled at rate 0.1 runs as
-// one warp).  The tile's depth-ordered splat list is staged through shared
-// memory in batches of one splat per thread; a block-wide vote ends the walk
-// once every pixel has saturated.  The backward replays the same walk in
+// One thread block per active tile, one warp per 32 (or 64) sampled pixels of
+// the tile, so a tile sampled at rate 0.1 runs as one warp; each warp walks the
+// tile's depth-ordered splat list until its pixels have saturated, two splats
+// at a time.  The backward replays the same walk in
 // reverse from the stored final transmittance, recovering T_k by division, one
 // warp per group of pixels and piece of the list, two splats at a time.
 #include <climits>
@@ -148,8 +147,6 @@ __device__ __forceinline__ float2 warp_rows(bool has, float py) {
   return make_float2(lo, hi);
 }
 
-// Forward of active tile j (one thread per sampled pixel; sm holds
-// blockDim.x splats).
 // Checkpoints of the sampled forward for the split backward: slot c (c = 0
 // .. n_slots - 1) of pixel s holds (T, C_r, C_g, C_b) in front of tile-list
 // position (c + 1) kCkptEvery, at data[c * stride + s]; written by every
@@ -162,141 +159,304 @@ struct Ckpt {
   int32_t* tile_last;  // [active rank] longest blended run of the tile's pixels (nullable)
 };
 
-// SELECT: the blend of each group of kUnroll splats with selects instead of
-// branches (more instructions, shorter dependent chains) - the better choice
-// when few warps share an SM (a sparse step); with many warps per SM the
-// branches' skipped work wins.  Both produce the same bits.
-template <bool SELECT>
-__device__ __forceinline__ void render_tile_fwd(const RasterArgs& a, int j, Splat* sm, float* __restrict__ out_rgb,
+// Two fp32 values in one 64-bit register pair: each operation is the IEEE
+// operation on both, in one issue slot.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float y;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
+// The rectangle (x0, y0, x1, y1) outside which a splat's alpha stays below
+// 1/255: splat_rows along both axes (half-width sqrt(2 tau c / det)), with
+// approximate functions and tau rounded up by 1e-6, well inside the margins.
+__device__ __forceinline__ float4 splat_reach(float2 xy, const float4& c) {
+  const float x = 255.f * c.w;
+  if (!(x > 1.f)) return make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
+  const float det = c.x * c.z - c.y * c.y;
+  if (!(det > 0.f) || !(c.x > 0.f)) return make_float4(-INFINITY, -INFINITY, INFINITY, INFINITY);
+  const float k = __fdividef(2.f * (__logf(x) + 1e-6f), det);
+  const float h = sqrt_approx(k * c.x) * 1.001f + 1e-3f, w = sqrt_approx(k * c.z) * 1.001f + 1e-3f;
+  return make_float4(xy.x - w, xy.y - h, xy.x + w, xy.y + h);
+}
+__device__ __forceinline__ bool splat_reaches(float2 xy, const float4& c, float4 box) {
+  const float4 r = splat_reach(xy, c);
+  return r.w >= box.y && r.y <= box.w && r.z >= box.x && r.x <= box.z;
+}
+
+// ---------------------------------------------------------------------------
+// The forward walk.  Every warp takes 32 PPL sampled pixels of a tile and
+// walks the tile's list on its own, in chunks of 32 positions: one splat per
+// lane is fetched (a chunk ahead) and tested against the rectangle of the
+// warp's pixels, the ones that can reach it are kept in shared memory in pairs,
+// and the pairs are evaluated in packed fp32 arithmetic, two splats an issue
+// slot.  Only the blend goes through a pair one after the other, with the same
+// operations in the same order as a walk of single splats, so the results are
+// that walk's bits: a splat that a pixel skips has alpha 0 there, which leaves
+// T and the colour as they are.
+//
+// Bound: instruction issue (every tile of 1M Gaussians at 1957x1091: 80 %
+// issue); in sparse launches the chain of the longest list.  Against one thread
+// per pixel over splats staged by the block, one splat at a time: that view
+// 511 -> 313 us, the dense view of 500k Gaussians 279 -> 181, 720 tiles of 85
+// pixels 56 -> 47, 3600 of 25 pixels 95 -> 67, eight views of 3M Gaussians 690 ->
+// 541.  Two pixels a lane halve the per-chunk work (358 -> 313 and 194 -> 181 us
+// for the whole tiles above) but lengthen the chains (20 whole tiles: 9.6 ->
+// 12.2 us; 85 pixels a tile: 541 -> 646 us, half of the second warp idles).
+// Staging the list once per block saves gathers (the L1 is 55-73 % busy with
+// them) but its barriers cost more: 390 -> 421 us for the first view.
+// ---------------------------------------------------------------------------
+struct __align__(16) FwdPair {
+  f32x2 nx, ny;  // minus the centre
+  f32x2 ca, cb;  // the pre-scaled conic
+  f32x2 cc, op;  // and the opacity
+  f32x2 cr, cg;  // colour
+  f32x2 cbl;
+  int end[2];    // 1 + position in the tile's list
+};
+constexpr int kFwdPairs = 16;  // a chunk's splats
+
+static size_t fwd_smem(int threads) { return (size_t)(threads / 32) * kFwdPairs * sizeof(FwdPair); }
+
+__device__ __forceinline__ void fwd_stage(FwdPair* Q, int i, const SplatRaw& w, int end) {
+  FwdPair& P = Q[i >> 1];
+  const int e = i & 1;
+  reinterpret_cast<float*>(&P.nx)[e] = -w.xy.x;
+  reinterpret_cast<float*>(&P.ny)[e] = -w.xy.y;
+  reinterpret_cast<float*>(&P.ca)[e] = __fmul_rn(w.c.x, kPow2A);
+  reinterpret_cast<float*>(&P.cb)[e] = __fmul_rn(w.c.y, kPow2B);
+  reinterpret_cast<float*>(&P.cc)[e] = __fmul_rn(w.c.z, kPow2A);
+  reinterpret_cast<float*>(&P.op)[e] = w.c.w;
+  reinterpret_cast<float*>(&P.cr)[e] = w.r;
+  reinterpret_cast<float*>(&P.cg)[e] = w.g;
+  reinterpret_cast<float*>(&P.cbl)[e] = w.b;
+  P.end[e] = end;
+}
+
+// One pixel's state.
+struct FwdPix {
+  float T, C0, C1, C2;
+  int last;
+  bool done;
+};
+
+// A pair against one pixel.
+__device__ __forceinline__ void fwd_pair(const FwdPair& P, f32x2 X, f32x2 Y, FwdPix& q) {
+  const f32x2 dx = add2(X, P.nx), dy = add2(Y, P.ny);
+  const f32x2 p = fma2(fma2(P.ca, dx, mul2(P.cb, dy)), dx, mul2(mul2(P.cc, dy), dy));  // splat_pow2 of both
+  const float p0 = lo2(p), p1 = hi2(p);
+  const f32x2 og = mul2(P.op, pk2(ex2_approx(p0), ex2_approx(p1)));
+  const f32x2 over = add2(og, pk2(-kAlphaMin, -kAlphaMin));  // not negative where alpha >= 1/255
+  const bool ok0 = fminf(-p0, lo2(over)) >= 0.f && !q.done, ok1 = fminf(-p1, hi2(over)) >= 0.f && !q.done;
+  const float a0 = ok0 ? fminf(kAlphaMax, lo2(og)) : 0.f, a1 = ok1 ? fminf(kAlphaMax, hi2(og)) : 0.f;
+  const float T1 = __fmul_rn(q.T, __fsub_rn(1.f, a0)), T2 = __fmul_rn(T1, __fsub_rn(1.f, a1));
+  float w0 = __fmul_rn(a0, q.T), w1 = __fmul_rn(a1, T1), Tn = T2;
+  int l = ok1 ? P.end[1] : ok0 ? P.end[0] : q.last;
+  if (T2 < kTStop) {  // T itself is not below the stop: the walk ends in this pair, once a pixel
+    q.done = true;
+    w1 = 0.f;
+    Tn = T1;
+    l = ok0 ? P.end[0] : q.last;
+    if (T1 < kTStop) {
+      w0 = 0.f;
+      Tn = q.T;
+      l = q.last;
+    }
+  }
+  q.C0 = __fmaf_rn(w1, hi2(P.cr), __fmaf_rn(w0, lo2(P.cr), q.C0));
+  q.C1 = __fmaf_rn(w1, hi2(P.cg), __fmaf_rn(w0, lo2(P.cg), q.C1));
+  q.C2 = __fmaf_rn(w1, hi2(P.cbl), __fmaf_rn(w0, lo2(P.cbl), q.C2));
+  q.T = Tn;
+  q.last = l;
+}
+
+// Entry i of the queue against one pixel (where a record is not finite).
+__device__ __forceinline__ void fwd_single(const FwdPair* Q, int i, float px, float py, FwdPix& q) {
+  const float* P = reinterpret_cast<const float*>(Q + (i >> 1)) + (i & 1);
+  const float4 co = make_float4(P[4], P[6], P[8], P[10]);
+  float al, G;
+  if (q.done || !splat_alpha(co, __fadd_rn(px, P[0]), __fadd_rn(py, P[2]), al, G)) return;
+  const float Tn = __fmul_rn(q.T, __fsub_rn(1.f, al));
+  if (Tn < kTStop) {
+    q.done = true;
+    return;
+  }
+  const float wt = __fmul_rn(al, q.T);
+  q.C0 = __fmaf_rn(wt, P[12], q.C0);
+  q.C1 = __fmaf_rn(wt, P[14], q.C1);
+  q.C2 = __fmaf_rn(wt, P[16], q.C2);
+  q.T = Tn;
+  q.last = Q[i >> 1].end[i & 1];
+}
+
+// Forward of active tile j by a block of one warp per 32 PPL sampled pixels.
+template <int PPL>
+__device__ __forceinline__ void render_tile_fwd(const RasterArgs& a, int j, FwdPair* sm, float* __restrict__ out_rgb,
                                                 float* __restrict__ out_T, int32_t* __restrict__ out_last,
-                                                Ckpt ck = Ckpt{nullptr, 0, 0, nullptr, nullptr}) {
+                                                const Ckpt& ck) {
+  const unsigned full = 0xffffffffu;
+  __shared__ int s_tl;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  FwdPair* Q = sm + warp * kFwdPairs;
   const int t = a.active_tiles ? a.active_tiles[j] : j;
   const int p0 = a.pix_off[j], p1 = a.pix_off[j + 1];
-  const bool has_pix = p0 + (int)threadIdx.x < p1;
-  const int s = p0 + threadIdx.x;
-  float px = 0.f, py = 0.f;
-  if (has_pix) {
-    const int l = a.pix_idx[s];
-    px = (float)((t % a.tiles_x) * TGS_TILE + (l & 15)) + 0.5f;
-    py = (float)((t / a.tiles_x) * TGS_TILE + (l >> 4)) + 0.5f;
+  int s[PPL];
+  float px[PPL], py[PPL];
+  f32x2 X[PPL], Y[PPL];
+  FwdPix q[PPL];
+  float4 box = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+  for (int u = 0; u < PPL; ++u) {
+    s[u] = p0 + 32 * (PPL * warp + u) + lane;
+    // a whole tile: the warps take 8 x 4 (8 x 8) blocks of it, which fewer splats reach than bands of rows
+    if (p1 - p0 == TGS_TILE_PIX)
+      s[u] = p0 + (4 * (PPL * (warp >> 1) + u) + (lane >> 3)) * TGS_TILE + 8 * (warp & 1) + (lane & 7);
+    q[u] = FwdPix{1.f, 0.f, 0.f, 0.f, 0, s[u] >= p1};
+    px[u] = py[u] = 0.f;
+    if (s[u] < p1) {
+      const int l = a.pix_idx[s[u]];
+      px[u] = (float)((t % a.tiles_x) * TGS_TILE + (l & 15)) + 0.5f;
+      py[u] = (float)((t / a.tiles_x) * TGS_TILE + (l >> 4)) + 0.5f;
+      box = make_float4(fminf(box.x, px[u]), fminf(box.y, py[u]), fmaxf(box.z, px[u]), fmaxf(box.w, py[u]));
+    }
+    X[u] = pk2(px[u], px[u]);
+    Y[u] = pk2(py[u], py[u]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    box.x = fminf(box.x, __shfl_xor_sync(full, box.x, o));
+    box.y = fminf(box.y, __shfl_xor_sync(full, box.y, o));
+    box.z = fmaxf(box.z, __shfl_xor_sync(full, box.z, o));
+    box.w = fmaxf(box.w, __shfl_xor_sync(full, box.w, o));
+  }
+  if (ck.tile_last) {  // the tile's longest blended run, for the pieces of the backward
+    if (threadIdx.x == 0) s_tl = 0;
+    __syncthreads();
   }
   const int2 range = a.ranges[j];
-  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-  int last = 0;
-  bool done = !has_pix;
-  const int B = blockDim.x;
-  const float2 band = warp_rows(has_pix, py);  // splats outside it are skipped by the whole warp
-  const int lane = threadIdx.x & 31;
-  // the next batch's records are fetched into registers while the current
-  // one is blended, and the list entries (ids) of the batch after it
-  SplatRaw nxt;
+  // a chunk's records are fetched while the chunk before is walked, and the
+  // list entries (ids) of the chunk after it
+  SplatRaw w;
   int idn = 0;
-  const int tid = threadIdx.x;
-  if (range.x + tid < range.y) fetch_splat(a, a.vals[range.x + tid], nxt);
-  if (range.x + B + tid < range.y) idn = a.vals[range.x + B + tid];
-  for (int base = range.x; base < range.y; base += B) {
-    if (__syncthreads_count(done) == B) break;
-    if (base + tid < range.y) finish_splat(nxt, sm[tid]);
-    __syncthreads();
-    if (base + B + tid < range.y) fetch_splat(a, idn, nxt);
-    if (base + 2 * B + tid < range.y) idn = a.vals[base + 2 * B + tid];
-    const int cnt = min(B, range.y - base);
-    // Runs of kCkptEvery positions (B is a multiple of it), walked by every
-    // thread so that the warp's ballot below stays converged: the checkpoint
-    // in front of each run, then the run's splats that can reach the warp's
-    // rows (a bit mask from one ballot), kUnroll at a time: their alphas do
-    // not depend on T, so they are evaluated together and only the blend runs
-    // in list order.  The splats left out fail every alpha test of the warp.
-    for (int q32 = 0; q32 < cnt; q32 += kCkptEvery) {
-      if (ck.data && !done) {
-        const int c = (base - range.x + q32) / kCkptEvery - 1;  // state in front of this run
-        if (c >= 0 && c < ck.n_slots) ck.data[c * ck.stride + s] = make_float4(T, C0, C1, C2);
+  if (range.x + lane < range.y) fetch_splat(a, a.vals[range.x + lane], w);
+  if (range.x + 32 + lane < range.y) idn = a.vals[range.x + 32 + lane];
+  for (int base = range.x; base < range.y; base += 32) {
+    bool all = true;
+#pragma unroll
+    for (int u = 0; u < PPL; ++u) all = all && q[u].done;
+    if (__all_sync(full, all)) break;
+    if (ck.data) {
+      const int c = (base - range.x) / kCkptEvery - 1;  // state in front of this chunk
+      if (c >= 0 && c < ck.n_slots) {
+#pragma unroll
+        for (int u = 0; u < PPL; ++u)
+          if (!q[u].done) ck.data[c * ck.stride + s[u]] = make_float4(q[u].T, q[u].C0, q[u].C1, q[u].C2);
       }
-      const int qe = min(cnt, q32 + kCkptEvery);
-      bool in_l = false;
-      if (q32 + lane < qe) {
-        const float2 yr = sm[q32 + lane].yr;
-        in_l = yr.y >= band.x && yr.x <= band.y;
+    }
+    const bool keep = base + lane < range.y && splat_reaches(w.xy, w.c, box);
+    const bool fin = !keep || fabsf(w.xy.x) + fabsf(w.xy.y) + fabsf(w.c.x) + fabsf(w.c.y) + fabsf(w.c.z) +
+                                      fabsf(w.r) + fabsf(w.g) + fabsf(w.b) <
+                                  INFINITY;
+    const unsigned m = __ballot_sync(full, keep);
+    const bool fast = __all_sync(full, fin);
+    __syncwarp();  // the chunk before is no longer read
+    const int n = __popc(m);
+    if (keep) fwd_stage(Q, __popc(m & ((1u << lane) - 1u)), w, base + lane + 1 - range.x);
+    if ((n & 1) && lane == 0) {  // the last pair's second half: a splat that blends nowhere
+      SplatRaw z;
+      z.xy = make_float2(0.f, 0.f);
+      z.c = make_float4(0.f, 0.f, 0.f, 0.f);
+      z.r = z.g = z.b = 0.f;
+      fwd_stage(Q, n, z, 0);
+    }
+    __syncwarp();
+    if (base + 32 + lane < range.y) fetch_splat(a, idn, w);
+    if (base + 64 + lane < range.y) idn = a.vals[base + 64 + lane];
+    if (fast) {
+      const int pairs = (n + 1) >> 1;
+#pragma unroll 2
+      for (int i = 0; i < pairs; ++i) {
+#pragma unroll
+        for (int u = 0; u < PPL; ++u) fwd_pair(Q[i], X[u], Y[u], q[u]);
       }
-      unsigned mask = __ballot_sync(0xffffffffu, in_l);
-      while (mask && !done) {
-        int qq[kUnroll];
-        float al[kUnroll];
-        bool ok[kUnroll];
+    } else {  // an infinite or NaN record: splat by splat, so that it stays with the pixels that blend it
+      for (int i = 0; i < n; ++i) {
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const bool val = mask != 0u;
-          qq[u] = val ? q32 + __ffs(mask) - 1 : q32;
-          mask &= mask - 1u;
-          const float2 xy = sm[qq[u]].xy;
-          float G;
-          ok[u] = (SELECT ? splat_alpha_nb(sm[qq[u]].co, __fsub_rn(px, xy.x), __fsub_rn(py, xy.y), al[u], G)
-                          : splat_alpha(sm[qq[u]].co, __fsub_rn(px, xy.x), __fsub_rn(py, xy.y), al[u], G)) &&
-                  val;
-        }
-        if (!SELECT) {
-#pragma unroll
-          for (int u = 0; u < kUnroll; ++u) {
-            if (!ok[u]) continue;
-            const float Tn = __fmul_rn(T, __fsub_rn(1.f, al[u]));
-            if (Tn < kTStop) {
-              done = true;
-              break;
-            }
-            const float4 rgb = sm[qq[u]].rgb;
-            const float w = al[u] * T;
-            C0 += w * rgb.x;
-            C1 += w * rgb.y;
-            C2 += w * rgb.z;
-            T = Tn;
-            last = base + qq[u] + 1 - range.x;
-          }
-          continue;
-        }
-        // the blend without branches: a splat past the stopping one, or
-        // skipped, leaves the state as it is
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const float Tn = __fmul_rn(T, __fsub_rn(1.f, al[u]));
-          const bool stop = ok[u] && !done && Tn < kTStop;
-          const bool take = ok[u] && !done && !stop;
-          done = done || stop;
-          const float4 rgb = sm[qq[u]].rgb;
-          const float w = al[u] * T;
-          C0 = take ? C0 + w * rgb.x : C0;
-          C1 = take ? C1 + w * rgb.y : C1;
-          C2 = take ? C2 + w * rgb.z : C2;
-          T = take ? Tn : T;
-          last = take ? base + qq[u] + 1 - range.x : last;
-        }
+        for (int u = 0; u < PPL; ++u) fwd_single(Q, i, px[u], py[u], q[u]);
       }
     }
   }
-  if (has_pix) {
-    out_rgb[3 * s] = C0 + T * a.bg[0];
-    out_rgb[3 * s + 1] = C1 + T * a.bg[1];
-    out_rgb[3 * s + 2] = C2 + T * a.bg[2];
-    out_T[s] = T;
-    out_last[s] = last;
+  int longest = 0;
+#pragma unroll
+  for (int u = 0; u < PPL; ++u) {
+    if (s[u] < p1) {
+      out_rgb[3 * s[u]] = q[u].C0 + q[u].T * a.bg[0];
+      out_rgb[3 * s[u] + 1] = q[u].C1 + q[u].T * a.bg[1];
+      out_rgb[3 * s[u] + 2] = q[u].C2 + q[u].T * a.bg[2];
+      out_T[s[u]] = q[u].T;
+      out_last[s[u]] = q[u].last;
+    }
+    longest = max(longest, q[u].last);
   }
-  if (ck.tile_last) {  // the tile's longest blended run, for the pieces of the backward
-    __shared__ int s_tl;
-    __syncthreads();
-    if (threadIdx.x == 0) s_tl = 0;
-    __syncthreads();
-    if (last > 0) atomicMax(&s_tl, last);
+  if (ck.tile_last) {
+    if (longest > 0) atomicMax(&s_tl, longest);
     __syncthreads();
     if (threadIdx.x == 0) ck.tile_last[j] = s_tl;
   }
 }
 
-template <bool SELECT>
-__global__ void k_render_fwd(RasterArgs a, float* __restrict__ out_rgb, float* __restrict__ out_T,
-                             int32_t* __restrict__ out_last, Ckpt ck) {
-  extern __shared__ Splat sm[];
+template <int PPL>
+__global__ void __launch_bounds__(TGS_TILE_PIX / PPL) k_render_fwd(RasterArgs a, float* __restrict__ out_rgb,
+                                                                   float* __restrict__ out_T,
+                                                                   int32_t* __restrict__ out_last, Ckpt ck) {
+  extern __shared__ __align__(16) FwdPair fwd_sm[];
   const int j = blockIdx.x;
   if (j >= *a.n_active) return;
-  render_tile_fwd<SELECT>(a, j, sm, out_rgb, out_T, out_last, ck);
+  render_tile_fwd<PPL>(a, j, fwd_sm, out_rgb, out_T, out_last, ck);
 }
 
 // The same forward with two threads per sampled pixel: a warp holds 16
@@ -472,141 +632,6 @@ __global__ void k_render_fwd_pair(RasterArgs a, float* __restrict__ out_rgb, flo
   const int j = blockIdx.x;
   if (j >= *a.n_active) return;
   render_tile_fwd_pair<SELECT>(a, j, sm, out_rgb, out_T, out_last, ck);
-}
-
-// The same forward with every warp on its own: a warp takes 32 sampled
-// pixels of one tile (piece `piece` of tile j; j < 0 for none), stages its
-// own 32-splat batches of the tile's list (one per lane, the next batch
-// fetched while the current one is blended), walks them for its pixels and
-// stops when they have saturated.  Same results as render_tile_fwd (the same
-// per-pixel operations in the same order).  Returns the lane's blended count.
-template <bool SELECT>
-__device__ __forceinline__ int render_tile_fwd_warp(const RasterArgs& a, int j, int piece, Splat* sm,
-                                                    float* __restrict__ out_rgb, float* __restrict__ out_T,
-                                                    int32_t* __restrict__ out_last, const Ckpt& ck) {
-  const int lane = threadIdx.x & 31;
-  const int t = j >= 0 ? (a.active_tiles ? a.active_tiles[j] : j) : 0;
-  const int p0 = j >= 0 ? a.pix_off[j] : 0, p1 = j >= 0 ? a.pix_off[j + 1] : 0;
-  const int s = p0 + 32 * piece + lane;
-  const bool has_pix = s < p1;
-  float px = 0.f, py = 0.f;
-  if (has_pix) {
-    const int l = a.pix_idx[s];
-    px = (float)((t % a.tiles_x) * TGS_TILE + (l & 15)) + 0.5f;
-    py = (float)((t / a.tiles_x) * TGS_TILE + (l >> 4)) + 0.5f;
-  }
-  const int2 range = j >= 0 ? a.ranges[j] : make_int2(0, 0);
-  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-  int last = 0;
-  bool done = !has_pix;
-  const float2 band = warp_rows(has_pix, py);
-  SplatRaw nxt;
-  int idn = 0;
-  if (range.x + lane < range.y) fetch_splat(a, a.vals[range.x + lane], nxt);
-  if (range.x + kCkptEvery + lane < range.y) idn = a.vals[range.x + kCkptEvery + lane];
-  for (int base = range.x; base < range.y; base += kCkptEvery) {
-    if (__all_sync(0xffffffffu, done)) break;
-    __syncwarp();
-    if (base + lane < range.y) finish_splat(nxt, sm[lane]);
-    __syncwarp();
-    if (base + kCkptEvery + lane < range.y) fetch_splat(a, idn, nxt);
-    if (base + 2 * kCkptEvery + lane < range.y) idn = a.vals[base + 2 * kCkptEvery + lane];
-    const int cnt = min(kCkptEvery, range.y - base);
-    if (ck.data && !done) {
-      const int c = (base - range.x) / kCkptEvery - 1;  // state in front of this run
-      if (c >= 0 && c < ck.n_slots) ck.data[c * ck.stride + s] = make_float4(T, C0, C1, C2);
-    }
-    bool in_l = false;
-    if (lane < cnt) {
-      const float2 yr = sm[lane].yr;
-      in_l = yr.y >= band.x && yr.x <= band.y;
-    }
-    unsigned mask = __ballot_sync(0xffffffffu, in_l);
-    while (mask && !done) {
-      int qq[kUnroll];
-      float al[kUnroll];
-      bool ok[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const bool val = mask != 0u;
-        qq[u] = val ? __ffs(mask) - 1 : 0;
-        mask &= mask - 1u;
-        const float2 xy = sm[qq[u]].xy;
-        float G;
-        ok[u] = (SELECT ? splat_alpha_nb(sm[qq[u]].co, __fsub_rn(px, xy.x), __fsub_rn(py, xy.y), al[u], G)
-                        : splat_alpha(sm[qq[u]].co, __fsub_rn(px, xy.x), __fsub_rn(py, xy.y), al[u], G)) &&
-                val;
-      }
-      if (!SELECT) {
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          if (!ok[u]) continue;
-          const float Tn = __fmul_rn(T, __fsub_rn(1.f, al[u]));
-          if (Tn < kTStop) {
-            done = true;
-            break;
-          }
-          const float4 rgb = sm[qq[u]].rgb;
-          const float w = al[u] * T;
-          C0 += w * rgb.x;
-          C1 += w * rgb.y;
-          C2 += w * rgb.z;
-          T = Tn;
-          last = base + qq[u] + 1 - range.x;
-        }
-        continue;
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const float Tn = __fmul_rn(T, __fsub_rn(1.f, al[u]));
-        const bool stop = ok[u] && !done && Tn < kTStop;
-        const bool take = ok[u] && !done && !stop;
-        done = done || stop;
-        const float4 rgb = sm[qq[u]].rgb;
-        const float w = al[u] * T;
-        C0 = take ? C0 + w * rgb.x : C0;
-        C1 = take ? C1 + w * rgb.y : C1;
-        C2 = take ? C2 + w * rgb.z : C2;
-        T = take ? Tn : T;
-        last = take ? base + qq[u] + 1 - range.x : last;
-      }
-    }
-  }
-  if (has_pix) {
-    out_rgb[3 * s] = C0 + T * a.bg[0];
-    out_rgb[3 * s + 1] = C1 + T * a.bg[1];
-    out_rgb[3 * s + 2] = C2 + T * a.bg[2];
-    out_T[s] = T;
-    out_last[s] = last;
-  }
-  return last;
-}
-
-// Several tiles per block for the warp-independent walk: wpt warps per tile
-// (32 sampled pixels each), blockDim.x / (32 wpt) tiles per block, so that
-// tiles of few sampled pixels (a warp each at 32 or fewer) still fill 8-warp
-// blocks.  The block meets once, at the end, for each tile's longest blended
-// run.
-template <bool SELECT>
-__global__ void __launch_bounds__(256) k_render_fwd_w(RasterArgs a, int wpt, float* __restrict__ out_rgb,
-                                                      float* __restrict__ out_T, int32_t* __restrict__ out_last,
-                                                      Ckpt ck) {
-  __shared__ Splat sm[8][kCkptEvery];
-  __shared__ int s_tl[8];
-  const int warp = threadIdx.x >> 5;
-  const int tpb = (int)(blockDim.x >> 5) / wpt;
-  const int lt = warp / wpt, piece = warp - lt * wpt;
-  const int n_act = *a.n_active;
-  if (blockIdx.x * tpb >= n_act) return;  // the whole block
-  const int j = blockIdx.x * tpb + lt < n_act ? blockIdx.x * tpb + lt : -1;
-  if (threadIdx.x < 8) s_tl[threadIdx.x] = 0;
-  __syncthreads();
-  const int last = render_tile_fwd_warp<SELECT>(a, j, piece, sm[warp], out_rgb, out_T, out_last, ck);
-  if (ck.tile_last) {  // the tile's longest blended run, for the pieces of the backward
-    if (last > 0) atomicMax(&s_tl[lt], last);
-    __syncthreads();
-    if (j >= 0 && piece == 0 && (threadIdx.x & 31) == 0) ck.tile_last[j] = s_tl[lt];
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -847,58 +872,6 @@ constexpr int kBwdPpl = 4;      // most pixels a lane
 // with four warps a block, 57 with one).  20 blocks an SM: 96 registers.
 constexpr int kBwdBlocksPerSm = 20;
 
-// Two fp32 values in one 64-bit register pair: each operation is the IEEE
-// operation on both, in one issue slot.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float lo2(f32x2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return a;
-}
-__device__ __forceinline__ float hi2(f32x2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return b;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float min3(float a, float b, float c) {
-  float y;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-  return y;
-}
-
 // Two kept splats as the replay reads them (element e in half e).
 struct __align__(16) BwdPair {
   f32x2 nx, ny;      // minus the centre
@@ -912,19 +885,6 @@ struct __align__(16) BwdPair {
   int id[2];
 };
 constexpr int kBwdPairs = 17;  // a chunk's 32 splats and one left over
-
-// Whether a splat's alpha can reach 1/255 in the rectangle box (x0, y0, x1,
-// y1): splat_rows along both axes (half-width sqrt(2 tau c / det)), with
-// approximate functions and tau rounded up by 1e-6, well inside the margins.
-__device__ __forceinline__ bool splat_reaches(float2 xy, const float4& c, float4 box) {
-  const float x = 255.f * c.w;
-  if (!(x > 1.f)) return false;
-  const float det = c.x * c.z - c.y * c.y;
-  if (!(det > 0.f) || !(c.x > 0.f)) return true;
-  const float k = __fdividef(2.f * (__logf(x) + 1e-6f), det);
-  const float h = sqrt_approx(k * c.x) * 1.001f + 1e-3f, w = sqrt_approx(k * c.z) * 1.001f + 1e-3f;
-  return xy.y + h >= box.y && xy.y - h <= box.w && xy.x + w >= box.x && xy.x - w <= box.z;
-}
 
 // Entry i of the warp's queue.
 __device__ __forceinline__ void bwd_stage(BwdPair* Q, int i, const SplatRaw& w, float pos) {
@@ -1403,12 +1363,13 @@ __device__ __forceinline__ void item_view(const BatchArgs& b, int item, int& v, 
   q = item - b.base[v];
 }
 
-__global__ void k_render_fwd_batched(BatchArgs b, int* __restrict__ counter) {
-  extern __shared__ Splat sm[];
+template <int PPL>
+__global__ void __launch_bounds__(TGS_TILE_PIX / PPL) k_render_fwd_batched(BatchArgs b, int* __restrict__ counter) {
+  extern __shared__ __align__(16) FwdPair fwd_sm[];
   __shared__ int s_item;
   int v, j;
   while (next_item(b, counter, &s_item, v, j)) {
-    if (j < *b.a[v].n_active) render_tile_fwd<false>(b.a[v], j, sm, b.rgb[v], b.T[v], b.last[v], b.ck[v]);
+    if (j < *b.a[v].n_active) render_tile_fwd<PPL>(b.a[v], j, fwd_sm, b.rgb[v], b.T[v], b.last[v], b.ck[v]);
   }
 }
 
@@ -1518,6 +1479,14 @@ static BwdSplit bwd_split(int64_t tiles, int n_pix_max, const Ckpt& ck) {
 
 static int block_for(int n_pix_max) { return std::min(256, std::max(32, (n_pix_max + 31) / 32 * 32)); }
 
+// Fewer than 16 warps per SM at one pixel a thread (B threads a tile).
+static bool few_warps(int64_t n_tiles, int B) { return n_tiles * (B / 32) < 16 * (int64_t)device_sm_count(); }
+
+// Pixels a lane of the forward walk: two for tiles of more than 128 pixels,
+// where the launch has warps to spare.
+static int fwd_ppl(int B, bool few) { return B > 128 && !few ? 2 : 1; }
+static int fwd_threads(int B, int ppl) { return (B / 32 + ppl - 1) / ppl * 32; }
+
 
 // Whether the automatic choice may pick the split walk: measured slower than
 // the sequential walk at 500k Gaussians, 720 tiles of 85 pixels (0.085-0.089
@@ -1530,13 +1499,9 @@ static int g_fwd_split = 0;
 
 // The automatic choice of the walk with two threads per pixel: for tiles of
 // at most 32 sampled pixels in a sparse launch, where one warp per tile
-// leaves the GPU short of warps.  Measured at 500k Gaussians, 1280x720, 720
-// tiles of 25 pixels: 0.046 ms, against 0.054 for the warp-independent walk
-// (eight tiles per block) and 0.064 for one 32-thread block per tile.  At 85
-// pixels per tile (0.068 against 0.060) and in launches of several waves
-// (3600 tiles of 85 pixels: 0.216 against 0.162) the sequential block walk
-// stays faster: the composition and the second half's walk past the stop
-// cost more than the shorter chains gain.
+// leaves the GPU short of warps.  Elsewhere the composition and the second
+// half's walk past the stop cost more than the shorter chains gain (at 85
+// pixels per tile 0.068 ms against 0.047).
 static bool pair_walk_auto(int B, bool sparse) { return B == 32 && sparse; }
 
 // Groups per tile of the split forward for a launch of n_active tiles of B
@@ -1624,11 +1589,10 @@ extern "C" tgs_status tgs_render_sampled(const tgs_projected* proj, const int32_
                                                                                                  n_last, ck);
     return check_launch();
   }
-  // selects when the launch gives fewer than 16 warps per SM
-  const bool sparse = (int64_t)n_active_max * (B / 32) < 16 * (int64_t)device_sm_count();
-  if (g_fwd_split == 5 || (g_fwd_split == 0 && pair_walk_auto(B, sparse))) {  // two threads per pixel
+  const bool few = few_warps(n_active_max, B);
+  if (g_fwd_split == 5 || (g_fwd_split == 0 && pair_walk_auto(B, few))) {  // two threads per pixel
     const int B2 = 32 * ((n_pix_max + 15) / 16);
-    if (sparse)
+    if (few)
       k_render_fwd_pair<true><<<n_active_max, B2, B2 * sizeof(Splat), (cudaStream_t)stream>>>(a, rgb, T_final, n_last,
                                                                                               ck);
     else
@@ -1636,19 +1600,9 @@ extern "C" tgs_status tgs_render_sampled(const tgs_projected* proj, const int32_
                                                                                                n_last, ck);
     return check_launch();
   }
-  if (g_fwd_split == 3) {
-    const int wpt = B / 32, tpb = 8 / wpt;
-    const int grid = (n_active_max + tpb - 1) / tpb;
-    if (sparse)
-      k_render_fwd_w<true><<<grid, 32 * wpt * tpb, 0, (cudaStream_t)stream>>>(a, wpt, rgb, T_final, n_last, ck);
-    else
-      k_render_fwd_w<false><<<grid, 32 * wpt * tpb, 0, (cudaStream_t)stream>>>(a, wpt, rgb, T_final, n_last, ck);
-    return check_launch();
-  }
-  if (sparse)
-    k_render_fwd<true><<<n_active_max, B, B * sizeof(Splat), (cudaStream_t)stream>>>(a, rgb, T_final, n_last, ck);
-  else
-    k_render_fwd<false><<<n_active_max, B, B * sizeof(Splat), (cudaStream_t)stream>>>(a, rgb, T_final, n_last, ck);
+  const int ppl = fwd_ppl(B, few), threads = fwd_threads(B, ppl);
+  (ppl == 2 ? k_render_fwd<2> : k_render_fwd<1>)<<<n_active_max, threads, fwd_smem(threads), (cudaStream_t)stream>>>(
+      a, rgb, T_final, n_last, ck);
   return check_launch();
 }
 
@@ -1807,7 +1761,9 @@ extern "C" tgs_status tgs_render_batched_resident(int32_t n_pix_max, int32_t bac
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_batched_kernel(std::min(B / 32, kBwdPpl), false),
                                                   32, 0);
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_fwd_batched, B, B * sizeof(Splat));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_ppl(B, false) == 2 ? k_render_fwd_batched<2> : k_render_fwd_batched<1>,
+                                                  fwd_threads(B, fwd_ppl(B, false)),
+                                                  fwd_smem(fwd_threads(B, fwd_ppl(B, false))));
   *ctas = sms * per_sm;
   return check_launch();
 }
@@ -1822,7 +1778,8 @@ extern "C" tgs_status tgs_render_sampled_batched(const tgs_view_batch* views, in
   cudaStream_t s = (cudaStream_t)stream;
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   if (b.base[n_views] == 0) return check_launch();
-  k_render_fwd_batched<<<grid_ctas, B, B * sizeof(Splat), s>>>(b, counter);
+  const int ppl = fwd_ppl(B, false), threads = fwd_threads(B, ppl);
+  (ppl == 2 ? k_render_fwd_batched<2> : k_render_fwd_batched<1>)<<<grid_ctas, threads, fwd_smem(threads), s>>>(b, counter);
   return check_launch();
 }
 

@@ -563,78 +563,163 @@ __global__ void __launch_bounds__(kBwThreads, 1) k_mlp_backward_tc(
 // same kernel: per 128-row tile, D1 = X W1^T and D2 = H1 W2^T on the tensor
 // cores, h1, h2 and y from them in the epilogues, then the backward above
 // (dH1 = [H1 > 0] (dH2 W2), dW2 | db2 and dW1 | db1 as contractions over the
-// rows).  The activations never leave the SM: the pair of kernels that stores
-// h1 and h2 (512 bytes a row) and reads them back moved about 1.7 GB at the
-// 200-view size.  256 threads, thread t on row t % 128 and hidden units
-// 64 (t / 128) .. + 63; dW3 and db3 (fp32 dy times the bf16 h2, as in the
-// backward above) in registers per thread over the whole pass, reduced once.
-// TMEM: D1, then dH1, in columns 0-127; dW2 | db2 in 128-271; dW1 | db1 in
-// 288-319; D2 in 320-447.  Shared memory holds each operand once, as rows
-// (bf16 X, H1, dH2 and dH1 of the tile's 128 rows): the forward's
-// contractions read them K-major, the weight gradients (contractions over the
-// rows) MN-major through the same core matrices, so no operand is copied
-// transposed; X and H1 carry a column of ones for the bias gradients.  The roundings are the
-// forward's and the backward's: x, h1, h2, dH2 and dH1 in bf16, fp32 sums; y
-// sums its two halves of 64 units and then adds b3.
-constexpr uint32_t FT_W2T = 0;                            // W2^T [128 j][128 k] (B of dH1)
-constexpr uint32_t FT_W2 = FT_W2T + TH * TH * 2;          // W2 [128 n][128 k] (B of layer 2)
+// rows).  The activations never leave the SM.  256 epilogue threads, thread t on row
+// t % 128 and hidden units 64 (t / 128) .. + 63; dW3 and db3 (fp32 dy times the
+// bf16 h2, as in the backward above) in registers per thread over the whole
+// pass, reduced once.
+//
+// A CTA has two tiles in flight, in two slots: while the tensor cores work on
+// one, the threads run the other's epilogue.  A tile's four steps depend on one
+// another, and with one tile a CTA waited for the tensor cores four times a
+// tile, an SM 16 % busy with them.  What lets two fit:
+//   - one accumulator of 128 TMEM columns a slot, since D1, D2 and dH1 of a
+//     tile follow one another (slots in columns 0-127 and 128-255, dW2 | db2 in
+//     256-399 and dW1 | db1 in 416-447, for both);
+//   - dH1 in the buffer of dH2, once both contractions that read dH2 are done;
+//   - W2 kept once, read K-major by layer 2 and MN-major by dH1 = dH2 W2.
+// A ninth warp issues the contractions.  The epilogue threads meet it, and it
+// them, only through mbarriers (full: a slot's operands are written, 256
+// arrivals; done: its contractions are complete; part: the two halves of a row
+// have their part of y, 64 arrivals), so a warp goes on to the other slot as
+// soon as its own rows are written.  Every wait is bounded: the first that
+// runs out sets a flag, and every thread leaves its loop at its next wait.
+// One thread issues every contraction, so the shared accumulators are added to
+// in order.  The epilogues handle two units an instruction where they can
+// (packed fp32 sums and products, bf16 pairs for ReLU and masks; the mask
+// h1 > 0 is read back from the row tile).
+// Shared memory holds each operand as rows (bf16 X, H1, dH2 / dH1): the
+// forward's contractions read them K-major, the weight gradients (contractions
+// over the rows) MN-major through the same core matrices, so no operand is
+// copied transposed; X and H1 carry a column of ones for the bias gradients.
+// The roundings are the forward's and the backward's: x, h1, h2, dH2 and dH1 in
+// bf16, fp32 sums; y sums its two halves of 64 units and then adds b3.
+// Measured on GB300, 1.7 M rows: 346 us (545 TFLOP/s bf16 of the contractions'
+// 189 GFLOP); one tile at a time with a barrier a step took 528.  Bound by
+// shared memory: 68 % of its cycles carry the epilogues' and the tensor cores'
+// accesses, and the issue slots are 31 % busy.  With 512 epilogue threads of 32
+// units (128 registers) 359 us; with the issuing thread one of the 256 epilogue
+// threads and a barrier a step 368.
+constexpr uint32_t FT_W2 = 0;                             // W2 [128 n][128 k]
 constexpr uint32_t FT_W1 = FT_W2 + TH * TH * 2;           // W1 [128 n][16 k] (B of layer 1)
-// the row tiles (XW, HW, SBO_X, SBO_H above)
-constexpr uint32_t FT_X = FT_W1 + TH * TI * 2;            // [X | 1 | 0]   [128 r][32]: A of layer 1, B of dW1
+constexpr uint32_t FT_SLOT = FT_W1 + TH * TI * 2;         // the slots' row tiles (XW, HW, SBO_X, SBO_H above):
+constexpr uint32_t FT_X = 0;                              // [X | 1 | 0]   [128 r][32]: A of layer 1, B of dW1
 constexpr uint32_t FT_H1 = FT_X + TM * XW * 2;            // [H1 | 1 | 0]  [128 r][144]: A of layer 2, B of dW2
-constexpr uint32_t FT_DH2 = FT_H1 + TM * HW * 2;          // dH2 [128 r][128]: A of dH1 and of dW2
-constexpr uint32_t FT_DH1 = FT_DH2 + TM * TH * 2;         // dH1 [128 r][128]: A of dW1
-constexpr uint32_t FT_PAR = FT_DH1 + TM * TH * 2;         // b1, b2, w3 (fp32) [128 each], b3, y halves [2][128]
-constexpr uint32_t FT_SMEM = FT_PAR + (3 * TH + 4) * 4 + 2 * TM * 4;
+constexpr uint32_t FT_DH = FT_H1 + TM * HW * 2;           // dH2 [128 r][128]: A of dH1 and of dW2; then dH1: A of dW1
+constexpr uint32_t FT_SLOT_BYTES = FT_DH + TM * TH * 2;
+constexpr uint32_t FT_PAR = FT_SLOT + 2 * FT_SLOT_BYTES;  // b1, b2, w3 (fp32) [128 each], b3, y halves [2 slots][2][128]
+constexpr uint32_t FT_SMEM = FT_PAR + (3 * TH + 4) * 4 + 2 * 2 * TM * 4;
 static_assert(FT_SMEM <= 227 * 1024 && 2 * FT_SMEM > 228 * 1024,
               "the training pass's tiles fit one CTA's shared memory, and only one CTA an SM (512 TMEM columns)");
 // requested: more than the tiles use, so that every operand the contractions
 // address, read with either stride order, lies inside the CTA's allocation
 constexpr uint32_t FT_SMEM_REQ = 225 * 1024;
 static_assert(FT_SMEM <= FT_SMEM_REQ, "request covers the layout");
-constexpr uint32_t kColD2 = 320;
+constexpr int kFtThreads = 256 + 128;  // the epilogue's, and the issuing warp's group: registers move by groups of four warps
+constexpr uint32_t kFtColW2 = 256, kFtColW1 = 416;
+// dH1 = dH2 W2: A K-major, B (W2) MN-major
+constexpr uint32_t kIdescBT = kIdesc | (1u << 16);
 
-__global__ void __launch_bounds__(kBwThreads, 1) k_mlp_train_tc(
+__device__ __forceinline__ uint32_t relu2(uint32_t p) {  // of a pair of bf16 (NaN to 0, as fmaxf)
+  const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+  const __nv_bfloat162 m = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&p), z);
+  return *reinterpret_cast<const uint32_t*>(&m);
+}
+__device__ __forceinline__ uint32_t positive2(uint32_t p) {  // all ones in the halves that are above 0
+  const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+  return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&p), z);
+}
+// a + b of two fp32 values each, and a b + c, in one issue slot
+__device__ __forceinline__ float2 add2f(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\t"
+      "mov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 mul2f(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 z, x, y;\n\t"
+      "mov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2f(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, w, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 w, {%6, %7};\n\t"
+      "fma.rn.f32x2 z, x, y, w;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint32_t p) {
+  return make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u));
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+}
+__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
+  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(b)) : "memory");
+}
+
+__global__ void __launch_bounds__(kFtThreads, 1) k_mlp_train_tc(
     TcArgs w, const float* __restrict__ x, const float* __restrict__ tgt, int64_t R,
     const int32_t* __restrict__ R_dev, float* __restrict__ y_out, float* __restrict__ grads,
     double* __restrict__ loss, int32_t* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_mbar;
+  __shared__ __align__(8) uint64_t s_full[2], s_done[2], s_part[2][4];
+  __shared__ int s_fail;
   const int t = threadIdx.x, warp = t >> 5;
-  const int r = t & (TM - 1), hf = t >> 7, u0 = 64 * hf;
   float* par = reinterpret_cast<float*>(sm + FT_PAR);  // b1 | b2 | w3 | b3 | y halves
   float* s_yh = par + 3 * TH + 4;
-  for (int i = t; i < TH * (TH / 8); i += kBwThreads) {
+  for (int i = t; i < TH * (TH / 8); i += kFtThreads) {
     const int n = i % TH, k8 = (i / TH) * 8;
-    uint32_t q[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      q[e] = (uint32_t)w.w2[(k8 + 2 * e) * TH + n] | ((uint32_t)w.w2[(k8 + 2 * e + 1) * TH + n] << 16);
-    *reinterpret_cast<uint4*>(sm + FT_W2T + core_off(n, k8, SBO_K128)) = make_uint4(q[0], q[1], q[2], q[3]);
     *reinterpret_cast<uint4*>(sm + FT_W2 + core_off(n, k8, SBO_K128)) =
         *reinterpret_cast<const uint4*>(w.w2 + n * TH + k8);
   }
-  for (int i = t; i < TH * (TI / 8); i += kBwThreads) {
+  for (int i = t; i < TH * (TI / 8); i += kFtThreads) {
     const int n = i / (TI / 8), k8 = (i % (TI / 8)) * 8;
     *reinterpret_cast<uint4*>(sm + FT_W1 + core_off(n, k8, SBO_K16)) =
         *reinterpret_cast<const uint4*>(w.w1 + n * TI + k8);
   }
-  for (int i = t; i < TH; i += kBwThreads) {
+  for (int i = t; i < TH; i += kFtThreads) {
     par[i] = w.b1[i];
     par[TH + i] = w.b2[i];
     par[2 * TH + i] = __uint_as_float((uint32_t)w.w3[i] << 16);
   }
-  for (int r = t; r < TM; r += kBwThreads) {  // the constant columns: a one, then zeros (the bias gradients)
+  for (int i = t; i < 2 * TM; i += kFtThreads) {  // the constant columns: a one, then zeros (the bias gradients)
     const uint4 one = make_uint4(0x3F80u, 0u, 0u, 0u), zero = make_uint4(0u, 0u, 0u, 0u);
-    *reinterpret_cast<uint4*>(sm + FT_X + core_off(r, TI, SBO_X)) = one;
-    *reinterpret_cast<uint4*>(sm + FT_X + core_off(r, TI + 8, SBO_X)) = zero;
-    *reinterpret_cast<uint4*>(sm + FT_H1 + core_off(r, TH, SBO_H)) = one;
-    *reinterpret_cast<uint4*>(sm + FT_H1 + core_off(r, TH + 8, SBO_H)) = zero;
+    unsigned char* q = sm + FT_SLOT + (i / TM) * FT_SLOT_BYTES;
+    const int row = i % TM;
+    *reinterpret_cast<uint4*>(q + FT_X + core_off(row, TI, SBO_X)) = one;
+    *reinterpret_cast<uint4*>(q + FT_X + core_off(row, TI + 8, SBO_X)) = zero;
+    *reinterpret_cast<uint4*>(q + FT_H1 + core_off(row, TH, SBO_H)) = one;
+    *reinterpret_cast<uint4*>(q + FT_H1 + core_off(row, TH + 8, SBO_H)) = zero;
   }
   if (t == 0) {
     par[3 * TH] = w.b3[0];
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar)));
+    s_fail = 0;
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&s_full[s], 256);
+      mbar_init(&s_done[s], 1);
+      for (int k = 0; k < 4; ++k) mbar_init(&s_part[s][k], 64);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -647,230 +732,294 @@ __global__ void __launch_bounds__(kBwThreads, 1) k_mlp_train_tc(
   __syncthreads();
   fence_after();
   const uint32_t tmem = s_tmem;
-  const uint32_t mbar = smem_u32(&s_mbar);
   const uint32_t base = smem_u32(sm);
-  const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;  // TMEM lanes of this warp's rows
-  const int64_t Re = R_dev ? (*R_dev > 0 ? (*R_dev < R ? (int64_t)*R_dev : R) : 0) : R;
-  const float inv = Re > 0 ? 1.f / (float)Re : 0.f;
-  double lsum = 0.0;
-  float w3acc[64];
-#pragma unroll
-  for (int k = 0; k < 64; ++k) w3acc[k] = 0.f;
-  float b3 = 0.f;
-  uint32_t phase = 0;
-  bool failed = false, pending = false, any = false;
   const int64_t tiles = (R + TM - 1) / TM;
-  auto mma_wait = [&]() -> bool {  // every thread: the committed MMAs are complete
-    if (__syncthreads_or(!wait_parity(mbar, phase))) return false;
-    phase ^= 1u;
-    fence_after();
-    return true;
+  const int64_t stride = 2 * (int64_t)gridDim.x;
+  // a bounded wait; false once any thread's has run out
+  auto wait1 = [&](uint64_t* b, uint32_t& ph) -> bool {
+    if (!wait_parity(smem_u32(b), ph)) *(volatile int*)&s_fail = 1;
+    ph ^= 1u;
+    return *(volatile int*)&s_fail == 0;
   };
-  // the x row and target of the CTA's next tile, loaded while this one runs
-  float4 XR[TI / 4];
-  float tg = 0.f;
-  auto load_rows = [&](int64_t tl) {
-    const int64_t rw = tl * TM + r;
-    const bool in = tl < tiles && rw < R;
-#pragma unroll
-    for (int k4 = 0; k4 < TI / 4; ++k4)
-      XR[k4] = in && hf == 0 ? *reinterpret_cast<const float4*>(x + rw * TI + 4 * k4) : make_float4(0.f, 0.f, 0.f, 0.f);
-    tg = (tl < tiles && rw < Re) ? tgt[rw] : 0.f;
-  };
-  load_rows(blockIdx.x);
-  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int64_t row = tile * TM + r;
-    const bool valid = row < R, counted = row < Re;
-    const float tgv = tg;
-    if (hf == 0) {  // the row's 16 features in bf16: X A tile and X^T
-      float xv[TI];
-#pragma unroll
-      for (int k = 0; k < TI; k += 4) {
-        const float4 v = XR[k / 4];
-        xv[k] = v.x; xv[k + 1] = v.y; xv[k + 2] = v.z; xv[k + 3] = v.w;
-      }
-#pragma unroll
-      for (int k8 = 0; k8 < TI; k8 += 8) {
-        const uint32_t p[4] = {pack2(xv[k8], xv[k8 + 1]), pack2(xv[k8 + 2], xv[k8 + 3]),
-                               pack2(xv[k8 + 4], xv[k8 + 5]), pack2(xv[k8 + 6], xv[k8 + 7])};
-        *reinterpret_cast<uint4*>(sm + FT_X + core_off(r, k8, SBO_X)) = make_uint4(p[0], p[1], p[2], p[3]);
-      }
-    }
-    load_rows(tile + gridDim.x);  // in flight during this tile's contractions
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (t == 0) {  // layer 1: D1 = X W1^T
-      mma_bf16(tmem, sdesc(base + FT_X, 128, SBO_X), sdesc(base + FT_W1, 128, SBO_K16), 0u);
-      commit(mbar);
-    }
-    if (!mma_wait()) {
-      failed = pending = true;
-      break;
-    }
-    // h1 = bf16(relu(D1 + b1)): the H1 A tile, [H1^T; 1; 0] and the mask h1 > 0
-    uint64_t m1 = 0;
+  auto wait = [&](uint64_t* b, uint32_t& ph) -> bool { return __all_sync(0xffffffffu, wait1(b, ph)); };  // whole warps
+  // launched with 168 registers a thread: the four warps of the issuing group
+  // give theirs up (128 x 40) for the epilogue's (256 x 232), 64512 in all
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    // the issuing thread: a tile's four steps, the slots in turn, in the order the epilogue threads take them
+    if (t == 256) {
+      uint32_t pf[2] = {0u, 0u};
+      uint32_t accu = 0u;  // the weight-gradient accumulators hold something
+      bool ok = true;
+      uint32_t done_n[2] = {0u, 0u};
+      for (int64_t tile0 = blockIdx.x; tile0 < tiles && ok; tile0 += stride) {
+        const int ns = tile0 + gridDim.x < tiles ? 2 : 1;
 #pragma unroll 1
-    for (int c0 = 0; c0 < 64; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + lane_addr + (uint32_t)(u0 + c0), v);
-      uint32_t pk[16];
-#pragma unroll
-      for (int k = 0; k < 32; k += 2)
-        pk[k / 2] = pack2(fmaxf(v[k] + par[u0 + c0 + k], 0.f), fmaxf(v[k + 1] + par[u0 + c0 + k + 1], 0.f));
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4*>(sm + FT_H1 + core_off(r, u0 + c0 + 8 * q, SBO_H)) =
-            make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        if (__uint_as_float(pk[k] << 16) > 0.f) m1 |= 1ull << (c0 + 2 * k);
-        if (__uint_as_float(pk[k] & 0xffff0000u) > 0.f) m1 |= 1ull << (c0 + 2 * k + 1);
-      }
-    }
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (t == 0) {  // layer 2: D2 = H1 W2^T
-#pragma unroll
-      for (int kk = 0; kk < TH / 16; ++kk)
-        mma_bf16(tmem + kColD2, sdesc(base + FT_H1 + kk * 256, 128, SBO_H),
-                 sdesc(base + FT_W2 + kk * 256, 128, SBO_K128), kk > 0 ? 1u : 0u);
-      commit(mbar);
-    }
-    if (!mma_wait()) {
-      failed = pending = true;
-      break;
-    }
-    // h2 = bf16(relu(D2 + b2)); y = W3 . h2 + b3 from the two halves
-    uint32_t h2p[32];
-    float acc = 0.f;
-#pragma unroll
-    for (int c0 = 0; c0 < 64; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + lane_addr + kColD2 + (uint32_t)(u0 + c0), v);
-#pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        const int c = u0 + c0 + k;
-        const uint32_t pk = pack2(fmaxf(v[k] + par[TH + c], 0.f), fmaxf(v[k + 1] + par[TH + c + 1], 0.f));
-        h2p[(c0 + k) / 2] = pk;
-        acc += __uint_as_float(pk << 16) * par[2 * TH + c] + __uint_as_float(pk & 0xffff0000u) * par[2 * TH + c + 1];
-      }
-    }
-    s_yh[hf * TM + r] = acc;
-    __syncthreads();
-    const float yv = s_yh[r] + s_yh[TM + r] + par[3 * TH];
-    if (y_out && valid && hf == 0) y_out[row] = yv;
-    const float e = counted ? yv - tgv : 0.f;
-    const float d = e * inv;
-    if (hf == 0) {
-      lsum += 0.5 * (double)e * (double)e * (double)inv;
-      b3 += d;
-    }
-    // dH2 = [h2 > 0] d w3 (bf16): its row tile, the A operand of dH1 and of dW2;
-    // dW3 partials d h2
-#pragma unroll
-    for (int q8 = 0; q8 < 8; ++q8) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = 8 * q8 + 2 * q, c = u0 + j;
-        const float lo = __uint_as_float(h2p[j / 2] << 16), hi = __uint_as_float(h2p[j / 2] & 0xffff0000u);
-        pk[q] = pack2(lo > 0.f ? d * par[2 * TH + c] : 0.f, hi > 0.f ? d * par[2 * TH + c + 1] : 0.f);
-        w3acc[j] += d * lo;
-        w3acc[j + 1] += d * hi;
-      }
-      *reinterpret_cast<uint4*>(sm + FT_DH2 + core_off(r, u0 + 8 * q8, SBO_K128)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    }
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (t == 0) {  // dH1 (before the mask) = dH2 W2
-#pragma unroll
-      for (int kk = 0; kk < TH / 16; ++kk)
-        mma_bf16(tmem, sdesc(base + FT_DH2 + kk * 256, 128, SBO_K128), sdesc(base + FT_W2T + kk * 256, 128, SBO_K128),
-                 kk > 0 ? 1u : 0u);
-      commit(mbar);
-    }
-    if (!mma_wait()) {
-      failed = pending = true;
-      break;
-    }
-    // dh1 = bf16([h1 > 0] D): the row tile of dW1's A
+        for (int step = 0; step < 4 && ok; ++step) {
 #pragma unroll 1
-    for (int c0 = 0; c0 < 64; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + lane_addr + (uint32_t)(u0 + c0), v);
-      uint32_t pk[16];
+          for (int s = 0; s < ns && ok; ++s) {
+            ok = s ? wait1(&s_full[1], pf[1]) : wait1(&s_full[0], pf[0]);
+            if (!ok) break;
+            fence_after();
+            const uint32_t qb = base + FT_SLOT + s * FT_SLOT_BYTES, d = tmem + s * TH;
+            if (step == 0) {  // layer 1: D = X W1^T
+              mma_bf16(d, sdesc(qb + FT_X, 128, SBO_X), sdesc(base + FT_W1, 128, SBO_K16), 0u);
+            } else if (step == 1) {  // layer 2: D = H1 W2^T
 #pragma unroll
-      for (int k = 0; k < 32; k += 2)
-        pk[k / 2] = pack2((m1 >> (c0 + k)) & 1ull ? v[k] : 0.f, (m1 >> (c0 + k + 1)) & 1ull ? v[k + 1] : 0.f);
+              for (int kk = 0; kk < TH / 16; ++kk)
+                mma_bf16(d, sdesc(qb + FT_H1 + kk * 256, 128, SBO_H), sdesc(base + FT_W2 + kk * 256, 128, SBO_K128),
+                         kk > 0 ? 1u : 0u);
+            } else if (step == 2) {  // dH1 before its mask, D = dH2 W2, and dW2 | db2
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4*>(sm + FT_DH1 + core_off(r, u0 + c0 + 8 * q, SBO_K128)) =
-            make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-    }
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (t == 0) {  // dW2 | db2 and dW1 | db1, accumulated over the CTA's tiles
+              for (int kk = 0; kk < TH / 16; ++kk)
+                mma_bf16_n(d, sdesc(qb + FT_DH + kk * 256, 128, SBO_K128),
+                           sdesc(base + FT_W2 + kk * 2 * SBO_K128, SBO_K128, 128), kIdescBT, kk > 0 ? 1u : 0u);
 #pragma unroll
-      for (int kk = 0; kk < TM / 16; ++kk) {
-        const uint32_t accu = (any || kk > 0) ? 1u : 0u;
-        // MN-major: LBO steps along K (the rows, 8 at a time), SBO along M / N (8 units)
-        mma_bf16_n(tmem + kColW2, sdesc(base + FT_DH2 + kk * 2 * SBO_K128, SBO_K128, 128),
-                   sdesc(base + FT_H1 + kk * 2 * SBO_H, SBO_H, 128), kIdescN2T, accu);
-        mma_bf16_n(tmem + kColW1, sdesc(base + FT_DH1 + kk * 2 * SBO_K128, SBO_K128, 128),
-                   sdesc(base + FT_X + kk * 2 * SBO_X, SBO_X, 128), kIdescN1T, accu);
-      }
-      commit(mbar);
-    }
-    any = true;
-    if (!mma_wait()) {
-      failed = pending = true;
-      break;
-    }
-  }
-  if (failed) {
-    if (t == 0 && status) atomicExch(status, 1);
-    if (pending) wait_parity(mbar, phase);
-  } else if (any) {
-    if (t < TM) {  // row t of the weight-gradient accumulators: hidden unit t
-#pragma unroll 1
-      for (int c0 = 0; c0 < (int)N2; c0 += 32) {
-        float v[32];
-        tmem_ld32(tmem + lane_addr + kColW2 + (uint32_t)c0, v);
+              for (int kk = 0; kk < TM / 16; ++kk)  // MN-major: LBO steps along K (8 rows), SBO along M / N
+                mma_bf16_n(tmem + kFtColW2, sdesc(qb + FT_DH + kk * 2 * SBO_K128, SBO_K128, 128),
+                           sdesc(qb + FT_H1 + kk * 2 * SBO_H, SBO_H, 128), kIdescN2T, kk > 0 ? 1u : accu & 1u);
+              accu |= 1u;
+            } else {  // dW1 | db1
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const int c = c0 + k;
-          if (c < TH) atomicAdd(grads + kOffW2 + t * TH + c, v[k]);
-          else if (c == TH) atomicAdd(grads + kOffB2 + t, v[k]);
+              for (int kk = 0; kk < TM / 16; ++kk)
+                mma_bf16_n(tmem + kFtColW1, sdesc(qb + FT_DH + kk * 2 * SBO_K128, SBO_K128, 128),
+                           sdesc(qb + FT_X + kk * 2 * SBO_X, SBO_X, 128), kIdescN1T, kk > 0 ? 1u : accu >> 1);
+              accu |= 2u;
+            }
+            commit(smem_u32(&s_done[s]));
+            ++done_n[s];
+          }
         }
       }
-      float v[32];
-      tmem_ld32(tmem + lane_addr + kColW1, v);
+      // every commit is observed before the CTA frees its TMEM (bounded)
 #pragma unroll
-      for (int k = 0; k < TI; ++k) atomicAdd(grads + kOffW1 + t * TI + k, v[k]);
-      atomicAdd(grads + kOffB1 + t, v[TI]);
+      for (int s = 0; s < 2; ++s)
+        if (done_n[s] > 0) wait_parity(smem_u32(&s_done[s]), (done_n[s] - 1u) & 1u);
+      fence_after();
     }
-    // dW3 and db3: the rows' partials summed over each warp, one atomic per warp and unit
+    __syncwarp();
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    const int r = t & (TM - 1), hf = t >> 7, u0 = 64 * hf;
+    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;  // TMEM lanes of this warp's rows
+    float2 w3acc[32];
 #pragma unroll
-    for (int k = 0; k < 64; ++k) {
-      const float sum = warp_sum(w3acc[k]);
-      if ((t & 31) == 0) atomicAdd(grads + kOffW3 + u0 + k, sum);
+    for (int k = 0; k < 32; ++k) w3acc[k] = make_float2(0.f, 0.f);
+    float b3 = 0.f, l_hi = 0.f, l_lo = 0.f;  // sum of e^2 as an unevaluated pair of floats
+    const int64_t Re = R_dev ? (*R_dev > 0 ? (*R_dev < R ? (int64_t)*R_dev : R) : 0) : R;
+    const float inv = Re > 0 ? 1.f / (float)Re : 0.f;
+    const float4* b1v = reinterpret_cast<const float4*>(par + u0);
+    const float4* b2v = reinterpret_cast<const float4*>(par + TH + u0);
+    const float4* w3v = reinterpret_cast<const float4*>(par + 2 * TH + u0);
+    uint32_t pd[2] = {0u, 0u}, pp[2] = {0u, 0u};
+    uint32_t xp[2][TI / 2];  // the next tile's x row in bf16, and its target
+    float tg[2];
+    auto load_row = [&](int64_t tl, float4 (&xr)[TI / 4], float& tv) {
+      const int64_t rw = tl * TM + r;
+      const bool in = tl < tiles && rw < R && hf == 0;
+#pragma unroll
+      for (int k4 = 0; k4 < TI / 4; ++k4)
+        xr[k4] = in ? *reinterpret_cast<const float4*>(x + rw * TI + 4 * k4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      tv = (tl < tiles && rw < Re) ? tgt[rw] : 0.f;
+    };
+    auto pack_row = [&](const float4 (&xr)[TI / 4], uint32_t (&p)[TI / 2]) {
+#pragma unroll
+      for (int k4 = 0; k4 < TI / 4; ++k4) {
+        p[2 * k4] = pack2(xr[k4].x, xr[k4].y);
+        p[2 * k4 + 1] = pack2(xr[k4].z, xr[k4].w);
+      }
+    };
+    // operands written and TMEM read: the issuer may go on with the slot
+    auto arrive = [&](int s) {
+      fence_async_smem();
+      fence_before();
+      mbar_arrive(&s_full[s]);
+    };
+    {
+      float4 xr[TI / 4];
+      load_row(blockIdx.x, xr, tg[0]);
+      pack_row(xr, xp[0]);
+      load_row(blockIdx.x + (int64_t)gridDim.x, xr, tg[1]);
+      pack_row(xr, xp[1]);
     }
-    b3 = warp_sum(b3);
-    if ((t & 31) == 0 && hf == 0) atomicAdd(grads + kOffB3, b3);
+    bool ok = true, used[2] = {false, false};
+    for (int64_t tile0 = blockIdx.x; tile0 < tiles && ok; tile0 += stride) {
+      const int ns = tile0 + gridDim.x < tiles ? 2 : 1;  // slots in use (the second is idle at the end of the rows)
+      float tgv[2];
+      // X rows
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if (s >= ns || !ok) continue;
+        if (used[s]) ok = wait(&s_done[s], pd[s]);  // the slot's last contraction, dW1, has read X and dH1
+        if (!ok) continue;
+        unsigned char* q = sm + FT_SLOT + s * FT_SLOT_BYTES;
+        tgv[s] = tg[s];
+        if (hf == 0) {
+#pragma unroll
+          for (int k8 = 0; k8 < TI / 8; ++k8)
+            *reinterpret_cast<uint4*>(q + FT_X + core_off(r, 8 * k8, SBO_X)) =
+                make_uint4(xp[s][4 * k8], xp[s][4 * k8 + 1], xp[s][4 * k8 + 2], xp[s][4 * k8 + 3]);
+        }
+        used[s] = true;
+        arrive(s);
+      }
+      // h1 = bf16(relu(D + b1))
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if (s >= ns || !ok) continue;
+        ok = wait(&s_done[s], pd[s]);
+        if (!ok) continue;
+        fence_after();
+        unsigned char* q = sm + FT_SLOT + s * FT_SLOT_BYTES;
+        float v[32];
+#pragma unroll
+        for (int k8 = 0; k8 < 8; ++k8) {
+          if (k8 % 4 == 0) tmem_ld32(tmem + s * TH + lane_addr + (uint32_t)(u0 + 8 * k8), v);
+          uint32_t pk[4];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float4 b = b1v[2 * k8 + k];
+            const float* z = v + 8 * (k8 % 4) + 4 * k;
+            const float2 z0 = add2f(make_float2(z[0], z[1]), make_float2(b.x, b.y));
+            const float2 z1 = add2f(make_float2(z[2], z[3]), make_float2(b.z, b.w));
+            pk[2 * k] = relu2(pack2(z0.x, z0.y));
+            pk[2 * k + 1] = relu2(pack2(z1.x, z1.y));
+          }
+          *reinterpret_cast<uint4*>(q + FT_H1 + core_off(r, u0 + 8 * k8, SBO_H)) =
+              make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+        arrive(s);
+      }
+      // h2, y and dH2 = [h2 > 0] d w3
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if (s >= ns || !ok) continue;
+        ok = wait(&s_done[s], pd[s]);
+        if (!ok) continue;
+        fence_after();
+        unsigned char* q = sm + FT_SLOT + s * FT_SLOT_BYTES;
+        float* yh = s_yh + s * 2 * TM;
+        const int64_t row = (tile0 + s * (int64_t)gridDim.x) * TM + r;
+        const bool valid = row < R, counted = row < Re;
+        uint32_t h2p[32];
+        float2 acc = make_float2(0.f, 0.f);
+        {
+          float v[32];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            if (k % 8 == 0) tmem_ld32(tmem + s * TH + lane_addr + (uint32_t)(u0 + 4 * k), v);
+            const float4 b = b2v[k], w4 = w3v[k];
+            const float* z = v + 4 * (k % 8);
+            const float2 z0 = add2f(make_float2(z[0], z[1]), make_float2(b.x, b.y));
+            const float2 z1 = add2f(make_float2(z[2], z[3]), make_float2(b.z, b.w));
+            h2p[2 * k] = relu2(pack2(z0.x, z0.y));
+            h2p[2 * k + 1] = relu2(pack2(z1.x, z1.y));
+            acc = fma2f(unpack2(h2p[2 * k]), make_float2(w4.x, w4.y), acc);
+            acc = fma2f(unpack2(h2p[2 * k + 1]), make_float2(w4.z, w4.w), acc);
+          }
+        }
+        yh[hf * TM + r] = acc.x + acc.y;
+        mbar_arrive(&s_part[s][warp & 3]);
+        ok = wait(&s_part[s][warp & 3], pp[s]);
+        if (!ok) continue;
+        const float yv = yh[r] + yh[TM + r] + par[3 * TH];
+        if (y_out && valid && hf == 0) y_out[row] = yv;
+        const float e = counted ? yv - tgv[s] : 0.f;
+        const float d = e * inv;
+        if (hf == 0) {  // e^2 exactly as sq + rest, added to the pair
+          const float sq = __fmul_rn(e, e), rest = __fmaf_rn(e, e, -sq);
+          const float sum = __fadd_rn(l_hi, sq), bb = __fsub_rn(sum, l_hi);
+          l_lo += (l_hi - __fsub_rn(sum, bb)) + (sq - bb) + rest;
+          l_hi = sum;
+          b3 += d;
+        }
+        const float2 dd = make_float2(d, d);
+#pragma unroll
+        for (int k8 = 0; k8 < 8; ++k8) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float4 w4 = w3v[2 * k8 + k];
+            const int i = 4 * k8 + 2 * k;
+            const float2 g0 = mul2f(dd, make_float2(w4.x, w4.y)), g1 = mul2f(dd, make_float2(w4.z, w4.w));
+            pk[2 * k] = pack2(g0.x, g0.y) & positive2(h2p[i]);
+            pk[2 * k + 1] = pack2(g1.x, g1.y) & positive2(h2p[i + 1]);
+            w3acc[i] = fma2f(dd, unpack2(h2p[i]), w3acc[i]);
+            w3acc[i + 1] = fma2f(dd, unpack2(h2p[i + 1]), w3acc[i + 1]);
+          }
+          *reinterpret_cast<uint4*>(q + FT_DH + core_off(r, u0 + 8 * k8, SBO_K128)) =
+              make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+        arrive(s);
+      }
+      // dH1 = bf16([h1 > 0] D); the slot's next x row loads meanwhile
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if (s >= ns || !ok) continue;
+        float4 xr[TI / 4];
+        load_row(tile0 + s * (int64_t)gridDim.x + stride, xr, tg[s]);
+        ok = wait(&s_done[s], pd[s]);
+        if (!ok) continue;
+        fence_after();
+        unsigned char* q = sm + FT_SLOT + s * FT_SLOT_BYTES;
+        float v[32];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (k % 4 == 0) tmem_ld32(tmem + s * TH + lane_addr + (uint32_t)(u0 + 8 * k), v);
+          const uint4 h = *reinterpret_cast<const uint4*>(q + FT_H1 + core_off(r, u0 + 8 * k, SBO_H));
+          const float* z = v + 8 * (k % 4);
+          *reinterpret_cast<uint4*>(q + FT_DH + core_off(r, u0 + 8 * k, SBO_K128)) =
+              make_uint4(pack2(z[0], z[1]) & positive2(h.x), pack2(z[2], z[3]) & positive2(h.y),
+                         pack2(z[4], z[5]) & positive2(h.z), pack2(z[6], z[7]) & positive2(h.w));
+        }
+        arrive(s);
+        pack_row(xr, xp[s]);
+      }
+    }
+    // the slots' last contractions
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+      if (used[s] && ok) ok = wait(&s_done[s], pd[s]);
+    fence_after();
+    if (ok && used[0]) {
+      if (hf == 0) {  // row r of the weight-gradient accumulators: hidden unit r
+#pragma unroll 1
+        for (int c0 = 0; c0 < (int)N2; c0 += 16) {
+          float v[16];
+          tmem_ld16(tmem + lane_addr + kFtColW2 + (uint32_t)c0, v);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const int c = c0 + k;
+            if (c < TH) atomicAdd(grads + kOffW2 + r * TH + c, v[k]);
+            else if (c == TH) atomicAdd(grads + kOffB2 + r, v[k]);
+          }
+        }
+        float v[16];
+        tmem_ld16(tmem + lane_addr + kFtColW1, v);
+#pragma unroll
+        for (int k = 0; k < TI; ++k) atomicAdd(grads + kOffW1 + r * TI + k, v[k]);
+        tmem_ld16(tmem + lane_addr + kFtColW1 + TI, v);
+        atomicAdd(grads + kOffB1 + r, v[0]);
+      }
+      // dW3 and db3: the rows' partials summed over each warp, one atomic per warp and unit
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const float sx = warp_sum(w3acc[k].x), sy = warp_sum(w3acc[k].y);
+        if ((t & 31) == 0) {
+          atomicAdd(grads + kOffW3 + u0 + 2 * k, sx);
+          atomicAdd(grads + kOffW3 + u0 + 2 * k + 1, sy);
+        }
+      }
+      b3 = warp_sum(b3);
+      if ((t & 31) == 0 && hf == 0) atomicAdd(grads + kOffB3, b3);
+      const double lsum = warp_sum_d(((double)l_hi + (double)l_lo) * 0.5 * (double)inv);
+      if ((t & 31) == 0 && lsum != 0.0) atomicAdd(loss, lsum);
+    }
   }
-  lsum = warp_sum_d(lsum);
-  if ((t & 31) == 0 && lsum != 0.0) atomicAdd(loss, lsum);
   fence_before();
-  __syncthreads();
+  __syncthreads();  // every contraction has been seen complete (or a wait has run out)
   fence_after();
+  if (t == 0 && s_fail && status) atomicExch(status, 1);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kBwTmemCols));
 }
 }  // namespace
@@ -910,7 +1059,7 @@ tgs_status launch_mlp_train_tc(const tgs_mlp* w, const float* x, const float* ta
   }
   const int64_t tiles = (R + TM - 1) / TM;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, device_sm_count()));
-  k_mlp_train_tc<<<grid, kBwThreads, FT_SMEM_REQ, s>>>(TcArgs{w->w1, w->w2, w->w3, w->b1, w->b2, w->b3}, x, target, R,
+  k_mlp_train_tc<<<grid, kFtThreads, FT_SMEM_REQ, s>>>(TcArgs{w->w1, w->w2, w->w3, w->b1, w->b2, w->b3}, x, target, R,
                                                    R_dev, y, grads, loss, status);
   return check_launch();
 }

@@ -130,6 +130,40 @@ def test_train_pass_parity(P, orc, R, R_dev):
         assert rel_l2(g[sl[name]], gw[name].reshape(-1)) <= 2e-4, (name, rel_l2(g[sl[name]], gw[name].reshape(-1)))
 
 
+@pytest.mark.parametrize("tiles,extra,R_dev", [(1, 1, None), (2, 3, None), (3, 5, 200), (4, 0, None)])
+def test_train_pass_slots(P, orc, tiles, extra, R_dev):
+    """The training pass where each SM's thread block runs several 128-row tiles
+    through its two slots: a second tile for one block only (1), both slots
+    reused (2), the second slot idle in the last round (3, with counted rows
+    that end early, so that whole tiles hold none) and every slot full (4).
+    One tile dropped, doubled or taken from the other slot moves a gradient by
+    about 1 / tiles of its value (at least 1.6e-3), over the tolerances of
+    test_train_pass_parity, which hold at any number of rows."""
+    B, TileErrorMLP = P
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    R = sms * 128 * tiles + extra
+    mlp = TileErrorMLP(seed=tiles)
+    rng = np.random.default_rng(20 + tiles)
+    x = rng.normal(size=(R, 16)).astype(np.float32)
+    t = (2.0 + rng.normal(size=R)).astype(np.float32)      # a mean error, so that the gradients do not cancel
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    y = torch.full((R,), float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rd = None if R_dev is None else torch.tensor([R_dev], dtype=torch.int32, device="cuda")
+    B.mlp_train_tc(mlp.net(), xd, td, mlp.grads, mlp.loss, y=y, status=status, rows_dev=rd)
+    assert int(status.item()) == 0
+    Re = R if R_dev is None else R_dev
+    loss, gw = orc.mlp_backward(x[:Re], t[:Re], mlp.weights_fp(), bf16=True)
+    y_f = torch.empty(R, device="cuda")
+    B.mlp_forward_tc(mlp.net(), xd, y_f, status=status)
+    assert rel_l2(y.cpu().numpy(), y_f.cpu().numpy()) <= 1e-6
+    assert float(mlp.loss.item()) == pytest.approx(loss, rel=2e-5)
+    g = mlp.grads.double().cpu().numpy()
+    sl = mlp._slices()
+    for name in ("W1", "b1", "W2", "b2", "W3", "b3"):
+        assert rel_l2(g[sl[name]], gw[name].reshape(-1)) <= 2e-4, (name, rel_l2(g[sl[name]], gw[name].reshape(-1)))
+
+
 def test_adam_step_and_training(P):
     B, TileErrorMLP = P
     mlp = TileErrorMLP(seed=3, lr=2e-3)

@@ -276,62 +276,209 @@ __global__ void __launch_bounds__(kSelThreads) k_select_block(SelWs w, SelGeom g
   }
 }
 
-// Pixel sampling inside one chosen tile: one block of 256 threads (one per
-// local pixel); each phase is one exact block-wide k-selection.
-__global__ void __launch_bounds__(256) k_sample_pixels(const uint16_t* __restrict__ err,
-                                                       const uint16_t* __restrict__ age, SelGeom g, int n_pix,
-                                                       int hard_pm, int stable_pm, HashKeys hk,
-                                                       const int32_t* __restrict__ active_tiles,
-                                                       const int32_t* __restrict__ n_active,
-                                                       const int32_t* __restrict__ pix_off,
-                                                       uint8_t* __restrict__ pix_idx) {
-  __shared__ uint32_t s_cnt[8];
-  __shared__ RadixSelSmem sm;
-  __shared__ int64_t s64[32];
-  const int j = blockIdx.x;
-  if (j >= *n_active) return;
-  const int t = active_tiles[j];
-  const int l = threadIdx.x;
-  const int lane = l & 31;
-  const int x = (t % g.tx) * TGS_TILE + (l & 15), y = (t / g.tx) * TGS_TILE + (l >> 4);
-  const bool valid = x < g.W && y < g.H;
+// ---------------------------------------------------------------------------
+// Pixel sampling inside the chosen tiles: one warp per tile, lane l on the
+// local pixels l, l + 32, ..., l + 224 (two rows of the tile at a time), so
+// that every count is a ballot or a warp sum and nothing waits at a barrier.
+//
+// The error-proportional draw takes the kh smallest of L / w, in the exact
+// order of hard_key: L a logarithm by 32 squarings of 64-bit integers and a
+// quotient in FP64, about 500 instructions a pixel.  Which pixels those are is
+// nearly always clear from a few digits, so the warp first orders the pixels by
+// an approximate quotient in fp32 with a bound on its error, and takes the kh
+// smallest of these if the largest bound of the taken lies below the smallest
+// bound of the others (then the exact order takes the same); otherwise the
+// pixels between those two bounds, two as a rule, are ordered by their exact
+// keys.  With one block of 256 threads per tile, exact keys throughout and a
+// block-wide radix selection, the kernel was bound by its instructions (73 % of
+// the issue slots, 15000 warp instructions a tile; 2600 here): every tile of
+// 1280x720, 85 of 256 pixels: 66 -> 19 us; 1420 tiles 30 -> 12; eight views of
+// 1200 to 4500 tiles 436 -> 125.
+// ---------------------------------------------------------------------------
+constexpr int kPix = 256 / 32;  // pixels a lane
+
+// The k smallest (key, index) of the warp's eligible pixels, as a bit mask per
+// lane (bit j: pixel lane + 32 j).  The k-th smallest key is found one bit at
+// a time from the first bit in which the eligible keys differ; once the keys
+// that match the bits found are exactly those still wanted, the rest decides
+// nothing.  Ties at the last key go to the lower index.
+template <typename Key>
+__device__ __forceinline__ uint32_t warp_select(const Key (&key)[kPix], uint32_t elig, int k) {
+  const unsigned full = 0xffffffffu;
+  if (k <= 0) return 0u;
+  int play = __reduce_add_sync(full, __popc(elig));  // keys that match the bits found
+  if (k >= play) return elig;
+  // the bits in which they differ
+  Key any = 0, all = ~(Key)0;
+#pragma unroll
+  for (int j = 0; j < kPix; ++j)
+    if ((elig >> j) & 1u) {
+      any |= key[j];
+      all &= key[j];
+    }
+  Key diff;
+  if (sizeof(Key) == 8) {
+    const uint32_t lo = __reduce_or_sync(full, (uint32_t)any) ^ __reduce_and_sync(full, (uint32_t)all);
+    const uint32_t hi = __reduce_or_sync(full, (uint32_t)((uint64_t)any >> 32)) ^
+                        __reduce_and_sync(full, (uint32_t)((uint64_t)all >> 32));
+    diff = (Key)(((uint64_t)hi << 32) | lo);
+  } else {
+    diff = (Key)(__reduce_or_sync(full, (uint32_t)any) ^ __reduce_and_sync(full, (uint32_t)all));
+  }
+  uint32_t in = elig, below = 0u;  // pixels that match the bits found; pixels below them
+  int kk = k;
+  while (diff && kk < play) {
+    const int bit = sizeof(Key) == 8 ? 63 - __clzll((long long)diff) : 31 - __clz((int)diff);
+    uint32_t zero = 0u;
+#pragma unroll
+    for (int j = 0; j < kPix; ++j) zero |= (((key[j] >> bit) & 1u) ? 0u : 1u) << j;
+    zero &= in;
+    const int c = __reduce_add_sync(full, __popc(zero));
+    if (kk <= c) {
+      in = zero;
+      play = c;
+    } else {
+      below |= zero;
+      in &= ~zero;
+      kk -= c;
+      play -= c;
+    }
+    diff &= ~((Key)1 << bit);
+  }
+  if (kk < play) {  // equal keys: the first kk in index order
+    uint32_t t = 0u;
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+#pragma unroll
+    for (int j = 0; j < kPix; ++j) {
+      const uint32_t b = __ballot_sync(full, (in >> j) & 1u);
+      if (((in >> j) & 1u) && __popc(b & lt) < kk) t |= 1u << j;
+      kk = max(0, kk - __popc(b));
+    }
+    in = t;
+  }
+  return below | in;
+}
+
+// -log2 of the hash, in units of 1, to within kLogErr and 2^-24 of itself (the
+// difference's rounding): the top 24 bits of the mantissa (2^-22.5), the fast
+// logarithm of a value in [1, 2) (2^-21.4) and the truncations of neglog2_q32
+// (2^-31) are together below half of kLogErr.
+constexpr float kLogErr = 0x1p-19f;
+__device__ __forceinline__ float neglog2_approx(uint64_t h) {
+  const uint64_t u = h | 1ull;
+  const int lz = __clzll((long long)u);
+  return fmaxf((float)(lz + 1) - __log2f((float)(uint32_t)((u << lz) >> 40) * 0x1p-23f), 0.f);
+}
+
+constexpr int kSampleWarps = 4;  // tiles per block
+
+__global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(
+    const uint16_t* __restrict__ err, const uint16_t* __restrict__ age, SelGeom g, int n_pix, int hard_pm,
+    int stable_pm, HashKeys hk, const int32_t* __restrict__ active_tiles, const int32_t* __restrict__ n_active,
+    const int32_t* __restrict__ pix_off, uint8_t* __restrict__ pix_idx) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int j0 = blockIdx.x * kSampleWarps + (threadIdx.x >> 5);
+  if (j0 >= *n_active) return;
+  const int t = active_tiles[j0];
+  const int x = (t % g.tx) * TGS_TILE + (lane & 15), y = (t / g.tx) * TGS_TILE + (lane >> 4);  // pixel j: row y + 2 j
+  uint32_t valid = 0u;
+#pragma unroll
+  for (int j = 0; j < kPix; ++j)
+    if (x < g.W && y + 2 * j < g.H) valid |= 1u << j;
   const int nv = tile_valid(g, t);
   const int n = min(n_pix, nv);
   int kh, ks;
   split_counts(n, hard_pm, stable_pm, kh, ks);
-  bool taken;
-  if (n >= nv) {
-    taken = valid;  // every valid pixel
-  } else {
-    uint64_t kh_key = 0, ku_key = 0;
-    uint32_t av = 0;
-    if (valid) {
-      const size_t k = (size_t)y * g.W + x;
-      av = age[k];
-      kh_key = hard_key(err_weight(err[k]),
-                        neglog2_q32(hash_item(hk.prefix(STREAM_PIX_HARD), (uint32_t)t, (uint32_t)l)));
-      ku_key = hash_item(hk.prefix(STREAM_PIX_UNIF), (uint32_t)t, (uint32_t)l) >> 32;
+  uint32_t taken = valid;  // n >= nv: every valid pixel
+  if (n < nv) {
+    const size_t p0 = (size_t)y * g.W + x;
+    uint16_t ev[kPix], av[kPix];
+#pragma unroll
+    for (int j = 0; j < kPix; ++j) {
+      const bool in = (valid >> j) & 1u;
+      ev[j] = in && kh > 0 ? err[p0 + (size_t)(2 * j) * g.W] : (uint16_t)0;
+      av[j] = in && ks > 0 ? age[p0 + (size_t)(2 * j) * g.W] : (uint16_t)0;
     }
-    // phase 0: error-proportional draw; 1: oldest of the rest; 2: uniform of the rest
-    uint64_t key[1] = {kh_key};
-    bool el[1] = {valid}, th[1], ts[1], tu[1];
-    block_radix_select<1>(key, el, kh, 64, th, sm, s64, 0);
-    key[0] = 0xFFFFull - av;
-    el[0] = valid && !th[0];
-    block_radix_select<1>(key, el, ks, 16, ts, sm, s64, 1);
-    key[0] = ku_key;
-    el[0] = valid && !th[0] && !ts[0];
-    block_radix_select<1>(key, el, n - kh - ks, 32, tu, sm, s64, 2);
-    taken = th[0] || ts[0] || tu[0];
+    uint32_t th = 0u;
+    if (kh > 0) {
+      const uint64_t pre = hk.prefix(STREAM_PIX_HARD);
+      uint32_t key[kPix];
+      float d[kPix];
+#pragma unroll
+      for (int j = 0; j < kPix; ++j) {
+        const float l = neglog2_approx(hash_item(pre, (uint32_t)t, (uint32_t)(lane + 32 * j)));
+        // weight 0 comes after every positive weight, whose quotients are at most 65
+        const float w = (float)err_weight(ev[j]);
+        const float rw = w > 0.f ? __fdividef(1.f, w) : 0x1p60f;
+        key[j] = __float_as_uint(l * rw);  // l >= 0: ordered like its bits
+        d[j] = kLogErr * rw;
+      }
+      th = warp_select<uint32_t>(key, valid, kh);
+      // taken and not taken, apart by their bounds (2^-19 of the quotient covers the roundings of the weight, the division and L)
+      float top = 0.f, low = 0x1p126f;
+#pragma unroll
+      for (int j = 0; j < kPix; ++j) {
+        const float a = __uint_as_float(key[j]);
+        if ((th >> j) & 1u) top = fmaxf(top, a + (a * 0x1p-19f + d[j]));
+        else if ((valid >> j) & 1u) low = fminf(low, a - (a * 0x1p-19f + d[j]));
+      }
+      const float t_top = __uint_as_float(__reduce_max_sync(full, __float_as_uint(top)));
+      const float t_low = __uint_as_float(__reduce_min_sync(full, __float_as_uint(fmaxf(low, 0.f))));
+      if (t_top >= t_low) {
+        // in doubt: the taken whose bound reaches the lowest of the others, and the others that reach the highest of
+        // the taken; the rest is as the approximate order has it
+        uint32_t doubt = 0u;
+#pragma unroll
+        for (int j = 0; j < kPix; ++j) {
+          const float a = __uint_as_float(key[j]), e = a * 0x1p-19f + d[j];
+          if ((th >> j) & 1u ? a + e >= t_low : ((valid >> j) & 1u) && a - e <= t_top) doubt |= 1u << j;
+        }
+        const int kk = __reduce_add_sync(full, __popc(doubt & th));
+        uint64_t exact[kPix];
+#pragma unroll
+        for (int q = 0; q < kPix; ++q) exact[q] = 0;
+#pragma unroll 1
+        for (uint32_t rem = doubt; __any_sync(full, rem); rem &= rem - 1u) {  // each lane's next one
+          const int j = __ffs(rem) - 1;
+          uint16_t e = 0;
+#pragma unroll
+          for (int q = 0; q < kPix; ++q) e = j == q ? ev[q] : e;
+          const uint64_t v =
+              hard_key(err_weight(e), neglog2_q32(hash_item(pre, (uint32_t)t, (uint32_t)(lane + 32 * j))));
+#pragma unroll
+          for (int q = 0; q < kPix; ++q) exact[q] = j == q ? v : exact[q];
+        }
+        th = (th & ~doubt) | warp_select<uint64_t>(exact, doubt, kk);
+      }
+    }
+    // the oldest of the rest, then the uniform draw of the rest
+    uint32_t ts = 0u, tu = 0u;
+    if (ks > 0) {
+      uint32_t key[kPix];
+#pragma unroll
+      for (int j = 0; j < kPix; ++j) key[j] = 0xFFFFu - av[j];
+      ts = warp_select<uint32_t>(key, valid & ~th, ks);
+    }
+    if (n - kh - ks > 0) {
+      const uint64_t pre = hk.prefix(STREAM_PIX_UNIF);
+      uint32_t key[kPix];
+#pragma unroll
+      for (int j = 0; j < kPix; ++j)
+        key[j] = (uint32_t)(hash_item(pre, (uint32_t)t, (uint32_t)(lane + 32 * j)) >> 32);
+      tu = warp_select<uint32_t>(key, valid & ~th & ~ts, n - kh - ks);
+    }
+    taken = th | ts | tu;
   }
-  // ascending compaction of the taken local indices
-  const unsigned b = __ballot_sync(0xffffffffu, taken);
-  if (lane == 0) s_cnt[l >> 5] = __popc(b);
-  __syncthreads();
-  int off = 0;
-  for (int k = 0; k < (l >> 5); ++k) off += s_cnt[k];
-  off += __popc(b & ((1u << lane) - 1u));
-  if (taken) pix_idx[pix_off[j] + off] = (uint8_t)l;
+  // the taken local indices, ascending
+  uint8_t* out = pix_idx + pix_off[j0];
+  const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int j = 0; j < kPix; ++j) {
+    const uint32_t b = __ballot_sync(full, (taken >> j) & 1u);
+    if ((taken >> j) & 1u) out[__popc(b & lt)] = (uint8_t)(lane + 32 * j);
+    out += __popc(b);
+  }
 }
 
 __global__ void k_sel_finish(const int64_t* __restrict__ total, int32_t* __restrict__ n_active,
@@ -411,8 +558,9 @@ static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map
     k_sel_finish<<<1, 1, 0, s>>>(w.total, n_active, pix_off);
   }
   if (n_sel > 0)
-    k_sample_pixels<<<n_sel, 256, 0, s>>>(err_map, age_map, g, n_pix, cfg->pix_hard_pm, cfg->pix_stable_pm, hk,
-                                          active_tiles, n_active, pix_off, pix_idx);
+    k_sample_pixels<<<(n_sel + kSampleWarps - 1) / kSampleWarps, 32 * kSampleWarps, 0, s>>>(
+        err_map, age_map, g, n_pix, cfg->pix_hard_pm, cfg->pix_stable_pm, hk, active_tiles, n_active, pix_off,
+        pix_idx);
   return check_launch();
 }
 

@@ -5,27 +5,6 @@
 
 namespace tgs {
 
-// Exact block-wide k-selection by radix select: the k smallest (key, index)
-// pairs among the eligible items of the block, keys < 2^nbits, items held
-// ITEMS per thread in index order (thread t holds t * ITEMS + j).  The k-th
-// smallest key K is found one 8-bit digit at a time from the top: a pass
-// first takes the block-wide minimum and maximum of the digit over the keys
-// that match the digits found so far (one digit: nothing to count), else
-// counts them in a shared histogram, and every warp then locates the digit
-// where the running count reaches k by itself (no second barrier).  Once the
-// chosen bin holds exactly the keys still wanted, those are taken and the
-// lower digits are never looked at; otherwise every key below K is taken, and
-// the ties at K in index order until k are reached.  Every thread of the
-// block must call it (it synchronises); k is the same on all threads.
-// Buffers that a pass writes before a barrier and reads after it alternate
-// between two copies, so that the next pass never overwrites what a slower
-// warp still reads.
-struct RadixSelSmem {
-  uint32_t hist[2][256];
-  uint32_t wmin[2][32], wmax[2][32];
-  int32_t wcnt[2][32];
-};
-
 // Exclusive prefix over threads of v (thread order); total receives the sum.
 __device__ __forceinline__ int64_t block_excl_sum(int64_t v, int64_t* s64, int64_t& total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -49,133 +28,158 @@ __device__ __forceinline__ int64_t block_excl_sum(int64_t v, int64_t* s64, int64
   return (w > 0 ? upto : 0) + x - v;
 }
 
-// call: 0, 1, 2 ... for consecutive selections of one kernel (buffer parity).
-template <int ITEMS>
-__device__ void block_radix_select(const uint64_t (&key)[ITEMS], const bool (&elig)[ITEMS], int k, int nbits,
-                                   bool (&taken)[ITEMS], RadixSelSmem& sm, int64_t* s64, int call) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+constexpr int kSelThreads = 1024;  // threads of a selecting block, and buckets of a pass
+constexpr int kSelCand = 64;       // keys of the last bucket that are ordered by counting
+
+struct SelectSmem {
+  uint32_t hist[kSelThreads];
+  uint32_t lo[32], hi[32];
+  int32_t cnt[32];
+  uint32_t wsum[32];
+  uint64_t ckey[kSelCand];
+  int32_t cidx[kSelCand];
+  int32_t n_cand;
+};
+
+__device__ __forceinline__ uint32_t warp_incl_sum(uint32_t v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) taken[j] = false;
-  if (k <= 0) return;
-  int mine = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) mine += elig[j];
-  mine = __reduce_add_sync(0xffffffffu, mine);
-  if (lane == 0) sm.wcnt[call & 1][w] = mine;
-  __syncthreads();
-  const int n_elig = __reduce_add_sync(0xffffffffu, lane < nw ? sm.wcnt[call & 1][lane] : 0);
-  if (k >= n_elig) {
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) taken[j] = elig[j];
-    return;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
   }
-  uint64_t prefix = 0, mask = 0;
-  int kk = k;  // rank (from 1) of the sought key among the keys matching the prefix
-  int hp = 0;  // histogram passes so far (buffer parity)
-  for (int shift = ((nbits + 7) / 8) * 8 - 8; shift >= 0; shift -= 8) {
-    const int par = (shift >> 3) & 1;
-    uint32_t dmin = 255u, dmax = 0u;
+  return v;
+}
+
+// Exact block-wide k-selection: of the items in elig (bit j: item t * ITEMS + j
+// of thread t, 1024 threads), the k smallest by (full key, index), as the same
+// kind of mask.  key[j] is the leading 32 bits of the full key, full(j) all of
+// it (MORE: it has 32 more bits; else the same value).
+// A pass spreads the keys in play over up to 1024 buckets of equal key width (a
+// power of two) between their smallest and largest, one shared-memory count
+// each, and finds the bucket that holds the k-th smallest: the keys below it
+// are taken, those above are not.  Its own keys are all taken when that many
+// are wanted, ordered by counting when there are few (a dozen of some thousand
+// well spread keys after the first pass), taken by their low words or in index
+// order when they are equal, and else spread again.  Every thread of the block
+// must call it (it synchronises); k is the same on all threads.
+// Bound by the instructions of one SM and by its chain of barriers and warp
+// sums, five barriers for a selection of one pass; a radix selection of 64-bit
+// keys by 8-bit digits took two a digit.  The tile selection (three selections
+// and the compaction), 256 tiles: 16 -> 7 us; 4056: 19 -> 12; 8160
+// tiles: 38 -> 25.
+template <int ITEMS, bool MORE, class Full>
+__device__ __forceinline__ uint32_t block_select(const uint32_t (&key)[ITEMS], const Full& full_key, uint32_t elig,
+                                                 int k, SelectSmem& sm, int64_t* s64) {
+  const unsigned full = 0xffffffffu;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  if (k <= 0) return 0u;
+  uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j)
-      if (elig[j] && (key[j] & mask) == prefix) {
-        const uint32_t d = (uint32_t)((key[j] >> shift) & 255u);
-        dmin = min(dmin, d);
-        dmax = max(dmax, d);
-      }
-    dmin = __reduce_min_sync(0xffffffffu, dmin);
-    dmax = __reduce_max_sync(0xffffffffu, dmax);
-    if (lane == 0) {
-      sm.wmin[par][w] = dmin;
-      sm.wmax[par][w] = dmax;
+  for (int j = 0; j < ITEMS; ++j)
+    if ((elig >> j) & 1u) {
+      lo = min(lo, key[j]);
+      hi = max(hi, key[j]);
     }
-    uint32_t* h = sm.hist[hp & 1];
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) h[b] = 0;
-    __syncthreads();
-    const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < nw ? sm.wmin[par][lane] : 255u);
-    const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < nw ? sm.wmax[par][lane] : 0u);
-    if (lo == hi) {  // one digit: every key in play has it
-      prefix |= (uint64_t)lo << shift;
-      mask |= 255ull << shift;
-      continue;
-    }
-    const uint32_t span = hi - lo + 1u;
-    if (span <= 32u) {
-      // few distinct digits (exponent bits, small ages): counted per warp by
-      // ballots, lane q holding digit lo + q, then one atomic per warp and
-      // digit (shared atomics on a few hot bins would serialise)
-      uint32_t cnt = 0;
+  const int mine = __reduce_add_sync(full, __popc(elig));
+  lo = __reduce_min_sync(full, lo);
+  hi = __reduce_max_sync(full, hi);
+  __syncthreads();  // the selection before this one has been read
+  if (lane == 0) {
+    sm.lo[w] = lo;
+    sm.hi[w] = hi;
+    sm.cnt[w] = mine;
+  }
+  sm.hist[t] = 0;
+  if (t == 0) sm.n_cand = 0;
+  __syncthreads();
+  const int n_elig = __reduce_add_sync(full, sm.cnt[lane]);
+  if (k >= n_elig) return elig;
+  lo = __reduce_min_sync(full, sm.lo[lane]);
+  hi = __reduce_max_sync(full, sm.hi[lane]);
+  uint32_t in = elig, below = 0u;  // items in [lo, hi], and below lo
+  int kk = k;                      // rank (from 1) of the sought key among the items in play
+  for (;;) {
+    const int sh = max(0, 22 - __clz((int)((hi - lo) | 1u)));
+    const uint32_t nb = ((hi - lo) >> sh) + 1u;
+    if (nb <= 8u) {  // few buckets (equal ages): counted by ballots, a shared counter would serialise
+      uint32_t c = 0;
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t d = elig[j] && (key[j] & mask) == prefix ? (uint32_t)((key[j] >> shift) & 255u) - lo : 32u;
-        for (uint32_t q = 0; q < span; ++q) {
-          const uint32_t b = __ballot_sync(0xffffffffu, d == q);
-          if ((uint32_t)lane == q) cnt += __popc(b);
+        const uint32_t d = (in >> j) & 1u ? (key[j] - lo) >> sh : 8u;
+        for (uint32_t q = 0; q < nb; ++q) {
+          const uint32_t b = __ballot_sync(full, d == q);
+          if ((uint32_t)lane == q) c += __popc(b);
         }
       }
-      if (cnt) atomicAdd(&h[lo + lane], cnt);
+      if (c) atomicAdd(&sm.hist[lane], c);
     } else {
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j)
-        if (elig[j] && (key[j] & mask) == prefix) atomicAdd(&h[(key[j] >> shift) & 255u], 1u);
+        if ((in >> j) & 1u) atomicAdd(&sm.hist[(key[j] - lo) >> sh], 1u);
     }
     __syncthreads();
-    ++hp;
-    // every warp: the digit where the running count reaches kk
-    uint32_t c[8], sum = 0;
+    const uint32_t ws = __reduce_add_sync(full, sm.hist[t]);
+    if (lane == 0) sm.wsum[w] = ws;
+    __syncthreads();
+    // every warp: the 32 buckets, then the bucket, where the running count reaches kk
+    const uint32_t s1 = sm.wsum[lane], i1 = warp_incl_sum(s1);
+    const int at1 = __ffs(__ballot_sync(full, i1 >= (uint32_t)kk)) - 1;
+    const uint32_t base = __shfl_sync(full, i1 - s1, at1);
+    const uint32_t s2 = sm.hist[32 * at1 + lane], i2 = base + warp_incl_sum(s2);
+    const int at2 = __ffs(__ballot_sync(full, i2 >= (uint32_t)kk)) - 1;
+    const int count = (int)__shfl_sync(full, s2, at2);
+    kk -= (int)__shfl_sync(full, i2 - s2, at2);
+    lo += (uint32_t)(32 * at1 + at2) << sh;
+    const uint32_t width = (1u << sh) - 1u;
+    hi = hi - lo > width ? lo + width : hi;
+    uint32_t lt = 0u, gt = 0u;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      c[q] = h[lane * 8 + q];
-      sum += c[q];
+    for (int j = 0; j < ITEMS; ++j) {
+      lt |= (key[j] < lo ? 1u : 0u) << j;
+      gt |= (key[j] > hi ? 1u : 0u) << j;
     }
-    uint32_t incl = sum;
+    below |= in & lt;
+    in &= ~(lt | gt);
+    if (kk == count) return below | in;
+    if (count <= kSelCand) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const uint32_t excl = incl - sum;
-    const unsigned at = __ballot_sync(0xffffffffu, excl < (uint32_t)kk && (uint32_t)kk <= incl);
-    const int src = __ffs(at) - 1;  // exactly one lane: 1 <= kk <= keys in play
-    int digit = 0, below = 0, count = 0;
-    if (lane == src) {
-      uint32_t run = excl;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (run + c[q] >= (uint32_t)kk) {
-          digit = lane * 8 + q;
-          below = (int)run;
-          count = (int)c[q];
-          break;
+      for (int j = 0; j < ITEMS; ++j)
+        if ((in >> j) & 1u) {
+          const int p = atomicAdd(&sm.n_cand, 1);
+          sm.ckey[p] = full_key(j);
+          sm.cidx[p] = t * ITEMS + j;
         }
-        run += c[q];
+      __syncthreads();
+      for (uint32_t rem = in; rem; rem &= rem - 1u) {
+        const int j = __ffs(rem) - 1, i = t * ITEMS + j;
+        const uint64_t mk = full_key(j);
+        int r = 0;
+        for (int q = 0; q < count; ++q) r += sm.ckey[q] < mk || (sm.ckey[q] == mk && sm.cidx[q] < i);
+        if (r < kk) below |= 1u << j;
       }
+      return below;
     }
-    digit = __shfl_sync(0xffffffffu, digit, src);
-    below = __shfl_sync(0xffffffffu, below, src);
-    count = __shfl_sync(0xffffffffu, count, src);
-    prefix |= (uint64_t)digit << shift;
-    mask |= 255ull << shift;
-    kk -= below;
-    if (kk == count) {
-      // every key matching the prefix is taken, so the digits below decide
-      // nothing: the k smallest are the keys whose leading digits are at most
-      // the prefix
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) taken[j] = elig[j] && (key[j] & mask) <= prefix;
-      return;
-    }
+    if (sh == 0) break;  // equal leading words
+    __syncthreads();
+    sm.hist[t] = 0;
+    __syncthreads();
   }
-  // every key below K = prefix is taken; of the keys equal to K, the first kk
-  int ties = 0;
+  if constexpr (MORE) {
+    uint32_t low[ITEMS];
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) ties += elig[j] && key[j] == prefix;
-  int64_t all_ties;
-  int before = (int)block_excl_sum(ties, s64, all_ties);
+    for (int j = 0; j < ITEMS; ++j) low[j] = (uint32_t)full_key(j);
+    return below | block_select<ITEMS, false>(low, [&](int j) { return full_key(j); }, in, kk, sm, s64);
+  } else {
+    int64_t all_ties;
+    int before = (int)block_excl_sum(__popc(in), s64, all_ties);
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const bool tie = elig[j] && key[j] == prefix;
-    taken[j] = elig[j] && (key[j] < prefix || (tie && before < kk));
-    before += tie;
+    for (int j = 0; j < ITEMS; ++j)
+      if ((in >> j) & 1u) {
+        if (before < kk) below |= 1u << j;
+        ++before;
+      }
+    return below;
   }
 }
 

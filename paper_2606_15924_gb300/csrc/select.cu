@@ -202,74 +202,75 @@ __global__ void __launch_bounds__(256) k_rank_tiles(SelWs w, int T, int phase, i
 // Tile level in one block of 1024 threads (up to 1024 * ITEMS tiles): the
 // three phases, then the ascending compaction into active_tiles, tile_rank,
 // pix_off and n_active.
-constexpr int kSelThreads = 1024;
 constexpr int kSelBlockMaxTiles = kSelThreads * 16;
 
 template <int ITEMS>
-__global__ void __launch_bounds__(kSelThreads) k_select_block(SelWs w, SelGeom g, int n_sel, int kh, int ks,
+__global__ void __launch_bounds__(kSelThreads, 1) k_select_block(SelWs w, SelGeom g, int n_sel, int kh, int ks,
                                                               int n_pix, int32_t* __restrict__ active_tiles,
                                                               int32_t* __restrict__ n_active,
                                                               int32_t* __restrict__ tile_rank,
                                                               int32_t* __restrict__ pix_off) {
-  __shared__ RadixSelSmem sm;
+  __shared__ SelectSmem sm;
   __shared__ int64_t s64[32];
   const int T = g.T;
   const bool all = n_sel >= T;
-  uint64_t key[ITEMS];
-  bool valid[ITEMS], elig[ITEMS], th[ITEMS], ts[ITEMS], tu[ITEMS];
+  const int i0 = threadIdx.x * ITEMS;
+  const uint32_t valid = i0 < T ? (ITEMS < T - i0 ? (1u << ITEMS) - 1u : (1u << (T - i0)) - 1u) : 0u;
+  uint32_t taken = 0u;
+  if (all) {
+    taken = valid;
+  } else if (n_sel > 0) {
+    uint32_t key[ITEMS];
+    // the hard keys are read again where their low words are wanted
+    auto hard = [&](int j) -> uint64_t { return (valid >> j) & 1u ? w.tile_key[i0 + j] : 0ull; };
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const int i = threadIdx.x * ITEMS + j;
-    valid[j] = i < T;
-    elig[j] = valid[j];
-    key[j] = (valid[j] && !all && n_sel > 0) ? w.tile_key[i] : 0;
+    for (int j = 0; j < ITEMS; ++j) key[j] = (uint32_t)(hard(j) >> 32);
+    const uint32_t th = block_select<ITEMS, true>(key, hard, valid, kh, sm, s64);
+    auto same = [&](int j) -> uint64_t {
+      uint32_t v = key[0];
+#pragma unroll
+      for (int q = 1; q < ITEMS; ++q) v = j == q ? key[q] : v;
+      return v;
+    };
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) key[j] = (valid >> j) & 1u ? 0xFFFFu - min(w.tile_age[i0 + j], 0xFFFFu) : 0u;
+    const uint32_t ts = block_select<ITEMS, false>(key, same, valid & ~th, ks, sm, s64);
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) key[j] = (valid >> j) & 1u ? (uint32_t)(w.tile_u[i0 + j] >> 32) : 0u;
+    const uint32_t tu = block_select<ITEMS, false>(key, same, valid & ~th & ~ts, n_sel - kh - ks, sm, s64);
+    taken = th | ts | tu;
   }
-  if (all || n_sel <= 0) {
+  // compaction: (taken count << 32 | pixel count) prefix in tile order; the
+  // tile's place in the image follows from the thread's first by steps
+  const int x0 = i0 % g.tx, y0 = i0 / g.tx;
+  auto each = [&](auto f) {
+    int x = x0, y = y0;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      th[j] = all && valid[j];
-      ts[j] = tu[j] = false;
+      const int nv = min(TGS_TILE, g.W - x * TGS_TILE) * min(TGS_TILE, g.H - y * TGS_TILE);
+      f(j, (1ll << 32) | (int64_t)min(n_pix, nv));
+      if (++x == g.tx) {
+        x = 0;
+        ++y;
+      }
     }
-  } else {
-    block_radix_select<ITEMS>(key, elig, kh, 64, th, sm, s64, 0);
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const int i = threadIdx.x * ITEMS + j;
-      elig[j] = valid[j] && !th[j];
-      key[j] = valid[j] ? 0xFFFFull - min(w.tile_age[i], 0xFFFFu) : 0;
-    }
-    block_radix_select<ITEMS>(key, elig, ks, 16, ts, sm, s64, 1);
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const int i = threadIdx.x * ITEMS + j;
-      elig[j] = valid[j] && !th[j] && !ts[j];
-      key[j] = valid[j] ? (w.tile_u[i] >> 32) : 0;
-    }
-    block_radix_select<ITEMS>(key, elig, n_sel - kh - ks, 32, tu, sm, s64, 2);
-  }
-  // compaction: (taken count << 32 | pixel count) prefix in tile order
+  };
   int64_t mine = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const int i = threadIdx.x * ITEMS + j;
-    if (th[j] || ts[j] || tu[j]) mine += (1ll << 32) | (int64_t)min(n_pix, tile_valid(g, i));
-  }
+  each([&](int j, int64_t v) { mine += (taken >> j) & 1u ? v : 0; });
   int64_t total;
   int64_t pre = block_excl_sum(mine, s64, total);
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const int i = threadIdx.x * ITEMS + j;
-    if (!valid[j]) continue;
-    if (th[j] || ts[j] || tu[j]) {
+  each([&](int j, int64_t v) {
+    const int i = i0 + j;
+    if ((taken >> j) & 1u) {
       const int r = (int)(pre >> 32);
       tile_rank[i] = r;
       active_tiles[r] = i;
       pix_off[r] = (int)(pre & 0xFFFFFFFFll);
-      pre += (1ll << 32) | (int64_t)min(n_pix, tile_valid(g, i));
-    } else {
+      pre += v;
+    } else if ((valid >> j) & 1u) {
       tile_rank[i] = -1;
     }
-  }
+  });
   if (threadIdx.x == 0) {
     *n_active = (int32_t)(total >> 32);
     pix_off[total >> 32] = (int32_t)(total & 0xFFFFFFFFll);
@@ -510,7 +511,10 @@ static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map
         err_map, age_map, g, hk, w, aligned16(err_map) && aligned16(age_map) && width % 8 == 0);
   if (T <= kSelBlockMaxTiles) {
     // one block: the three phases and the compaction
-    if (T <= kSelThreads * 4)
+    if (T <= kSelThreads)
+      k_select_block<1><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
+                                                   pix_off);
+    else if (T <= kSelThreads * 4)
       k_select_block<4><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
                                                    pix_off);
     else if (T <= kSelThreads * 8)

@@ -12,7 +12,7 @@ namespace tgs {
 constexpr uint32_t kStreamView = 5;  // hash stream of the view draw
 constexpr int kSumThreads = 256;
 constexpr int kSumVec = 4;           // 16-byte loads in flight per thread
-constexpr int kViewThreads = 1024;
+constexpr int kViewThreads = kSelThreads;
 
 // E * 2^24 of an fp16 value h with sign-and-exponent field s = h >> 10 is
 // ((h & 1023) | imp[s]) * mul[s]: a normal value (1024 + m) 2^(e - 25) counts
@@ -146,12 +146,12 @@ __device__ __forceinline__ bool anchor_better(bool ea, uint64_t sa, int ia, bool
 }
 
 template <int ITEMS>
-__global__ void __launch_bounds__(kViewThreads) k_sample_views(const uint64_t* __restrict__ err_sums,
+__global__ void __launch_bounds__(kViewThreads, 1) k_sample_views(const uint64_t* __restrict__ err_sums,
                                                               const tgs_camera* __restrict__ cams, int V, int K,
                                                               double lambda_d, double lambda_theta, uint64_t prefix,
                                                               uint8_t* __restrict__ stack,
                                                               int32_t* __restrict__ views) {
-  __shared__ RadixSelSmem sm;
+  __shared__ SelectSmem sm;
   __shared__ int64_t s64[32];
   __shared__ int s_cnt[32];
   __shared__ uint64_t s_bs[32];
@@ -236,13 +236,13 @@ __global__ void __launch_bounds__(kViewThreads) k_sample_views(const uint64_t* _
   const int anchor = s_anchor;
   // 3. Efraimidis-Spirakis keys of the geometric weights (Eq. 6)
   uint64_t key[ITEMS];
-  bool elig[ITEMS], taken[ITEMS];
+  uint32_t elig = 0u, lead[ITEMS];
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
     const int v = threadIdx.x * ITEMS + j;
-    elig[j] = on[j] && v != anchor;
     key[j] = 0;
-    if (elig[j]) {
+    if (on[j] && v != anchor) {
+      elig |= 1u << j;
       double c[3], d[3];
       view_pose(cams[v], c, d);
       const double dx = __dsub_rn(c[0], s_pose[0]), dy = __dsub_rn(c[1], s_pose[1]), dz = __dsub_rn(c[2], s_pose[2]);
@@ -257,18 +257,26 @@ __global__ void __launch_bounds__(kViewThreads) k_sample_views(const uint64_t* _
       key[j] = ordered_bits(__dadd_rn(__dadd_rn(lg, __dmul_rn(s, 1.4426950408889634)), 0.0));
     }
   }
-  block_radix_select<ITEMS>(key, elig, K - 1, 64, taken, sm, s64, 0);
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) lead[j] = (uint32_t)(key[j] >> 32);
+  auto full = [&](int j) -> uint64_t {
+    uint64_t v = key[0];
+#pragma unroll
+    for (int q = 1; q < ITEMS; ++q) v = j == q ? key[q] : v;
+    return v;
+  };
+  const uint32_t taken = block_select<ITEMS, true>(lead, full, elig, K - 1, sm, s64);
   // 4. outputs: anchor first, then the draws ascending; the K views leave the stack
   int mine = 0;
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) mine += taken[j];
+  for (int j = 0; j < ITEMS; ++j) mine += (taken >> j) & 1u;
   int64_t total;
   int off = 1 + (int)block_excl_sum(mine, s64, total);
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
     const int v = threadIdx.x * ITEMS + j;
-    if (taken[j]) views[off++] = v;
-    if (v < V) stack[v] = (uint8_t)(on[j] && !taken[j] && v != anchor);
+    if ((taken >> j) & 1u) views[off++] = v;
+    if (v < V) stack[v] = (uint8_t)(on[j] && !((taken >> j) & 1u) && v != anchor);
   }
   if (threadIdx.x == 0) views[0] = anchor;
 }

@@ -288,6 +288,17 @@ tgs_status tgs_project_gaussians(const tgs_gaussians* g, const tgs_camera* cam, 
                                  tgs_projected* out, tgs_stream stream);
 
 /*
+ * project_gaussians_multi - project_gaussians for 1 to 16 views of one step in
+ * one pass over the Gaussians: view k uses cams[k] and tile_rank[k] (tile_rank,
+ * or an entry of it, may be null: every tile) and writes out[k], the same
+ * values as a project_gaussians call of that view.  The outputs of the views do
+ * not overlap.
+ */
+tgs_status tgs_project_gaussians_multi(const tgs_gaussians* g, int32_t n_views, const tgs_camera* cams,
+                                       const int32_t* const* tile_rank, const tgs_projected* out,
+                                       tgs_stream stream);
+
+/*
  * bin_tiles - per-tile Gaussian lists sorted by depth (Sec. 3.1, the ordered
  * sets K(p)): every (active tile, Gaussian) pair whose tile rectangle covers
  * the tile, ordered by (tile, depth, Gaussian id): a counting sort on the

@@ -6,7 +6,9 @@ loss of Eq. 11 is an expectation over them).  ``MultiViewTrainer`` keeps one
 tiles and pixels, projection, tile lists) and shares the Gaussians, their
 gradients and the optimiser moments.  One step:
 
-  per view: select_tiles -> project_gaussians -> bin_tiles
+  per view: select_tiles
+  all views: project_gaussians_multi (one pass over the Gaussians)
+  per view: bin_tiles
   all views: render_sampled_batched (one persistent launch, (view, tile) queue)
   per view: loss_sparse_ncc (view_weight 1/K)
   all views: render_backward_batched (one persistent launch)
@@ -168,6 +170,25 @@ class MultiViewTrainer:
                                write_untouched=False, accumulate=True,
                                view_row=self.rows[k] if self.use_rows else None, sh_degree=self.sh_degree)
 
+    def _select(self):
+        for v in self.views:
+            v._select()
+
+    def _project(self):
+        """Projection of all views: one pass over the Gaussians (persistent), or
+        one launch per view."""
+        if self.persistent:
+            B.project_gaussians_multi(self.params, [v.ccam for v in self.views], [v.tile_rank for v in self.views],
+                                      [v.proj for v in self.views], self.sh_degree)
+            return
+        for v in self.views:
+            B.project_gaussians(self.params, v.ccam, v.tile_rank, v.proj, self.sh_degree)
+
+    def _bin(self):
+        for v in self.views:
+            B.bin_tiles(v.proj, self.n, v.ccam, v.tile_rank, v.n_select, v.ws_bin, v.capacity, v.vals, None,
+                        v.ranges, v.n_isect)
+
     def _render_fwd(self):
         if self.persistent:
             B.render_sampled_batched(self.fwd_batch, self.grid[0], self.counters[0:1])
@@ -193,11 +214,9 @@ class MultiViewTrainer:
 
     # ------------------------------------------------------------------ step
     def forward(self):
-        for v in self.views:
-            v._select()
-            B.project_gaussians(self.params, v.ccam, v.tile_rank, v.proj, self.sh_degree)
-            B.bin_tiles(v.proj, self.n, v.ccam, v.tile_rank, v.n_select, v.ws_bin, v.capacity, v.vals, None,
-                        v.ranges, v.n_isect)
+        self._select()
+        self._project()
+        self._bin()
         self._render_fwd()
 
     def loss_and_maps(self):
@@ -249,26 +268,13 @@ class MultiViewTrainer:
 
     def stage_calls(self):
         """The step as (name, callable) pairs, each call over all views."""
-        def select():
-            for v in self.views:
-                v._select()
-
-        def project():
-            for v in self.views:
-                B.project_gaussians(self.params, v.ccam, v.tile_rank, v.proj, self.sh_degree)
-
-        def bins():
-            for v in self.views:
-                B.bin_tiles(v.proj, self.n, v.ccam, v.tile_rank, v.n_select, v.ws_bin, v.capacity, v.vals, None,
-                            v.ranges, v.n_isect)
-
         def upd():
             self.update()
             B.advance_counters(self.it_dev, self.step_dev)
         tail = ([("project_backward_update", lambda: (self.backward_update(),
                                                       B.advance_counters(self.it_dev, self.step_dev)))]
                 if self.fused else [("project_backward", self._project_bwd), ("hybrid_step", upd)])
-        return [("select_tiles", select), ("project_gaussians", project), ("bin_tiles", bins),
+        return [("select_tiles", self._select), ("project_gaussians", self._project), ("bin_tiles", self._bin),
                 ("render_sampled", self._render_fwd), ("loss_sparse_ncc", self.loss_and_maps),
                 ("render_backward", self._render_bwd)] + tail
 

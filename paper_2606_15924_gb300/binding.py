@@ -125,6 +125,8 @@ _lib.tgs_select_tiles_noalloc.argtypes = [_p, _p, _i32, _i32, _i32, _i32, _P(Sam
                                           _p, _p, _p, _p, _p, _p]
 _lib.tgs_project_gaussians.restype = _i32
 _lib.tgs_project_gaussians.argtypes = [_P(Gaussians), _P(Camera), _p, _P(Projected), _p]
+_lib.tgs_project_gaussians_multi.restype = _i32
+_lib.tgs_project_gaussians_multi.argtypes = [_P(Gaussians), _i32, _p, _p, _p, _p]
 _lib.tgs_bin_tiles_workspace_size.restype = _sz
 _lib.tgs_bin_tiles_workspace_size.argtypes = [_i64, _i64, _i32]
 _lib.tgs_bin_tiles.restype = _i32
@@ -217,7 +219,7 @@ _lib.tgs_mlp_adam.argtypes = [_p, _p, _p, _p, _i32, C.c_float, C.c_float, C.c_fl
 EXPORTED = ["tgs_version", "tgs_last_cuda_error", "tgs_status_string", "tgs_device_check", "tgs_graph_count_kernels",
             "tgs_advance_counters",
             "tgs_select_tiles_workspace_size", "tgs_select_tiles", "tgs_select_tiles_noalloc",
-            "tgs_project_gaussians",
+            "tgs_project_gaussians", "tgs_project_gaussians_multi",
             "tgs_bin_tiles_workspace_size", "tgs_bin_tiles", "tgs_checkpoint_bytes", "tgs_set_forward_split", "tgs_render_sampled",
             "tgs_loss_sparse_ncc", "tgs_loss_sparse_ssim",
             "tgs_backward_sampled", "tgs_render_backward_sampled", "tgs_render_backward_sampled_stats", "tgs_error_stats_sampled", "tgs_project_backward", "tgs_project_backward_multi_workspace_size",
@@ -369,6 +371,19 @@ def project_gaussians(g: dict, cam, tile_rank, out: dict, sh_degree=3, stream=No
     pr = projected(out)
     _check("tgs_project_gaussians", _lib.tgs_project_gaussians(C.byref(gs), C.byref(cc), _ptr(tile_rank),
                                                                C.byref(pr), _stream(stream)))
+
+
+def project_gaussians_multi(g: dict, cams: list, tile_ranks: list, outs: list, sh_degree=3, stream=None):
+    """project_gaussians for several views in one pass over the Gaussians."""
+    gs = gaussians(g, sh_degree)
+    K = len(cams)
+    if not K == len(tile_ranks) == len(outs):
+        raise ValueError("one tile_rank (or None) and one output per camera")
+    cs = (Camera * K)(*[c if isinstance(c, Camera) else camera(c) for c in cams])
+    ranks = (C.c_void_p * K)(*[_ptr(r) for r in tile_ranks])
+    prs = (Projected * K)(*[projected(o) for o in outs])
+    _check("tgs_project_gaussians_multi", _lib.tgs_project_gaussians_multi(C.byref(gs), K, cs, ranks, prs,
+                                                                           _stream(stream)))
 
 
 def bin_tiles_workspace_size(n: int, capacity: int, n_active_max: int) -> int:

@@ -5,8 +5,9 @@
 //      active tile in shared memory and reserve their runs in each tile's
 //      list with one atomic per tile they touch (a block x tile table of
 //      offsets),
-//   2. each block scans the tiles' totals (their starts) and scatters
-//      (depth bits << 32 | id) into its runs with shared-memory cursors,
+//   2. each block scans the tiles' totals (their starts; one launch before it
+//      where there are many pairs) and scatters (depth bits << 32 | id) into its
+//      runs with shared-memory cursors,
 //   3. one block per tile orders its list (k_tile_sort).
 // Positive float depths order like their bit patterns, so the result is the
 // order (tile, depth, Gaussian id).  With more active tiles than the shared
@@ -209,13 +210,57 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_count(const float2* __res
     if (sh[r]) row[r] = atomicAdd(rank_cnt + r, (int32_t)sh[r]);
 }
 
-// 2. shared-memory path: the block first takes the exclusive prefix of the
-// ranks' totals itself (R values, from L2), the ranks' starts, instead of a
-// scan launch of its own (block 0 writes them to rank_start and their sum to
-// n_total for what follows); then it scatters with shared cursors that start
-// at its runs (clamped to the capacity; positions at or past it are dropped).
-// Entries of ranks that the block has no pair in are not used as positions.
-template <bool SMEM_RANK>
+// 2'. shared-memory path, many pairs: the ranks' starts and the pairs' total,
+// once, and the keys' places overwritten with whole lines before the scatter.
+// The scatter writes 8 bytes here and there; a first write to a part of a
+// 32-byte sector that the L2 does not hold fetches the sector from memory, so
+// with the keys of the last call long evicted the scatter waited for a read of
+// the whole array: 6.7M pairs, 8487 tiles: 92 us, 49 where the lines are in the
+// L2.
+// Taken from kStartsPairs of capacity (48 MB of keys).  Scatter alone, and with
+// this launch before it: 720 tiles of 500k Gaussians 12 us, 14; 1340 tiles of 2M
+// 41, 45; every tile of 500k 26, 25; every tile of 1M at 1957x1091 109, 73; eight
+// views of 3M (4 to 15M pairs each) 1072, 881.
+constexpr int kStartThreads = 1024;
+constexpr int64_t kStartsPairs = 6ll << 20;
+
+__global__ void __launch_bounds__(kStartThreads) k_hist_starts(const int32_t* __restrict__ rank_cnt, int R,
+                                                               int64_t* __restrict__ rank_start,
+                                                               int64_t* __restrict__ n_total,
+                                                               uint64_t* __restrict__ keys, int64_t cap) {
+  __shared__ int64_t s_wt[32];
+  int64_t total;
+  if (blockIdx.x == 0) {
+    const int per = (R + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int r0 = min(R, (int)threadIdx.x * per), r1 = min(R, r0 + per);
+    int64_t run = 0;
+    for (int r = r0; r < r1; ++r) run += rank_cnt[r];
+    int64_t pre = block_exclusive_scan<int64_t>(run, s_wt, total);
+    for (int r = r0; r < r1; ++r) {
+      rank_start[r] = pre;
+      pre += rank_cnt[r];
+    }
+    if (threadIdx.x == 0) *n_total = total;
+  } else {
+    int64_t run = 0;
+    for (int r = threadIdx.x; r < R; r += blockDim.x) run += rank_cnt[r];
+    block_exclusive_scan<int64_t>(run, s_wt, total);
+  }
+  const int64_t m = min(total, cap);
+  uint4* k2 = reinterpret_cast<uint4*>(keys);
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < m / 2; p += (int64_t)gridDim.x * blockDim.x)
+    k2[p] = make_uint4(0u, 0u, 0u, 0u);
+  if ((m & 1) && blockIdx.x == 0 && threadIdx.x == 0) keys[m - 1] = 0;
+}
+
+// 2. shared-memory path: scatters with shared cursors that start at the block's
+// runs (clamped to the capacity; positions at or past it are dropped).  The
+// ranks' starts come from k_hist_starts (STARTS), or the block takes the
+// exclusive prefix of the ranks' totals itself (R values, from L2) instead of a
+// launch of its own (block 0 writes them to rank_start and their sum to n_total
+// for what follows).  Entries of ranks that the block has no pair in are not
+// used as positions.
+template <bool SMEM_RANK, bool STARTS>
 __global__ void __launch_bounds__(kHistThreads) k_hist_scatter(const float2* __restrict__ xy,
                                                                const int32_t* __restrict__ radius,
                                                                const float* __restrict__ depth, int64_t n,
@@ -229,20 +274,24 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_scatter(const float2* __r
   __shared__ int64_t s_wt[32];
   const int R = geo.n_ranks, b = blockIdx.x;
   const int32_t* row = table + (size_t)b * R;
-  // thread t scans the contiguous run [t * per, (t + 1) * per) of the totals
-  const int per = (R + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int r0 = (int)threadIdx.x * per, r1 = min(R, r0 + per);
-  int64_t run = 0;
-  for (int r = r0; r < r1; ++r) run += rank_cnt[r];
-  int64_t total;
-  int64_t pre = block_exclusive_scan<int64_t>(run, s_wt, total);
-  for (int r = r0; r < r1; ++r) {
-    const int64_t c = rank_cnt[r];
-    if (b == 0) rank_start[r] = pre;
-    sh[r] = (uint32_t)min(row[r] + pre, cap);
-    pre += c;
+  if (STARTS) {
+    for (int r = threadIdx.x; r < R; r += blockDim.x) sh[r] = (uint32_t)min(row[r] + rank_start[r], cap);
+  } else {
+    // thread t scans the contiguous run [t * per, (t + 1) * per) of the totals
+    const int per = (R + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int r0 = (int)threadIdx.x * per, r1 = min(R, r0 + per);
+    int64_t run = 0;
+    for (int r = r0; r < r1; ++r) run += rank_cnt[r];
+    int64_t total;
+    int64_t pre = block_exclusive_scan<int64_t>(run, s_wt, total);
+    for (int r = r0; r < r1; ++r) {
+      const int64_t c = rank_cnt[r];
+      if (b == 0) rank_start[r] = pre;
+      sh[r] = (uint32_t)min(row[r] + pre, cap);
+      pre += c;
+    }
+    if (b == 0 && threadIdx.x == 0) *n_total = total;
   }
-  if (b == 0 && threadIdx.x == 0) *n_total = total;
   const uint16_t* rank = SMEM_RANK ? stage_ranks(sh + R, tile_rank, geo) : nullptr;
   __syncthreads();
   int64_t i0, i1;
@@ -583,8 +632,9 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
       if (!attr_set[dev]) {
         cudaFuncSetAttribute(k_hist_count<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
         cudaFuncSetAttribute(k_hist_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
-        cudaFuncSetAttribute(k_hist_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
-        cudaFuncSetAttribute(k_hist_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
+        for (auto f : {k_hist_scatter<false, false>, k_hist_scatter<false, true>, k_hist_scatter<true, false>,
+                       k_hist_scatter<true, true>})
+          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
         attr_set[dev] = true;
       }
     }
@@ -604,12 +654,19 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
     cudaMemsetAsync(tile_ranges, 0, sizeof(int2) * (size_t)R, s);
     return check_launch();
   }
-  if (shared_path)
-    (smem_rank ? k_hist_scatter<true> : k_hist_scatter<false>)<<<G, kHistThreads, smem, s>>>(
-        xy, proj->radius, proj->depth, n, geo, tile_rank, w.table, w.tile_start, w.tile_cnt, n_isect, w.keys, capacity);
-  else
+  if (shared_path) {
+    const bool starts = capacity >= kStartsPairs;
+    if (starts)
+      k_hist_starts<<<2 * std::max(1, device_sm_count()), kStartThreads, 0, s>>>(w.tile_cnt, R, w.tile_start, n_isect,
+                                                                                 w.keys, capacity);
+    auto scatter = starts ? (smem_rank ? k_hist_scatter<true, true> : k_hist_scatter<false, true>)
+                          : (smem_rank ? k_hist_scatter<true, false> : k_hist_scatter<false, false>);
+    scatter<<<G, kHistThreads, smem, s>>>(xy, proj->radius, proj->depth, n, geo, tile_rank, w.table, w.tile_start,
+                                          w.tile_cnt, n_isect, w.keys, capacity);
+  } else {
     k_scatter_pairs<<<(int)((n + 255) / 256), 256, 0, s>>>(xy, proj->radius, proj->depth, n, geo, tile_rank,
                                                            w.tile_start, w.tile_fill, w.keys, capacity);
+  }
   if (keys) k_inv_rank<<<(T + 255) / 256, 256, 0, s>>>(tile_rank, T, w.inv_rank, R);
   // The sort's block by the lists' mean length (from the capacity, which the
   // caller sizes from the pairs of all tiles): lists past its CAP are sorted

@@ -1,0 +1,61 @@
+"""Binning at a capacity of many pairs, where a launch of its own takes the
+tiles' starts and clears the keys before the scatter, bit for bit against the
+same scene at the capacity it needs: an odd and an even number of pairs, one
+pair, none, tile masks and no mask, and more pairs than the capacity (the
+lists before the cut are whole, the count is of all)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2606_15924_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+MANY = 6 << 20
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2606_15924_gb300 import binding
+    binding.device_check()
+    return binding
+
+
+def _cam(W, H):
+    return dict(viewmat=np.eye(4), fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
+
+
+@pytest.mark.parametrize("n,W,H,share", [(1, 64, 48, None), (1, 64, 48, 0.0), (3000, 250, 187, 0.3), (3001, 250, 187, None),
+                                         (40000, 1957, 1091, 0.2), (40000, 1957, 1091, None)])
+def test_starts_launch_is_bit_exact(B, n, W, H, share):
+    from gpu_util import bin_dev, projected_dev
+    T = ((W + 15) // 16) * ((H + 15) // 16)
+    pd = projected_dev(scenes.projected(n, W, H, seed=n))
+    rank, R = None, T
+    if share is not None:
+        on = np.random.default_rng(n).random(T) < share
+        R = max(1, int(on.sum()))
+        rank = torch.from_numpy(np.where(on, np.cumsum(on) - 1, -1).astype(np.int32)).cuda()
+    few = bin_dev(B, pd, n, _cam(W, H), rank, R, capacity=2 * 10 ** 6)
+    I = int(few["n_isect"].item())
+    assert I < 2 * 10 ** 6 and (I > 0 or share == 0.0)
+    many = bin_dev(B, pd, n, _cam(W, H), rank, R, capacity=MANY)
+    for k in ("n_isect", "ranges"):
+        assert torch.equal(few[k], many[k]), k
+    for k in ("vals", "keys"):
+        assert torch.equal(few[k][:I], many[k][:I]), k
+
+
+def test_more_pairs_than_the_capacity(B):
+    from gpu_util import bin_dev, projected_dev
+    n, W, H, T = 1800, 1280, 720, 3600
+    pr = scenes.projected(n, W, H, seed=3)
+    pr["radius"] = np.full(n, 3000, np.int32)                # every tile
+    pd = projected_dev(pr)
+    out = bin_dev(B, pd, n, _cam(W, H), None, T, capacity=MANY)
+    assert int(out["n_isect"].item()) == n * T > MANY
+    ends = np.minimum(np.arange(T + 1) * n, MANY)
+    np.testing.assert_array_equal(out["ranges"].cpu().numpy(), np.stack([ends[:-1], ends[1:]], 1))
+    order = np.lexsort((np.arange(n), pr["depth"]))          # one list, the same in every tile
+    whole = MANY // n
+    got = out["vals"][:whole * n].view(whole, n).cpu().numpy()
+    np.testing.assert_array_equal(got, np.broadcast_to(order, (whole, n)))

@@ -64,6 +64,7 @@ struct BinGeom {
 
 // Rank of tile t, from the view's table in global memory (nullptr: the id).
 struct RankGlobal {
+  static constexpr bool kMasked = false;
   const int32_t* tile_rank;
   int n_ranks;
   __device__ __forceinline__ int operator()(int t) const {
@@ -75,10 +76,24 @@ struct RankGlobal {
 // lanes look up 32 tiles, which costs the L1 a tag lookup a line and shared
 // memory a few bank conflicts.
 struct RankShared {
+  static constexpr bool kMasked = false;
   const uint16_t* rank;
   __device__ __forceinline__ int operator()(int t) const {
     const uint32_t r = rank[t];
     return r == 0xFFFFu ? -1 : (int)r;
+  }
+};
+// The same with a bit per tile, set where it has a rank.
+struct RankMasked {
+  static constexpr bool kMasked = true;
+  const uint16_t* rank;
+  const uint32_t* bits;  // one word past the last tile's
+  __device__ __forceinline__ int operator()(int t) const {
+    const uint32_t r = rank[t];
+    return r == 0xFFFFu ? -1 : (int)r;
+  }
+  __device__ __forceinline__ uint32_t row(int t, int w) const {  // tiles t .. t + w - 1, w <= 32
+    return __funnelshift_r(bits[t >> 5], bits[(t >> 5) + 1], t & 31) & (0xffffffffu >> (32 - w));
   }
 };
 
@@ -91,7 +106,13 @@ struct RankShared {
 // With the ranks looked up in shared memory: count 14.5 -> 10.1 and scatter
 // 17.2 -> 12.2 us at 500k Gaussians and 720 tiles, 71 -> 27 and 163 -> 109 at 1M
 // and every tile of 1957x1091.
+// Where only some tiles are active (RankMasked) the lane first gathers the
+// active tiles of its rectangle as one word, a row of the bit table at a time,
+// and takes only those, count and scatter: 720 of 3600 tiles, 500k Gaussians
+// 10.1 -> 9.0 and 12.2 -> 10.1 us; 1340 of 6700, 2M 34.5 -> 24.7 and 41.0 -> 36.6;
+// eight views of 3M with 15 to 55 % of the tiles 494 -> 359 and 776 -> 677.
 constexpr int kLaneTiles = 16;
+constexpr int kLaneTilesMasked = 32;  // bits of a word
 
 template <bool DEPTH, typename Rank, typename F>
 __device__ __forceinline__ void for_each_pair(const float2* __restrict__ xy, const int32_t* __restrict__ radius,
@@ -112,17 +133,30 @@ __device__ __forceinline__ void for_each_pair(const float2* __restrict__ xy, con
       tile_span(p.y, r, geo.ty, y0, y1);
     }
     const int w = x1 - x0, area = w * (y1 - y0);
-    int t = y0 * geo.tx + x0, row_end = t + w;
-    for (int left = area <= kLaneTiles ? area : 0; left > 0; --left) {
-      const int k = rank_of(t);
-      if (k >= 0) f(k, id, d);
-      if (++t == row_end) {
-        t += geo.tx - w;
-        row_end = t + w;
+    constexpr int kLane = Rank::kMasked ? kLaneTilesMasked : kLaneTiles;
+    if constexpr (Rank::kMasked) {
+      const int t0 = y0 * geo.tx + x0;
+      uint32_t on = 0u;
+      if (area <= kLane)
+        for (int t = t0, b = 0; b < area; t += geo.tx, b += w) on |= rank_of.row(t, w) << b;
+      const uint32_t inv = w > 0 ? 65536u / (uint32_t)w + 1u : 0u;  // b / w = b inv >> 16 for b < 32
+      for (; on; on &= on - 1u) {
+        const int b = __ffs(on) - 1, y = (int)(((uint32_t)b * inv) >> 16);
+        f((int)rank_of.rank[t0 + b + y * (geo.tx - w)], id, d);
+      }
+    } else {
+      int t = y0 * geo.tx + x0, row_end = t + w;
+      for (int left = area <= kLane ? area : 0; left > 0; --left) {
+        const int k = rank_of(t);
+        if (k >= 0) f(k, id, d);
+        if (++t == row_end) {
+          t += geo.tx - w;
+          row_end = t + w;
+        }
       }
     }
     __syncwarp();
-    for (unsigned big = __ballot_sync(full, area > kLaneTiles); big; big &= big - 1) {
+    for (unsigned big = __ballot_sync(full, area > kLane); big; big &= big - 1) {
       const int src = __ffs(big) - 1;
       const int o_area = __shfl_sync(full, area, src), o_w = __shfl_sync(full, w, src);
       const int o_t = __shfl_sync(full, y0 * geo.tx + x0, src);
@@ -177,18 +211,47 @@ __device__ __forceinline__ void chunk_of(int64_t n, int64_t& i0, int64_t& i1) {
   i1 = min(n, i0 + chunk);
 }
 
-// The view's ranks as 16-bit values in shared memory (at p).
-__device__ __forceinline__ const uint16_t* stage_ranks(uint32_t* p, const int32_t* __restrict__ tile_rank,
-                                                       const BinGeom& geo) {
+// The view's ranks as 16-bit values in shared memory (at p), and behind them a
+// bit per tile (MASKED; whole blocks call it).
+enum { kRankGlobal = 0, kRankShared = 1, kRankMasked = 2 };
+__host__ __device__ inline size_t rank_smem(int kind, int tiles) {
+  const size_t words = ((size_t)tiles + 1) / 2;
+  return kind == kRankGlobal ? 0 : 4 * (words + (kind == kRankMasked ? (size_t)(tiles + 31) / 32 + 1 : 0));
+}
+template <bool MASKED>
+__device__ __forceinline__ RankMasked stage_ranks(uint32_t* p, const int32_t* __restrict__ tile_rank,
+                                                  const BinGeom& geo) {
   uint16_t* out = reinterpret_cast<uint16_t*>(p);
-  for (int t = threadIdx.x; t < geo.tx * geo.ty; t += blockDim.x) {
-    const int r = tile_rank[t];
-    out[t] = r >= 0 && r < geo.n_ranks ? (uint16_t)r : (uint16_t)0xFFFFu;
+  const int T = geo.tx * geo.ty;
+  uint32_t* bits = p + (T + 1) / 2;
+  for (int t0 = threadIdx.x & ~31; t0 < T; t0 += blockDim.x) {
+    const int t = t0 + (threadIdx.x & 31);
+    const int r = t < T ? tile_rank[t] : -1;
+    const bool in = r >= 0 && r < geo.n_ranks;
+    if (t < T) out[t] = in ? (uint16_t)r : (uint16_t)0xFFFFu;
+    if (MASKED) {
+      const uint32_t b = __ballot_sync(0xffffffffu, in);
+      if ((threadIdx.x & 31) == 0) bits[t0 >> 5] = b;
+    }
   }
-  return out;
+  if (MASKED && threadIdx.x == 0) bits[(T + 31) / 32] = 0u;
+  return RankMasked{out, bits};
 }
 
-template <bool SMEM_RANK>
+// Walks the block's chunk with ranks of the given kind (staged at p).
+template <int KIND, bool DEPTH, typename F>
+__device__ __forceinline__ void walk_chunk(const float2* __restrict__ xy, const int32_t* __restrict__ radius,
+                                           const float* __restrict__ depth, int64_t n, const BinGeom& geo,
+                                           const int32_t* __restrict__ tile_rank, const RankMasked& staged, F f) {
+  int64_t i0, i1;
+  chunk_of(n, i0, i1);
+  if constexpr (KIND == kRankMasked) for_each_pair<DEPTH>(xy, radius, depth, i0, i1, geo, staged, f);
+  else if constexpr (KIND == kRankShared)
+    for_each_pair<DEPTH>(xy, radius, depth, i0, i1, geo, RankShared{staged.rank}, f);
+  else for_each_pair<DEPTH>(xy, radius, depth, i0, i1, geo, RankGlobal{tile_rank, geo.n_ranks}, f);
+}
+
+template <int KIND>
 __global__ void __launch_bounds__(kHistThreads) k_hist_count(const float2* __restrict__ xy,
                                                              const int32_t* __restrict__ radius, int64_t n,
                                                              BinGeom geo, const int32_t* __restrict__ tile_rank,
@@ -197,13 +260,11 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_count(const float2* __res
   extern __shared__ uint32_t sh[];
   const int R = geo.n_ranks;
   for (int r = threadIdx.x; r < R; r += blockDim.x) sh[r] = 0;
-  const uint16_t* rank = SMEM_RANK ? stage_ranks(sh + R, tile_rank, geo) : nullptr;
+  RankMasked staged{};
+  if constexpr (KIND != kRankGlobal) staged = stage_ranks<KIND == kRankMasked>(sh + R, tile_rank, geo);
   __syncthreads();
-  int64_t i0, i1;
-  chunk_of(n, i0, i1);
-  auto count = [&](int k, uint32_t, uint32_t) { atomicAdd(sh + k, 1u); };
-  if (SMEM_RANK) for_each_pair<false>(xy, radius, nullptr, i0, i1, geo, RankShared{rank}, count);
-  else for_each_pair<false>(xy, radius, nullptr, i0, i1, geo, RankGlobal{tile_rank, R}, count);
+  walk_chunk<KIND, false>(xy, radius, nullptr, n, geo, tile_rank, staged,
+                          [&](int k, uint32_t, uint32_t) { atomicAdd(sh + k, 1u); });
   __syncthreads();
   int32_t* row = table + (size_t)blockIdx.x * R;
   for (int r = threadIdx.x; r < R; r += blockDim.x)
@@ -260,7 +321,7 @@ __global__ void __launch_bounds__(kStartThreads) k_hist_starts(const int32_t* __
 // launch of its own (block 0 writes them to rank_start and their sum to n_total
 // for what follows).  Entries of ranks that the block has no pair in are not
 // used as positions.
-template <bool SMEM_RANK, bool STARTS>
+template <int KIND, bool STARTS>
 __global__ void __launch_bounds__(kHistThreads) k_hist_scatter(const float2* __restrict__ xy,
                                                                const int32_t* __restrict__ radius,
                                                                const float* __restrict__ depth, int64_t n,
@@ -292,16 +353,13 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_scatter(const float2* __r
     }
     if (b == 0 && threadIdx.x == 0) *n_total = total;
   }
-  const uint16_t* rank = SMEM_RANK ? stage_ranks(sh + R, tile_rank, geo) : nullptr;
+  RankMasked staged{};
+  if constexpr (KIND != kRankGlobal) staged = stage_ranks<KIND == kRankMasked>(sh + R, tile_rank, geo);
   __syncthreads();
-  int64_t i0, i1;
-  chunk_of(n, i0, i1);
-  auto scatter = [&](int k, uint32_t i, uint32_t d) {
+  walk_chunk<KIND, true>(xy, radius, depth, n, geo, tile_rank, staged, [&](int k, uint32_t i, uint32_t d) {
     const uint32_t pos = atomicAdd(sh + k, 1u);
     if ((int64_t)pos < cap) keys[pos] = ((uint64_t)d << 32) | (uint64_t)i;
-  };
-  if (SMEM_RANK) for_each_pair<true>(xy, radius, depth, i0, i1, geo, RankShared{rank}, scatter);
-  else for_each_pair<true>(xy, radius, depth, i0, i1, geo, RankGlobal{tile_rank, R}, scatter);
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -618,10 +676,13 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
   // every pair's atomic on a few hundred addresses, several times slower.
   const bool shared_path = R <= kHistMaxRanks;
   const int G = hist_blocks(n);
-  // the view's rank table beside the counters, where both fit twice on an SM
-  const size_t both = sizeof(int32_t) * (size_t)R + sizeof(uint16_t) * (size_t)T;
-  const bool smem_rank = tile_rank && both <= 100 * 1024;  // R < 0xFFFF
-  const size_t smem = smem_rank ? both : sizeof(int32_t) * (size_t)R;
+  // the view's rank table beside the counters, where both fit twice on an SM;
+  // with a bit table where some tile is inactive (with every tile active its
+  // rows save nothing: 500k Gaussians 11.5 and 26.9 us without, 12.5 and 28.4)
+  const size_t counters = sizeof(int32_t) * (size_t)R;
+  int kind = tile_rank ? (R < T ? kRankMasked : kRankShared) : kRankGlobal;
+  if (counters + rank_smem(kind, T) > 100 * 1024) kind = kRankGlobal;  // R < 0xFFFF
+  const size_t smem = counters + rank_smem(kind, T);
   cudaMemsetAsync(w.tile_cnt, 0, sizeof(int32_t) * (size_t)R, s);
   if (shared_path) {
     if (smem > 48 * 1024) {  // opt in to more than 48 KB of dynamic shared memory (per device)
@@ -630,15 +691,16 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
       cudaGetDevice(&dev);
       if (dev < 0 || dev >= 64) return TGS_ERR_DEVICE;
       if (!attr_set[dev]) {
-        cudaFuncSetAttribute(k_hist_count<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
-        cudaFuncSetAttribute(k_hist_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
-        for (auto f : {k_hist_scatter<false, false>, k_hist_scatter<false, true>, k_hist_scatter<true, false>,
-                       k_hist_scatter<true, true>})
+        for (auto f : {k_hist_count<0>, k_hist_count<1>, k_hist_count<2>})
+          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
+        for (auto f : {k_hist_scatter<0, false>, k_hist_scatter<0, true>, k_hist_scatter<1, false>,
+                       k_hist_scatter<1, true>, k_hist_scatter<2, false>, k_hist_scatter<2, true>})
           cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistMaxRanks * 4);
         attr_set[dev] = true;
       }
     }
-    (smem_rank ? k_hist_count<true> : k_hist_count<false>)<<<G, kHistThreads, smem, s>>>(xy, proj->radius, n, geo, tile_rank, w.table, w.tile_cnt);
+    auto count = kind == kRankMasked ? k_hist_count<2> : kind == kRankShared ? k_hist_count<1> : k_hist_count<0>;
+    count<<<G, kHistThreads, smem, s>>>(xy, proj->radius, n, geo, tile_rank, w.table, w.tile_cnt);
   } else {
     cudaMemsetAsync(w.tile_fill, 0, sizeof(int32_t) * (size_t)R, s);
     k_count_pairs<<<(int)((n + 255) / 256), 256, 0, s>>>(xy, proj->radius, n, geo, tile_rank, w.tile_cnt);
@@ -659,8 +721,9 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
     if (starts)
       k_hist_starts<<<2 * std::max(1, device_sm_count()), kStartThreads, 0, s>>>(w.tile_cnt, R, w.tile_start, n_isect,
                                                                                  w.keys, capacity);
-    auto scatter = starts ? (smem_rank ? k_hist_scatter<true, true> : k_hist_scatter<false, true>)
-                          : (smem_rank ? k_hist_scatter<true, false> : k_hist_scatter<false, false>);
+    auto scatter = kind == kRankMasked   ? (starts ? k_hist_scatter<2, true> : k_hist_scatter<2, false>)
+                   : kind == kRankShared ? (starts ? k_hist_scatter<1, true> : k_hist_scatter<1, false>)
+                                         : (starts ? k_hist_scatter<0, true> : k_hist_scatter<0, false>);
     scatter<<<G, kHistThreads, smem, s>>>(xy, proj->radius, proj->depth, n, geo, tile_rank, w.table, w.tile_start,
                                           w.tile_cnt, n_isect, w.keys, capacity);
   } else {

@@ -1,31 +1,11 @@
 // Fused sparse supervision (Sec. 3.7, Eqs. 9-11; App. A): Charbonnier L1,
 // tile-level sparse NCC (or, for Table 4's S-SSIM variant, SSIM) with the
 // gradient-balanced weight, the per-pixel error
-// of Eq. 2 and the error/age map updates of Eqs. 3-4.  One thread block per
-// active tile, one thread per sampled pixel; tile moments are two-pass block
-// reductions.
+// of Eq. 2 and the error/age map updates of Eqs. 3-4.  One warp per active
+// tile; tile moments are two-pass warp reductions.
 #include "tgs_common.cuh"
 
 namespace tgs {
-
-// Block-wide sum of K floats per thread; every thread receives the totals.
-template <int K>
-__device__ __forceinline__ void block_sum(float (&v)[K], float (*sm)[K]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < K; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < K; ++k) sm[w][k] = v[k];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    float s = 0.f;
-    for (int q = 0; q < nw; ++q) s += sm[q][k];
-    v[k] = s;
-  }
-  __syncthreads();
-}
 
 struct LossArgs {
   const float* rgb;
@@ -33,6 +13,7 @@ struct LossArgs {
   int W, H, tiles_x;
   const int32_t* active_tiles;
   const int32_t* n_active;
+  int n_active_max;
   const int32_t* pix_off;
   const uint8_t* pix_idx;
   float eps_c2, eps_n, beta, weight;
@@ -50,121 +31,169 @@ constexpr float kC1 = 1e-4f, kC2 = 9e-4f;
 // STRUCT 0: the sparse NCC term (Sec. 3.7); 1: the SSIM term of Table 4's
 // S-SSIM variant, per channel from the same tile moments:
 // SSIM = (2 mx my + C1)(2 cov + C2) / ((mx^2 + my^2 + C1)(var_x + var_y + C2)).
-template <int STRUCT>
-__global__ void k_loss(LossArgs a) {
-  __shared__ float sm[8][9];
-  const int j = blockIdx.x;
+//
+// A warp takes whole tiles in turn, PPL pixels a lane (pixel lane + 32 k), held in
+// registers from the loads to the stores: a sum over the tile is a lane's own
+// sum and one warp reduction, nothing waits at a barrier, and the loss leaves a
+// block as one atomic at its end.  Bound by the chains of loads and reductions of
+// the few warps that the registers leave.  With a block per tile and a thread
+// per pixel every one of a tile's eight warps took all 18 reductions, three
+// block sums of two barriers each, and one thread's FP64 divisions and atomic
+// ended every tile: every pixel of 1957x1091 116 -> 42 us, of 1280x720 49 -> 20;
+// 720 tiles of 85 pixels 10 -> 7.7, eight views of 1200 to 4500 such tiles 192 ->
+// 105.
+constexpr int kLossWarps = 4;
+// Blocks on an SM, and launched per SM: 168 registers hold eight pixels a lane
+// without spills (four blocks of 128: 51 us for 42; 105 for 115 at three pixels).
+__host__ __device__ constexpr int loss_blocks(int ppl) { return ppl > 4 ? 3 : 4; }
+
+template <int STRUCT, int PPL>
+__global__ void __launch_bounds__(32 * kLossWarps, loss_blocks(PPL)) k_loss(LossArgs a) {
+  __shared__ double s_sum[kLossWarps][2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int A = *a.n_active;
-  if (j >= A) return;
-  const int P = a.pix_off[A];
-  const int t = a.active_tiles ? a.active_tiles[j] : j;
-  const int p0 = a.pix_off[j], p1 = a.pix_off[j + 1];
-  const int n = p1 - p0;
-  const int s = p0 + threadIdx.x;
-  const bool on = (int)threadIdx.x < n;
-  float x[3] = {0.f, 0.f, 0.f}, y[3] = {0.f, 0.f, 0.f};
-  size_t pix = 0;
-  if (on) {
-    const int l = a.pix_idx[s];
-    const int px = (t % a.tiles_x) * TGS_TILE + (l & 15), py = (t / a.tiles_x) * TGS_TILE + (l >> 4);
-    pix = (size_t)py * a.W + px;
+  const int P = A > 0 ? a.pix_off[A] : 0;
+  double sum_l1 = 0.0, sum_lam = 0.0, sum_corr = 0.0;  // over the warp's tiles: L1, lambda, lambda times the structure sum
+  for (int j = blockIdx.x * kLossWarps + warp; j < min(A, a.n_active_max); j += gridDim.x * kLossWarps) {
+    const int t = a.active_tiles ? a.active_tiles[j] : j;
+    const int p0 = a.pix_off[j], n = a.pix_off[j + 1] - p0;
+    if (n <= 0) continue;
+    const int tx0 = (t % a.tiles_x) * TGS_TILE, ty0 = (t / a.tiles_x) * TGS_TILE;
+    float x[PPL][3], y[PPL][3];
+    uint32_t pix[PPL];
+    uint16_t old_err[PPL];
+    int loc[PPL];
+#pragma unroll
+    for (int k = 0; k < PPL; ++k) loc[k] = lane + 32 * k < n ? a.pix_idx[p0 + lane + 32 * k] : -1;
+#pragma unroll
+    for (int k = 0; k < PPL; ++k) {
+      const bool on = loc[k] >= 0;
+      pix[k] = on ? (uint32_t)(ty0 + (loc[k] >> 4)) * (uint32_t)a.W + (uint32_t)(tx0 + (loc[k] & 15)) : 0u;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        x[k][c] = on ? a.rgb[3 * (size_t)(p0 + lane + 32 * k) + c] : 0.f;
+        y[k][c] = on ? a.target[3 * (size_t)pix[k] + c] : 0.f;
+      }
+      // the pixel's error-map entry, read now so that the load overlaps the reductions
+      old_err[k] = on && a.err_map ? a.err_map[pix[k]] : (uint16_t)0;
+    }
+    const float inv_n = 1.f / (float)n;
+    // pass 1: means
+    float mx[3], my[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      x[c] = a.rgb[3 * (size_t)s + c];
-      y[c] = a.target[3 * pix + c];
+      float sx = x[0][c], sy = y[0][c];
+#pragma unroll
+      for (int k = 1; k < PPL; ++k) {
+        sx += x[k][c];
+        sy += y[k][c];
+      }
+      mx[c] = warp_sum(sx) * inv_n;
+      my[c] = warp_sum(sy) * inv_n;
     }
-  }
-  // the pixel's error-map entry, read now so that the load overlaps the
-  // block reductions (the barriers between would otherwise hold it back)
-  uint16_t old_err = 0;
-  if (on && a.err_map) old_err = a.err_map[pix];
-  if (n <= 0) return;  // uniform per block
-  const float inv_n = 1.f / (float)n;
-  // pass 1: means
-  float m[6] = {x[0], x[1], x[2], y[0], y[1], y[2]};
-  block_sum<6>(m, reinterpret_cast<float(*)[6]>(&sm[0][0]));
-  float mx[3], my[3];
+    // pass 2: variances and covariances
+    float mom[9];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    mx[c] = m[c] * inv_n;
-    my[c] = m[3 + c] * inv_n;
-  }
-  // pass 2: variances and covariances
-  float dx[3], dy[3];
+    for (int q = 0; q < 9; ++q) mom[q] = 0.f;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    dx[c] = on ? x[c] - mx[c] : 0.f;
-    dy[c] = on ? y[c] - my[c] : 0.f;
-  }
-  float mom[9] = {dx[0] * dx[0], dx[1] * dx[1], dx[2] * dx[2], dy[0] * dy[0], dy[1] * dy[1],
-                  dy[2] * dy[2], dx[0] * dy[0], dx[1] * dy[1], dx[2] * dy[2]};
-  block_sum<9>(mom, sm);
-  // NCC: D = sqrt(var_x var_y + eps), ncc = cov / D.  SSIM: ncc holds SSIM,
-  // q1 = 1 / (b1 b2), q2 = mx / b1, D = b2 (a1, a2, b1, b2 as in the SSIM formula)
-  float vy[3], D[3], ncc[3], a1[3], a2[3], q1[3], q2[3];
+    for (int k = 0; k < PPL; ++k)
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float vx = mom[c] * inv_n;
-    vy[c] = mom[3 + c] * inv_n;
-    const float cv = mom[6 + c] * inv_n;
-    if (STRUCT == 0) {
-      D[c] = sqrtf(vx * vy[c] + a.eps_n);
-      ncc[c] = cv / D[c];
-    } else {
-      a1[c] = 2.f * mx[c] * my[c] + kC1;
-      a2[c] = 2.f * cv + kC2;
-      const float b1 = mx[c] * mx[c] + my[c] * my[c] + kC1;
-      D[c] = vx + vy[c] + kC2;
-      q1[c] = 1.f / (b1 * D[c]);
-      q2[c] = mx[c] / b1;
-      ncc[c] = a1[c] * a2[c] * q1[c];
+      for (int c = 0; c < 3; ++c) {
+        const float dx = loc[k] >= 0 ? x[k][c] - mx[c] : 0.f, dy = loc[k] >= 0 ? y[k][c] - my[c] : 0.f;
+        mom[c] += dx * dx;
+        mom[3 + c] += dy * dy;
+        mom[6 + c] += dx * dy;
+      }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) mom[q] = warp_sum(mom[q]);
+    // NCC: D = sqrt(var_x var_y + eps), ncc = cov / D.  SSIM: ncc holds SSIM,
+    // q1 = 1 / (b1 b2), q2 = mx / b1, D = b2 (a1, a2, b1, b2 as in the SSIM formula)
+    // cx = ncc var_y / D, what a pixel's dx weighs in the NCC gradient
+    float D[3], ncc[3], cx[3], a1[3], a2[3], q1[3], q2[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float vx = mom[c] * inv_n;
+      const float vy = mom[3 + c] * inv_n;
+      const float cv = mom[6 + c] * inv_n;
+      if (STRUCT == 0) {
+        D[c] = sqrtf(vx * vy + a.eps_n);
+        ncc[c] = cv / D[c];
+        cx[c] = ncc[c] * vy / D[c];
+      } else {
+        a1[c] = 2.f * mx[c] * my[c] + kC1;
+        a2[c] = 2.f * cv + kC2;
+        const float b1 = mx[c] * mx[c] + my[c] * my[c] + kC1;
+        D[c] = vx + vy + kC2;
+        q1[c] = 1.f / (b1 * D[c]);
+        q2[c] = mx[c] / b1;
+        ncc[c] = a1[c] * a2[c] * q1[c];
+      }
     }
-  }
-  // per-pixel gradients of both terms and the balancing weight
-  float d1[3], dn[3], l1 = 0.f, e = 0.f;
-  float gs[2] = {0.f, 0.f};
+    // per-pixel gradients of both terms (in x and y from here on) and the balancing weight
+    float l1 = 0.f, g1 = 0.f, gn = 0.f, e[PPL];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float d = x[c] - y[c];
-    const float r = sqrtf(d * d + a.eps_c2);
-    d1[c] = d / r;                                             // dl1/dx
-    if (STRUCT == 0)
-      dn[c] = (dy[c] - ncc[c] * vy[c] * dx[c] / D[c]) / D[c];  // n dNCC_c/dx
-    else                                                        // n dSSIM_c/dx
-      dn[c] = 2.f * ((my[c] * a2[c] + a1[c] * dy[c]) * q1[c] - ncc[c] * (q2[c] + dx[c] / D[c]));
-    if (on) {
-      l1 += r;
-      e += fabsf(d);
-      gs[0] += fabsf(d1[c]);
-      gs[1] += fabsf(dn[c]);
+    for (int k = 0; k < PPL; ++k) {
+      e[k] = 0.f;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float d = x[k][c] - y[k][c], dx = x[k][c] - mx[c], dy = y[k][c] - my[c];
+        const float r = sqrtf(d * d + a.eps_c2);
+        const float d1 = d / r;                               // dl1/dx
+        float dn;
+        if (STRUCT == 0)
+          dn = (dy - cx[c] * dx) / D[c];                      // n dNCC_c/dx
+        else                                                  // n dSSIM_c/dx
+          dn = 2.f * ((my[c] * a2[c] + a1[c] * dy) * q1[c] - ncc[c] * (q2[c] + dx / D[c]));
+        if (loc[k] >= 0) {
+          l1 += r;
+          e[k] += fabsf(d);
+          g1 += fabsf(d1);
+          gn += fabsf(dn);
+        }
+        x[k][c] = d1;
+        y[k][c] = dn;
+      }
     }
-  }
-  float g2[2] = {gs[0], gs[1]};
-  {
-    float v9[9] = {g2[0], g2[1], on ? l1 : 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    block_sum<9>(v9, sm);
-    g2[0] = v9[0];
-    g2[1] = v9[1];
-    l1 = v9[2];
-  }
-  const float lam = fminf(1.f, fmaxf(0.f, (g2[0] * inv_n) / (g2[1] * inv_n + 1e-8f)));
-  if (on) {
+    l1 = warp_sum(l1);
+    g1 = warp_sum(g1);
+    gn = warp_sum(gn);
+    const float lam = fminf(1.f, fmaxf(0.f, (g1 * inv_n) / (gn * inv_n + 1e-8f)));
     const float invP = 1.f / (float)P;
     const float cn = lam / (3.f * (float)A) * inv_n;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) a.dL[3 * (size_t)s + c] = (d1[c] * invP - cn * dn[c]) * a.weight;
-    a.err_pix[s] = e;
-    if (a.err_map) {
-      const float old = __half2float(__ushort_as_half(old_err));
-      a.err_map[pix] = __half_as_ushort(__float2half_rn((1.f - a.beta) * old + a.beta * e));
+    for (int k = 0; k < PPL; ++k)
+      if (loc[k] >= 0) {
+        const size_t s = (size_t)(p0 + lane + 32 * k);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.dL[3 * s + c] = (x[k][c] * invP - cn * y[k][c]) * a.weight;
+        a.err_pix[s] = e[k];
+        if (a.err_map) {
+          const float old = __half2float(__ushort_as_half(old_err[k]));
+          a.err_map[pix[k]] = __half_as_ushort(__float2half_rn(__fmaf_rn(a.beta, e[k], __fmul_rn(1.f - a.beta, old))));
+        }
+        if (a.age_map) a.age_map[pix[k]] = 0;
+      }
+    if (lane == 0) {
+      a.lambda[j] = lam;
+      sum_l1 += (double)l1;
+      sum_lam += (double)lam;
+      sum_corr += (double)lam * ((double)ncc[0] + (double)ncc[1] + (double)ncc[2]);
     }
-    if (a.age_map) a.age_map[pix] = 0;
   }
-  if (threadIdx.x == 0) {
-    a.lambda[j] = lam;
-    const double tile_loss = (double)l1 / (double)P +
-                             (double)lam * (1.0 - ((double)ncc[0] + (double)ncc[1] + (double)ncc[2]) / 3.0) / (double)A;
-    atomicAdd(a.loss, tile_loss * (double)a.weight);
+  if (lane == 0) {
+    s_sum[warp][0] = sum_l1;
+    s_sum[warp][1] = 3.0 * sum_lam - sum_corr;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && P > 0 && blockIdx.x * kLossWarps < A) {
+    double l = 0.0, q = 0.0;
+    for (int w = 0; w < kLossWarps; ++w) {
+      l += s_sum[w][0];
+      q += s_sum[w][1];
+    }
+    // l / P + q / (3 A), in one FP64 division
+    const double a3 = 3.0 * (double)A;
+    atomicAdd(a.loss, (l * a3 + q * (double)P) / (a3 * (double)P) * (double)a.weight);
   }
 }
 
@@ -215,16 +244,24 @@ static tgs_status loss_impl(int structure, const float* rgb, const float* target
   if (n_active_max > 0) {
     LossArgs a;
     a.rgb = rgb; a.target = target; a.W = width; a.H = height; a.tiles_x = tiles_x(width);
-    a.active_tiles = active_tiles; a.n_active = n_active; a.pix_off = pix_off; a.pix_idx = pix_idx;
+    a.active_tiles = active_tiles; a.n_active = n_active; a.n_active_max = n_active_max; a.pix_off = pix_off; a.pix_idx = pix_idx;
     a.eps_c2 = params->eps_charbonnier * params->eps_charbonnier;
     a.eps_n = params->eps_ncc;
     a.beta = params->beta;
     a.weight = params->view_weight;
     a.err_map = err_map; a.age_map = age_map; a.dL = dL_drgb; a.lambda = lambda_tile; a.err_pix = err_pix;
     a.loss = loss;
-    const int B = std::min(256, std::max(32, (n_pix_max + 31) / 32 * 32));
-    if (structure == 0) k_loss<0><<<n_active_max, B, 0, s>>>(a);
-    else k_loss<1><<<n_active_max, B, 0, s>>>(a);
+    const int ppl = n_pix_max <= 128 ? (n_pix_max + 31) / 32 : 8;
+    const int blocks = std::min((n_active_max + kLossWarps - 1) / kLossWarps,
+                                loss_blocks(ppl) * std::max(1, device_sm_count()));
+    auto launch = [&](auto ncc, auto ssim) { (structure == 0 ? ncc : ssim)<<<blocks, 32 * kLossWarps, 0, s>>>(a); };
+    switch (ppl) {
+      case 1: launch(k_loss<0, 1>, k_loss<1, 1>); break;
+      case 2: launch(k_loss<0, 2>, k_loss<1, 2>); break;
+      case 3: launch(k_loss<0, 3>, k_loss<1, 3>); break;
+      case 4: launch(k_loss<0, 4>, k_loss<1, 4>); break;
+      default: launch(k_loss<0, 8>, k_loss<1, 8>); break;
+    }
   }
   return check_launch();
 }

@@ -71,14 +71,17 @@ struct HashKeys {
   }
 };
 
-// 32 tiles per block of 8 warps, 4 tiles per warp: lane l sums the error
-// weights and takes the minimum age of eight pixels of each (row l / 2,
-// columns 8 (l % 2) .. + 7; one 16-byte load per map where the row allows
-// it), all four tiles' loads in flight together, then the warp reduces.  The
-// draws (-log2 of a hash, 32 dependent squarings) then run one tile per lane
-// of the first warp.
-constexpr int kStatsTiles = 32;
+// 8 tiles per block of 8 warps, one per warp: lane l sums the error
+// weights and takes the minimum age of eight pixels (row l / 2, columns
+// 8 (l % 2) .. + 7; one 16-byte load per map where the row allows it), then the
+// warp reduces.  The draws (-log2 of a hash, 32 dependent squarings) then run
+// one tile per lane of the first warp.  Bound by latency: the loads, then the
+// draws.  With four tiles a warp (32 a block) a view of 4056 tiles had fewer
+// blocks than the chip has SMs: 12.8 us, 8.3 with two, 7.1 with one; 256 tiles
+// 6.2, 4.6, 3.9; 8160 tiles 8.6, 7.9, 7.4.
+constexpr int kStatsTiles = 8;
 constexpr int kStatsPerWarp = kStatsTiles / 8;
+static_assert(kStatsTiles % 8 == 0 && kStatsTiles <= 32, "whole tiles per warp, and a lane of the first warp each");
 
 __device__ __forceinline__ void pixel_row8(const uint16_t* __restrict__ err, const uint16_t* __restrict__ age,
                                            const SelGeom& g, int t, int lane, bool vec, uint64_t& wv,
@@ -150,13 +153,36 @@ __global__ void __launch_bounds__(256) k_tile_stats(const uint16_t* __restrict__
   }
   __syncthreads();
   const int t = t0 + lane;
-  if (warp == 0 && t < g.T) {
+  if (warp == 0 && lane < kStatsTiles && t < g.T) {
     w.tile_w[t] = s_w[lane];
     w.tile_age[t] = s_a[lane];
     // the FP64 division runs here, spread over the grid, and not in the
     // single-block selection (FP64 throughput is low on this part)
     w.tile_key[t] = hard_key(s_w[lane], neglog2_q32(hash_item(hk.prefix(STREAM_TILE_HARD), (uint32_t)t, 0)));
     w.tile_u[t] = hash_item(hk.prefix(STREAM_TILE_UNIF), (uint32_t)t, 0);
+  }
+}
+
+// Every tile selected: ranks are the tile ids, and the pixels before a tile
+// follow from its row and column (only the last row and column have tiles of
+// other sizes).  The single-block compaction took 6.3 us at 3600 tiles and 17.8
+// at 8487, this 2.8 and 1.5.
+__global__ void __launch_bounds__(256) k_select_all(SelGeom g, int n_pix, int32_t* __restrict__ active_tiles,
+                                                    int32_t* __restrict__ n_active, int32_t* __restrict__ tile_rank,
+                                                    int32_t* __restrict__ pix_off) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= g.T) return;
+  const int x = t % g.tx, y = t / g.tx, ty = g.T / g.tx;
+  const int w_last = g.W - (g.tx - 1) * TGS_TILE, h_last = g.H - (ty - 1) * TGS_TILE;
+  const int h = y == ty - 1 ? h_last : TGS_TILE, w = x == g.tx - 1 ? w_last : TGS_TILE;
+  const int row = (g.tx - 1) * min(n_pix, TGS_TILE * TGS_TILE) + min(n_pix, w_last * TGS_TILE);  // of a whole row
+  const int off = y * row + x * min(n_pix, TGS_TILE * h);
+  active_tiles[t] = t;
+  tile_rank[t] = t;
+  pix_off[t] = off;
+  if (t == g.T - 1) {
+    pix_off[g.T] = off + min(n_pix, w * h);
+    *n_active = g.T;
   }
 }
 
@@ -213,13 +239,10 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select_block(SelWs w, SelGeo
   __shared__ SelectSmem sm;
   __shared__ int64_t s64[32];
   const int T = g.T;
-  const bool all = n_sel >= T;
   const int i0 = threadIdx.x * ITEMS;
   const uint32_t valid = i0 < T ? (ITEMS < T - i0 ? (1u << ITEMS) - 1u : (1u << (T - i0)) - 1u) : 0u;
   uint32_t taken = 0u;
-  if (all) {
-    taken = valid;
-  } else if (n_sel > 0) {
+  if (n_sel > 0) {
     uint32_t key[ITEMS];
     // the hard keys are read again where their low words are wanted
     auto hard = [&](int j) -> uint64_t { return (valid >> j) & 1u ? w.tile_key[i0 + j] : 0ull; };
@@ -509,7 +532,9 @@ static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map
   if (n_sel < T && n_sel > 0)
     k_tile_stats<<<(T + kStatsTiles - 1) / kStatsTiles, 256, 0, s>>>(
         err_map, age_map, g, hk, w, aligned16(err_map) && aligned16(age_map) && width % 8 == 0);
-  if (T <= kSelBlockMaxTiles) {
+  if (n_sel >= T) {
+    k_select_all<<<(T + 255) / 256, 256, 0, s>>>(g, n_pix, active_tiles, n_active, tile_rank, pix_off);
+  } else if (T <= kSelBlockMaxTiles) {
     // one block: the three phases and the compaction
     if (T <= kSelThreads)
       k_select_block<1><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
@@ -528,7 +553,7 @@ static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map
     // tile is taken when rank_h < kh, or (not hard) rank_s < ks, or
     // (neither) rank_u < n_sel - kh - ks.
     cudaMemsetAsync(w.rank_h, 0, sizeof(int32_t) * 3 * (size_t)T, s);
-    if (n_sel < T && n_sel > 0) {
+    if (n_sel > 0) {
       dim3 grid((T + 255) / 256, (T + RANK_CHUNK - 1) / RANK_CHUNK);
       if (kh > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 0, kh, ks);
       if (ks > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 1, kh, ks);
@@ -537,14 +562,14 @@ static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map
     const int32_t* rh = w.rank_h;
     const int32_t* rs = w.rank_s;
     const int32_t* ru = w.rank_u;
-    const int all = n_sel >= T ? 1 : 0, none = n_sel == 0 ? 1 : 0;
+    const int none = n_sel == 0 ? 1 : 0;
     const int ku = n_sel - kh - ks;
     const int npx = n_pix;
     int32_t* at = active_tiles;
     int32_t* tr = tile_rank;
     int32_t* po = pix_off;
     auto load = [=] __device__(int64_t t) -> int64_t {
-      const bool taken = !none && (all || rh[t] < kh || rs[t] < ks || (rs[t] >= ks && ru[t] < ku));
+      const bool taken = !none && (rh[t] < kh || rs[t] < ks || (rs[t] >= ks && ru[t] < ku));
       if (!taken) return 0;
       return (1ll << 32) | (int64_t)min(npx, tile_valid(g, (int)t));
     };

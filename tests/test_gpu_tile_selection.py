@@ -39,3 +39,27 @@ def test_tile_selection_bit_exact(B, orc, tx, ty, kind, ages):
         assert got["n_active"] == want["n_active"]
         for k in ("active_tiles", "tile_rank", "pix_off"):
             np.testing.assert_array_equal(got[k], want[k])
+
+
+@pytest.mark.parametrize("W,H", [(16, 16), (17, 15), (250, 187), (256, 256), (64, 16), (16, 64), (1957, 1091), (4099, 1031)])
+@pytest.mark.parametrize("n_pix", [1, 85, 200, 256])
+def test_every_tile_bit_exact(B, orc, W, H, n_pix):
+    """Every tile selected (by itself and with a larger n_select): ragged last
+    rows and columns with fewer pixels than n_pix, one row, one column, more
+    tiles than the one-block selection takes."""
+    from gpu_util import select_dev, select_host
+    T = ((W + 15) // 16) * ((H + 15) // 16)
+    err, age = scenes.error_map(W, H, seed=T), scenes.age_map(W, H, seed=H, max_age=9)
+    for n_sel in (T, T + 5):
+        got = select_host(select_dev(B, err, age, W, H, n_sel, n_pix, seed=2, it=1, view=0))
+        assert got["n_active"] == T
+        np.testing.assert_array_equal(got["active_tiles"], np.arange(T))
+        np.testing.assert_array_equal(got["tile_rank"], np.arange(T))
+        w = np.minimum(16, W - 16 * np.arange((W + 15) // 16))
+        h = np.minimum(16, H - 16 * np.arange((H + 15) // 16))
+        n = np.minimum(n_pix, (h[:, None] * w[None, :]).reshape(-1))
+        np.testing.assert_array_equal(got["pix_off"], np.concatenate([[0], np.cumsum(n)]))
+        if T < 3000:
+            want = orc.select(err, age, W, H, n_select=n_sel, n_pix=n_pix, tile_hard_pm=400, tile_stable_pm=300,
+                              pix_hard_pm=400, pix_stable_pm=300, seed=2, it=1, view=0)
+            np.testing.assert_array_equal(got["pix_idx"], want["pix_idx"])

@@ -65,13 +65,14 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, int deg, flo
 // Colour before the clamp from the whole SH row (48 floats at every degree) and
 // the basis: the sums in one fixed form, so that every kernel gives the same
 // bits.
-__device__ __forceinline__ void sh_colour(const float4 (&row)[12], const float (&Y)[16], int sh_degree,
-                                          float (&acc)[3]) {
+template <class Row>
+__device__ __forceinline__ void sh_colour_from(const Row& row, const float (&Y)[16], int sh_degree, float (&acc)[3]) {
   const int nb = (sh_degree + 1) * (sh_degree + 1);
   acc[0] = acc[1] = acc[2] = 0.5f;
 #pragma unroll
   for (int k4 = 0; k4 < 12; ++k4) {
-    const float e[4] = {row[k4].x, row[k4].y, row[k4].z, row[k4].w};
+    const float4 q = row(k4);
+    const float e[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int f = 4 * k4 + j;  // flat index k * 3 + c
@@ -79,6 +80,18 @@ __device__ __forceinline__ void sh_colour(const float4 (&row)[12], const float (
       if (k < nb) acc[c] = __fmaf_rn(e[j], Y[k], acc[c]);
     }
   }
+}
+__device__ __forceinline__ void sh_colour(const float4 (&row)[12], const float (&Y)[16], int sh_degree,
+                                          float (&acc)[3]) {
+  sh_colour_from([&](int k4) { return row[k4]; }, Y, sh_degree, acc);
+}
+
+// Unit direction from the camera centre to mu, in one fixed form for the same
+// reason.
+__device__ __forceinline__ float3 view_direction(const CamK& cam, float3 mu) {
+  const float dx = mu.x - cam.campos[0], dy = mu.y - cam.campos[1], dz = mu.z - cam.campos[2];
+  const float il = rsqrtf(__fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy))));
+  return make_float3(dx * il, dy * il, dz * il);
 }
 
 // gradient of sum_k s_k Y_k with respect to the (unnormalised) polynomial argument
@@ -216,46 +229,100 @@ __device__ __forceinline__ bool touches_active(const CamK& cam, const float xy[2
   return false;
 }
 
-__global__ void __launch_bounds__(256) k_project(
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_wait_all() {
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+}
+constexpr int kShPad = 52;  // floats per staged SH row: float4 reads by row are conflict-free
+
+// One view.  A lane takes a Gaussian; the SH rows of a warp's visible ones are
+// copied to shared memory by the whole warp, consecutive 16-byte pieces a copy,
+// sixteen rows a round, and read back by row.  With each lane loading its own
+// row of 192 bytes (32 lines a load) the kernel was bound by the L1, 60-71 %
+// busy at 41 % of the copy rate; now by latency at ten blocks an SM (32 rows a
+// round and eight blocks: 33.9, 34.9, 120.8, 56.3 us for the sizes below).
+// ROWS: geometric fields in 64-byte rows (means, log-scale 0 | log-scales 1, 2,
+// opacity logit, unused | quaternion), three loads a Gaussian in place of eight.
+// 500k Gaussians, 720 tiles 33.8 -> 30.8 us, every tile 37.3 -> 32.1; 2M, 1340
+// tiles 106.7 -> 105.2; 1M, every tile 57.0 -> 51.9.
+constexpr int kProjectThreads = 128;
+constexpr int kShRows = 16;
+
+template <bool ROWS>
+__global__ void __launch_bounds__(kProjectThreads, 10) k_project(
     GeoC geo, const float4* __restrict__ sh, int64_t n, int sh_degree, CamK cam,
     const int32_t* __restrict__ tile_rank, float2* __restrict__ xy_out, float4* __restrict__ conic_out,
     float* __restrict__ rgb_out, float* __restrict__ depth_out, int32_t* __restrict__ radius_out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float3 mu = geo.mean(i);
-  float3 ls = geo.lsc(i);
-  float4 qr = geo.quat(i);
+  __shared__ __align__(16) float s_sh[kProjectThreads / 32 * kShRows][kShPad];
+  __shared__ uint8_t s_list[kProjectThreads];
+  const int64_t i = (int64_t)blockIdx.x * kProjectThreads + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const bool in = i < n;
+  float3 mu = make_float3(0.f, 0.f, 0.f), ls = mu;
+  float4 qr = make_float4(0.f, 0.f, 0.f, 0.f);
+  float op = 0.f;
+  if (in) {
+    if (ROWS) {
+      const float4* row = reinterpret_cast<const float4*>(geo.m) + 4 * i;
+      const float4 r0 = row[0], r1 = row[1];
+      qr = row[2];
+      mu = make_float3(r0.x, r0.y, r0.z);
+      ls = make_float3(r0.w, r1.x, r1.y);
+      op = r1.z;
+    } else {
+      mu = geo.mean(i);
+      ls = geo.lsc(i);
+      qr = geo.quat(i);
+      op = geo.opac(i);
+    }
+  }
   Geo g;
-  bool vis = geometry(cam, mu, ls, qr, g) && touches_active(cam, g.xy, g.radius, tile_rank);
-  if (!vis) {
+  const bool vis = in && geometry(cam, mu, ls, qr, g) && touches_active(cam, g.xy, g.radius, tile_rank);
+  if (in && !vis) {
     xy_out[i] = make_float2(0.f, 0.f);
     conic_out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     rgb_out[3 * i] = 0.f; rgb_out[3 * i + 1] = 0.f; rgb_out[3 * i + 2] = 0.f;
     depth_out[i] = 0.f;
     radius_out[i] = 0;
-    return;
   }
-  // colour from SH in the viewing direction
-  float dx = mu.x - cam.campos[0], dy = mu.y - cam.campos[1], dz = mu.z - cam.campos[2];
-  float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-  dx *= il; dy *= il; dz *= il;
-  float Y[16];
-  sh_basis(dx, dy, dz, sh_degree, Y);
-  const float4* shp = sh + 12 * i;
-  // the whole row (48 floats at every degree) in one round of loads: a loop
-  // that stops at the degree would wait for each load in turn
-  float4 row[12];
-#pragma unroll
-  for (int k4 = 0; k4 < 12; ++k4) row[k4] = ldg_f4_now(shp + k4);
-  float acc[3];
-  sh_colour(row, Y, sh_degree, acc);
-  xy_out[i] = make_float2(g.xy[0], g.xy[1]);
-  conic_out[i] = make_float4(g.conic[0], g.conic[1], g.conic[2], 1.f / (1.f + expf(-geo.opac(i))));
-  rgb_out[3 * i] = fmaxf(acc[0], 0.f);
-  rgb_out[3 * i + 1] = fmaxf(acc[1], 0.f);
-  rgb_out[3 * i + 2] = fmaxf(acc[2], 0.f);
-  depth_out[i] = g.pc[2];
-  radius_out[i] = g.radius;
+  if (vis) {
+    xy_out[i] = make_float2(g.xy[0], g.xy[1]);
+    conic_out[i] = make_float4(g.conic[0], g.conic[1], g.conic[2], 1.f / (1.f + expf(-op)));
+    depth_out[i] = g.pc[2];
+    radius_out[i] = g.radius;
+  }
+  // colour from SH in the viewing direction, kShRows of the warp's visible Gaussians a round
+  const unsigned seen = __ballot_sync(0xffffffffu, vis);
+  const int slot = __popc(seen & ((1u << lane) - 1u)), rows = __popc(seen);
+  float (*dst)[kShPad] = s_sh + (threadIdx.x >> 5) * kShRows;
+  uint8_t* list = s_list + (threadIdx.x - lane);
+  if (vis) list[slot] = (uint8_t)lane;
+  __syncwarp();
+  const float4* src = sh + 12 * (i - lane);
+#pragma unroll 1
+  for (int r0 = 0; r0 < rows; r0 += kShRows) {
+    const int nr = min(kShRows, rows - r0);
+    for (int p = lane; p < 12 * nr; p += 32) {
+      const int r = p / 12, c = p - 12 * r;
+      cp_async16(&dst[r][4 * c], src + 12 * (int)list[r0 + r] + c);
+    }
+    cp_async_commit_wait_all();
+    __syncwarp();
+    if (vis && slot >= r0 && slot < r0 + kShRows) {
+      const float3 d = view_direction(cam, mu);
+      float Y[16];
+      sh_basis(d.x, d.y, d.z, sh_degree, Y);
+      float acc[3];
+      sh_colour_from([&](int k4) { return *reinterpret_cast<const float4*>(&dst[slot - r0][4 * k4]); }, Y, sh_degree, acc);
+      rgb_out[3 * i] = fmaxf(acc[0], 0.f);
+      rgb_out[3 * i + 1] = fmaxf(acc[1], 0.f);
+      rgb_out[3 * i + 2] = fmaxf(acc[2], 0.f);
+    }
+    __syncwarp();
+  }
 }
 
 // Several views of one step in one pass: each Gaussian's parameters are read
@@ -318,11 +385,9 @@ __global__ void __launch_bounds__(256) k_project_multi(GeoC geo, const float4* _
     const ProjectView& o = views.v[v];
     float acc[3] = {0.f, 0.f, 0.f};
     if ((seen >> v) & 1u) {
-      float dx = mu.x - o.cam.campos[0], dy = mu.y - o.cam.campos[1], dz = mu.z - o.cam.campos[2];
-      const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-      dx *= il; dy *= il; dz *= il;
+      const float3 d = view_direction(o.cam, mu);
       float Y[16];
-      sh_basis(dx, dy, dz, sh_degree, Y);
+      sh_basis(d.x, d.y, d.z, sh_degree, Y);
       sh_colour(row, Y, sh_degree, acc);
     }
 #pragma unroll
@@ -979,14 +1044,6 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_update(
   }
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_wait_all() {
-  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
 // The fused adjoint + update for geometric fields in 64-byte rows (geo_stride
 // 16, rows on 16-byte boundaries).  The same two roles and the same
 // arithmetic as k_adj_update, but a round first copies the whole rows it
@@ -1002,7 +1059,6 @@ __device__ __forceinline__ void cp_async_commit_wait_all() {
 // (7 and 12..15) are written back with the values read.
 constexpr int kRowsG = 64;  // Gaussians a round of the staged-row kernel (128 threads a block)
 constexpr int kGeoPad = 20;  // floats per staged geometric row: float4 reads by row are conflict-free
-constexpr int kShPad = 52;   // floats per staged SH row
 
 template <int G>
 struct __align__(16) AdjRowsSmem {
@@ -1364,8 +1420,9 @@ extern "C" tgs_status tgs_project_gaussians(const tgs_gaussians* g, const tgs_ca
       !aligned16(out->conic_opac))
     return TGS_ERR_INVALID_ARG;
   CamK k = make_cam(*cam);
-  int blocks = (int)((g->n + 255) / 256);
-  k_project<<<blocks, 256, 0, (cudaStream_t)stream>>>(
+  const int blocks = (int)((g->n + kProjectThreads - 1) / kProjectThreads);
+  const bool rows = g->geo_stride == 16 && aligned16(g->means);  // 64-byte rows on 16-byte boundaries
+  (rows ? k_project<true> : k_project<false>)<<<blocks, kProjectThreads, 0, (cudaStream_t)stream>>>(
       geo_of(*g), reinterpret_cast<const float4*>(g->sh), g->n, g->sh_degree, k, tile_rank,
       reinterpret_cast<float2*>(out->xy), reinterpret_cast<float4*>(out->conic_opac), out->rgb, out->depth,
       out->radius);

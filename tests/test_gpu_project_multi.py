@@ -2,7 +2,9 @@
 bit for bit: one view (which takes the single-view kernel), a few and sixteen,
 of different sizes and poses, numbers of Gaussians at the edges of a block,
 every SH degree, packed arrays and rows, tile masks (no mask, some tiles, none:
-a Gaussian that no view sees) and Gaussians behind every camera."""
+a Gaussian that no view sees), Gaussians behind every camera, and warps with up
+to 16, 17 and 32 visible Gaussians (the single-view kernel stages sixteen SH
+rows a round)."""
 import numpy as np
 import pytest
 import torch
@@ -20,12 +22,13 @@ def B():
 
 
 @pytest.mark.parametrize("n,K,degree,rows", [(1, 2, 3, False), (255, 16, 0, True), (257, 3, 1, False), (5000, 1, 3, True),
-                                             (5000, 5, 2, True), (20000, 8, 3, False)])
+                                             (5000, 5, 2, True), (20000, 8, 3, False), (16, 4, 3, True),
+                                             (17, 4, 2, False), (33, 4, 3, False), (31, 4, 1, True)])
 def test_views_in_one_pass_are_bit_exact(B, n, K, degree, rows):
     from gpu_util import empty_projected, gaussians_dev
     from paper_2606_15924_gb300.pipeline import as_geo_rows
     g = scenes.gaussians(n, seed=n)
-    if n > 100:
+    if n > 1000:
         g["means"][::7] *= 40.0                        # far off, and behind some of the cameras
         g["quats"][5] *= 3.0                             # not of unit length
     p = gaussians_dev(g)

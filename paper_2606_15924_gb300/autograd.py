@@ -50,6 +50,9 @@ class SampledRaster:
         self.n_last = torch.zeros(max(int(pix_idx.shape[0]), 1), dtype=torch.int32, device=dev)
         self.grad2d = torch.zeros(n, 12, device=dev)
         self.touched = torch.zeros(n, dtype=torch.uint8, device=dev)
+        # the pair count on the host: copied out after the binning, read once the render is under way
+        self._need = torch.zeros(1, dtype=torch.int64, pin_memory=True)
+        self._binned = torch.cuda.Event()
 
     @staticmethod
     def from_tiles(cam: dict, n_gaussians: int, tiles, device="cuda", **kw):
@@ -96,22 +99,37 @@ class SampledRaster:
                                   dtype=torch.uint8, device=dev)
         self.vals = torch.zeros(self.capacity, dtype=torch.int32, device=dev)
 
-    def forward_buffers(self, params: dict) -> torch.Tensor:
-        """project -> bin -> render; returns rgb [P, 3] (new tensor)."""
-        B.project_gaussians(params, self.ccam, self.tile_rank, self.proj, self.sh_degree)
-        self._ensure_bins()
+    def _bin(self):
         B.bin_tiles(self.proj, self.n, self.ccam, self.tile_rank, self.n_active_max, self.ws_bin, self.capacity,
                     self.vals, None, self.ranges, self.n_isect)
-        need = int(self.n_isect.item())
-        if need > self.capacity:  # the Gaussians moved: grow and bin again
+
+    def _render(self, rgb: torch.Tensor):
+        B.render_sampled(self.proj, self.ranges, self.vals, self.active_tiles, self.n_active, self.n_active_max,
+                         self.pix_off, self.pix_idx, self.n_pix, self.ccam, self.bg, rgb, self.T_final, self.n_last)
+
+    def forward_buffers(self, params: dict) -> torch.Tensor:
+        """project -> bin -> render; returns rgb [P, 3] (new tensor).  The render
+        is launched before the host waits for the number of pairs (lists are cut
+        at the capacity, so it is in bounds either way) and again if they did not
+        fit: a wait in between left the GPU idle for the launches that follow."""
+        B.project_gaussians(params, self.ccam, self.tile_rank, self.proj, self.sh_degree)
+        self._ensure_bins()
+        self._bin()
+        self._need.copy_(self.n_isect, non_blocking=True)
+        self._binned.record()
+        n_out = max(int(self.pix_idx.shape[0]), 1)
+        # every entry below P is written
+        make = torch.empty if self.P == n_out else torch.zeros
+        rgb = make(n_out, 3, device=self.active_tiles.device)
+        self._render(rgb)
+        self._binned.synchronize()
+        need = int(self._need[0])
+        if need > self.capacity:  # the Gaussians moved: grow, bin and render again
             self.capacity = int(need * 1.25) + 1024
             self.vals = None
             self._ensure_bins()
-            B.bin_tiles(self.proj, self.n, self.ccam, self.tile_rank, self.n_active_max, self.ws_bin,
-                        self.capacity, self.vals, None, self.ranges, self.n_isect)
-        rgb = torch.zeros(max(int(self.pix_idx.shape[0]), 1), 3, device=self.active_tiles.device)
-        B.render_sampled(self.proj, self.ranges, self.vals, self.active_tiles, self.n_active, self.n_active_max,
-                         self.pix_off, self.pix_idx, self.n_pix, self.ccam, self.bg, rgb, self.T_final, self.n_last)
+            self._bin()
+            self._render(rgb)
         return rgb[:self.P]
 
 
@@ -132,8 +150,12 @@ class _RenderSampled(torch.autograd.Function):
         means, log_scales, quats, opacity_logits, sh = ctx.saved_tensors
         params = dict(means=means, log_scales=log_scales, quats=quats, opacity_logits=opacity_logits, sh=sh)
         grads = {k: torch.empty_like(v) for k, v in params.items()}
-        g = torch.zeros(max(int(raster.pix_idx.shape[0]), 1), 3, device=means.device)
-        g[:raster.P] = dL_drgb
+        n_out = max(int(raster.pix_idx.shape[0]), 1)
+        if raster.P == n_out and dL_drgb.dtype == torch.float32 and dL_drgb.device == means.device:
+            g = dL_drgb.contiguous()
+        else:  # entries past the sampled pixels, or values to convert
+            g = torch.zeros(n_out, 3, device=means.device)
+            g[:raster.P] = dL_drgb
         B.backward_sampled(params, raster.ccam, raster.proj, raster.ranges, raster.vals, raster.active_tiles,
                            raster.n_active, raster.n_active_max, raster.pix_off, raster.pix_idx, raster.n_pix,
                            raster.bg, raster.T_final, raster.n_last, g, raster.grad2d, grads, raster.touched,

@@ -215,6 +215,32 @@ tgs_status tgs_select_tiles_noalloc(const uint16_t* err_map, const uint16_t* age
                                     uint8_t* pix_idx, tgs_stream stream);
 
 /*
+ * select_tiles_batched - select_tiles for 1 to 16 views of one step, which share
+ * the launches: view k with its maps, sizes, seed, view id, workspace and
+ * outputs, the sampling ratios and the iteration (iter, or *iter_dev) common.
+ * The results are those of one select_tiles call per view; outputs and
+ * workspaces of different views do not overlap.
+ */
+typedef struct {
+  const uint16_t* err_map;
+  const uint16_t* age_map;
+  int32_t width, height;
+  int32_t n_select, n_pix;
+  uint64_t seed;
+  uint32_t view;
+  void* workspace;
+  size_t workspace_bytes;
+  int32_t* active_tiles;
+  int32_t* n_active;
+  int32_t* tile_rank;
+  int32_t* pix_off;
+  uint8_t* pix_idx;
+} tgs_select_view;
+tgs_status tgs_select_tiles_batched(int32_t n_views, const tgs_select_view* views, const tgs_sampling* cfg,
+                                    uint64_t iter, const uint64_t* iter_dev, tgs_stream stream);
+
+
+/*
  * view_error_sums - the per-view error totals behind the anchor choice of
  * geometry-aware view sampling (Sec. 3.4, Eq. 5: the mean of E_v over the
  * image domain, which is this sum divided by W H).

@@ -6,7 +6,7 @@ loss of Eq. 11 is an expectation over them).  ``MultiViewTrainer`` keeps one
 tiles and pixels, projection, tile lists) and shares the Gaussians, their
 gradients and the optimiser moments.  One step:
 
-  per view: select_tiles
+  all views: select_tiles_batched (shared launches)
   all views: project_gaussians_multi (one pass over the Gaussians)
   per view: bin_tiles
   all views: render_sampled_batched (one persistent launch, (view, tile) queue)
@@ -171,8 +171,17 @@ class MultiViewTrainer:
                                view_row=self.rows[k] if self.use_rows else None, sh_degree=self.sh_degree)
 
     def _select(self):
-        for v in self.views:
-            v._select()
+        """Tile and pixel selection of all views, in shared launches (persistent)
+        or one after the other."""
+        if not self.persistent:
+            for v in self.views:
+                v._select()
+            return
+        B.select_tiles_batched(
+            [dict(err_map=v.err_map, age_map=v.age_map, width=v.W, height=v.H, n_select=v.n_select, n_pix=v.n_pix,
+                  seed=v.seed, view=v.view, workspace=v.ws_sel, active_tiles=v.active_tiles, n_active=v.n_active,
+                  tile_rank=v.tile_rank, pix_off=v.pix_off, pix_idx=v.pix_idx) for v in self.views],
+            self.cfg.sampling.permille(), 0, iter_dev=self.it_dev)
 
     def _project(self):
         """Projection of all views: one pass over the Gaussians (persistent), or

@@ -63,6 +63,14 @@ class Sampling(C.Structure):
                 ("pix_stable_pm", C.c_int32)]
 
 
+class SelectView(C.Structure):
+    _fields_ = [("err_map", C.c_void_p), ("age_map", C.c_void_p), ("width", C.c_int32), ("height", C.c_int32),
+                ("n_select", C.c_int32), ("n_pix", C.c_int32), ("seed", C.c_uint64), ("view", C.c_uint32),
+                ("workspace", C.c_void_p), ("workspace_bytes", C.c_size_t), ("active_tiles", C.c_void_p),
+                ("n_active", C.c_void_p), ("tile_rank", C.c_void_p), ("pix_off", C.c_void_p),
+                ("pix_idx", C.c_void_p)]
+
+
 class LossParams(C.Structure):
     _fields_ = [("eps_charbonnier", C.c_float), ("eps_ncc", C.c_float), ("beta", C.c_float),
                 ("view_weight", C.c_float)]
@@ -120,6 +128,8 @@ _lib.tgs_select_tiles_workspace_size.argtypes = [_i32, _i32]
 _lib.tgs_select_tiles.restype = _i32
 _lib.tgs_select_tiles.argtypes = [_p, _p, _i32, _i32, _i32, _i32, _P(Sampling), _u64, _u64, _p, _u32, _p, _sz,
                                   _p, _p, _p, _p, _p, _p]
+_lib.tgs_select_tiles_batched.restype = _i32
+_lib.tgs_select_tiles_batched.argtypes = [_i32, _p, _P(Sampling), _u64, _p, _p]
 _lib.tgs_select_tiles_noalloc.restype = _i32
 _lib.tgs_select_tiles_noalloc.argtypes = [_p, _p, _i32, _i32, _i32, _i32, _P(Sampling), _u64, _u64, _p, _u32,
                                           _p, _p, _p, _p, _p, _p]
@@ -218,7 +228,7 @@ _lib.tgs_mlp_adam.argtypes = [_p, _p, _p, _p, _i32, C.c_float, C.c_float, C.c_fl
 
 EXPORTED = ["tgs_version", "tgs_last_cuda_error", "tgs_status_string", "tgs_device_check", "tgs_graph_count_kernels",
             "tgs_advance_counters",
-            "tgs_select_tiles_workspace_size", "tgs_select_tiles", "tgs_select_tiles_noalloc",
+            "tgs_select_tiles_workspace_size", "tgs_select_tiles", "tgs_select_tiles_batched", "tgs_select_tiles_noalloc",
             "tgs_project_gaussians", "tgs_project_gaussians_multi",
             "tgs_bin_tiles_workspace_size", "tgs_bin_tiles", "tgs_checkpoint_bytes", "tgs_set_forward_split", "tgs_render_sampled",
             "tgs_loss_sparse_ncc", "tgs_loss_sparse_ssim",
@@ -352,6 +362,20 @@ def select_tiles(err_map, age_map, width, height, n_select, n_pix, sampling, see
         int(seed) & (2**64 - 1), int(it) & (2**64 - 1), _ptr(iter_dev), int(view), _ptr(workspace),
         workspace.numel(),
         _ptr(active_tiles), _ptr(n_active), _ptr(tile_rank), _ptr(pix_off), _ptr(pix_idx), _stream(stream)))
+
+
+def select_tiles_batched(views: list, sampling, it, stream=None, iter_dev=None):
+    """select_tiles for several views in shared launches.  views: dicts with
+    err_map, age_map, width, height, n_select, n_pix, seed, view, workspace,
+    active_tiles, n_active, tile_rank, pix_off, pix_idx."""
+    cfg = Sampling(*sampling)
+    arr = (SelectView * len(views))(*[
+        SelectView(_ptr(v["err_map"]), _ptr(v["age_map"]), int(v["width"]), int(v["height"]), int(v["n_select"]),
+                   int(v["n_pix"]), int(v["seed"]) & (2**64 - 1), int(v["view"]), _ptr(v["workspace"]),
+                   v["workspace"].numel(), _ptr(v["active_tiles"]), _ptr(v["n_active"]), _ptr(v["tile_rank"]),
+                   _ptr(v["pix_off"]), _ptr(v["pix_idx"])) for v in views])
+    _check("tgs_select_tiles_batched", _lib.tgs_select_tiles_batched(
+        len(views), arr, C.byref(cfg), int(it) & (2**64 - 1), _ptr(iter_dev), _stream(stream)))
 
 
 def select_tiles_noalloc(err_map, age_map, width, height, n_select, n_pix, sampling, seed, it, view, active_tiles,

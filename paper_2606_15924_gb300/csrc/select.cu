@@ -118,9 +118,34 @@ __device__ __forceinline__ void pixel_row8(const uint16_t* __restrict__ err, con
   }
 }
 
-__global__ void __launch_bounds__(256) k_tile_stats(const uint16_t* __restrict__ err,
-                                                    const uint16_t* __restrict__ age, SelGeom g, HashKeys hk,
-                                                    SelWs w, bool vec) {
+// The views of a launch; its second grid dimension counts them.
+constexpr int kMaxSelViews = 16;
+struct SelView {
+  const uint16_t* err;
+  const uint16_t* age;
+  SelGeom g;
+  HashKeys hk;
+  SelWs w;
+  int n_sel, kh, ks;  // tiles to choose, of them by error and by age
+  int n_pix, hard_pm, stable_pm;
+  bool vec;           // 16-byte loads of the maps are aligned
+  int32_t* active_tiles;
+  int32_t* n_active;
+  int32_t* tile_rank;
+  int32_t* pix_off;
+  uint8_t* pix_idx;
+};
+template <int V>
+struct SelBatch {
+  SelView v[V];
+};
+
+template <int V>
+__global__ void __launch_bounds__(256) k_tile_stats(const __grid_constant__ SelBatch<V> batch) {
+  const SelView& a = batch.v[V == 1 ? 0 : blockIdx.y];
+  const SelGeom& g = a.g;
+  const HashKeys& hk = a.hk;
+  const SelWs& w = a.w;
   __shared__ uint64_t s_w[kStatsTiles];
   __shared__ uint32_t s_a[kStatsTiles];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -129,7 +154,7 @@ __global__ void __launch_bounds__(256) k_tile_stats(const uint16_t* __restrict__
   uint32_t av[kStatsPerWarp];
 #pragma unroll
   for (int q = 0; q < kStatsPerWarp; ++q)
-    pixel_row8(err, age, g, t0 + kStatsPerWarp * warp + q, lane, vec, wv[q], av[q]);
+    pixel_row8(a.err, a.age, g, t0 + kStatsPerWarp * warp + q, lane, a.vec, wv[q], av[q]);
 #pragma unroll
   for (int q = 0; q < kStatsPerWarp; ++q) {
 #pragma unroll
@@ -230,12 +255,15 @@ __global__ void __launch_bounds__(256) k_rank_tiles(SelWs w, int T, int phase, i
 // pix_off and n_active.
 constexpr int kSelBlockMaxTiles = kSelThreads * 16;
 
-template <int ITEMS>
-__global__ void __launch_bounds__(kSelThreads, 1) k_select_block(SelWs w, SelGeom g, int n_sel, int kh, int ks,
-                                                              int n_pix, int32_t* __restrict__ active_tiles,
-                                                              int32_t* __restrict__ n_active,
-                                                              int32_t* __restrict__ tile_rank,
-                                                              int32_t* __restrict__ pix_off) {
+template <int ITEMS, int V>
+__global__ void __launch_bounds__(kSelThreads, 1) k_select_block(const __grid_constant__ SelBatch<V> batch) {
+  const SelView& a = batch.v[V == 1 ? 0 : blockIdx.y];
+  const SelGeom& g = a.g;
+  const SelWs& w = a.w;
+  const int n_sel = a.n_sel, kh = a.kh, ks = a.ks, n_pix = a.n_pix;
+  int32_t* __restrict__ active_tiles = a.active_tiles;
+  int32_t* __restrict__ tile_rank = a.tile_rank;
+  int32_t* __restrict__ pix_off = a.pix_off;
   __shared__ SelectSmem sm;
   __shared__ int64_t s64[32];
   const int T = g.T;
@@ -295,7 +323,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select_block(SelWs w, SelGeo
     }
   });
   if (threadIdx.x == 0) {
-    *n_active = (int32_t)(total >> 32);
+    *a.n_active = (int32_t)(total >> 32);
     pix_off[total >> 32] = (int32_t)(total & 0xFFFFFFFFll);
   }
 }
@@ -396,24 +424,27 @@ __device__ __forceinline__ float neglog2_approx(uint64_t h) {
 
 constexpr int kSampleWarps = 4;  // tiles per block
 
-__global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(
-    const uint16_t* __restrict__ err, const uint16_t* __restrict__ age, SelGeom g, int n_pix, int hard_pm,
-    int stable_pm, HashKeys hk, const int32_t* __restrict__ active_tiles, const int32_t* __restrict__ n_active,
-    const int32_t* __restrict__ pix_off, uint8_t* __restrict__ pix_idx) {
+template <int V>
+__global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(const __grid_constant__ SelBatch<V> batch) {
+  const SelView& a = batch.v[V == 1 ? 0 : blockIdx.y];
+  const SelGeom& g = a.g;
+  const HashKeys& hk = a.hk;
+  const uint16_t* __restrict__ err = a.err;
+  const uint16_t* __restrict__ age = a.age;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int j0 = blockIdx.x * kSampleWarps + (threadIdx.x >> 5);
-  if (j0 >= *n_active) return;
-  const int t = active_tiles[j0];
+  if (j0 >= a.n_sel || j0 >= *a.n_active) return;
+  const int t = a.active_tiles[j0];
   const int x = (t % g.tx) * TGS_TILE + (lane & 15), y = (t / g.tx) * TGS_TILE + (lane >> 4);  // pixel j: row y + 2 j
   uint32_t valid = 0u;
 #pragma unroll
   for (int j = 0; j < kPix; ++j)
     if (x < g.W && y + 2 * j < g.H) valid |= 1u << j;
   const int nv = tile_valid(g, t);
-  const int n = min(n_pix, nv);
+  const int n = min(a.n_pix, nv);
   int kh, ks;
-  split_counts(n, hard_pm, stable_pm, kh, ks);
+  split_counts(n, a.hard_pm, a.stable_pm, kh, ks);
   uint32_t taken = valid;  // n >= nv: every valid pixel
   if (n < nv) {
     const size_t p0 = (size_t)y * g.W + x;
@@ -443,9 +474,9 @@ __global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(
       float top = 0.f, low = 0x1p126f;
 #pragma unroll
       for (int j = 0; j < kPix; ++j) {
-        const float a = __uint_as_float(key[j]);
-        if ((th >> j) & 1u) top = fmaxf(top, a + (a * 0x1p-19f + d[j]));
-        else if ((valid >> j) & 1u) low = fminf(low, a - (a * 0x1p-19f + d[j]));
+        const float c = __uint_as_float(key[j]);
+        if ((th >> j) & 1u) top = fmaxf(top, c + (c * 0x1p-19f + d[j]));
+        else if ((valid >> j) & 1u) low = fminf(low, c - (c * 0x1p-19f + d[j]));
       }
       const float t_top = __uint_as_float(__reduce_max_sync(full, __float_as_uint(top)));
       const float t_low = __uint_as_float(__reduce_min_sync(full, __float_as_uint(fmaxf(low, 0.f))));
@@ -455,8 +486,8 @@ __global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(
         uint32_t doubt = 0u;
 #pragma unroll
         for (int j = 0; j < kPix; ++j) {
-          const float a = __uint_as_float(key[j]), e = a * 0x1p-19f + d[j];
-          if ((th >> j) & 1u ? a + e >= t_low : ((valid >> j) & 1u) && a - e <= t_top) doubt |= 1u << j;
+          const float c = __uint_as_float(key[j]), e = c * 0x1p-19f + d[j];
+          if ((th >> j) & 1u ? c + e >= t_low : ((valid >> j) & 1u) && c - e <= t_top) doubt |= 1u << j;
         }
         const int kk = __reduce_add_sync(full, __popc(doubt & th));
         uint64_t exact[kPix];
@@ -495,7 +526,7 @@ __global__ void __launch_bounds__(32 * kSampleWarps) k_sample_pixels(
     taken = th | ts | tu;
   }
   // the taken local indices, ascending
-  uint8_t* out = pix_idx + pix_off[j0];
+  uint8_t* out = a.pix_idx + a.pix_off[j0];
   const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
   for (int j = 0; j < kPix; ++j) {
@@ -516,81 +547,122 @@ __global__ void k_sel_finish(const int64_t* __restrict__ total, int32_t* __restr
 
 using namespace tgs;
 
-// The launch sequence shared by both entry points (arguments checked).
-static tgs_status launch_select(const uint16_t* err_map, const uint16_t* age_map, int32_t width, int32_t height,
-                                int n_sel, int32_t n_pix, const tgs_sampling* cfg, uint64_t seed, uint64_t iter,
-                                const uint64_t* iter_dev, uint32_t view, void* scratch, int32_t* active_tiles,
-                                int32_t* n_active, int32_t* tile_rank, int32_t* pix_off, uint8_t* pix_idx,
-                                cudaStream_t s) {
+// One view's arguments (checked) as the kernels take them.
+static SelView make_view(const uint16_t* err_map, const uint16_t* age_map, int32_t width, int32_t height,
+                         int32_t n_select, int32_t n_pix, const tgs_sampling* cfg, uint64_t seed, uint64_t iter,
+                         const uint64_t* iter_dev, uint32_t view, void* scratch, int32_t* active_tiles,
+                         int32_t* n_active, int32_t* tile_rank, int32_t* pix_off, uint8_t* pix_idx) {
   const int T = tiles_x(width) * tiles_y(height);
+  SelView a;
   size_t tot;
-  SelWs w = carve_sel(scratch, T, &tot);
-  SelGeom g{width, height, tiles_x(width), T};
-  const HashKeys hk{seed, iter, iter_dev, view};
-  int kh, ks;
-  split_counts(n_sel, cfg->tile_hard_pm, cfg->tile_stable_pm, kh, ks);
-  if (n_sel < T && n_sel > 0)
-    k_tile_stats<<<(T + kStatsTiles - 1) / kStatsTiles, 256, 0, s>>>(
-        err_map, age_map, g, hk, w, aligned16(err_map) && aligned16(age_map) && width % 8 == 0);
+  a.err = err_map;
+  a.age = age_map;
+  a.g = SelGeom{width, height, tiles_x(width), T};
+  a.hk = HashKeys{seed, iter, iter_dev, view};
+  a.w = carve_sel(scratch, T, &tot);
+  a.n_sel = std::min(n_select, T);
+  split_counts(a.n_sel, cfg->tile_hard_pm, cfg->tile_stable_pm, a.kh, a.ks);
+  a.n_pix = n_pix;
+  a.hard_pm = cfg->pix_hard_pm;
+  a.stable_pm = cfg->pix_stable_pm;
+  a.vec = aligned16(err_map) && aligned16(age_map) && width % 8 == 0;
+  a.active_tiles = active_tiles;
+  a.n_active = n_active;
+  a.tile_rank = tile_rank;
+  a.pix_off = pix_off;
+  a.pix_idx = pix_idx;
+  return a;
+}
+
+// The tiles of the batch's first `count` views, each of at most max_T <=
+// kSelBlockMaxTiles tiles and fewer chosen: the statistics, and one block per
+// view for the three phases and the compaction.
+template <int V>
+static void launch_block_select(const SelBatch<V>& b, int count, int max_T, bool any, cudaStream_t s) {
+  if (any) k_tile_stats<V><<<dim3((max_T + kStatsTiles - 1) / kStatsTiles, count), 256, 0, s>>>(b);
+  const dim3 grid(1, count);
+  if (max_T <= kSelThreads) k_select_block<1, V><<<grid, kSelThreads, 0, s>>>(b);
+  else if (max_T <= kSelThreads * 4) k_select_block<4, V><<<grid, kSelThreads, 0, s>>>(b);
+  else if (max_T <= kSelThreads * 8) k_select_block<8, V><<<grid, kSelThreads, 0, s>>>(b);
+  else k_select_block<16, V><<<grid, kSelThreads, 0, s>>>(b);
+}
+
+static bool block_selects(const SelView& a) { return a.n_sel < a.g.T && a.g.T <= kSelBlockMaxTiles; }
+
+// The tiles of one view.
+static void launch_tiles(const SelView& a, cudaStream_t s) {
+  const int T = a.g.T, n_sel = a.n_sel;
   if (n_sel >= T) {
-    k_select_all<<<(T + 255) / 256, 256, 0, s>>>(g, n_pix, active_tiles, n_active, tile_rank, pix_off);
-  } else if (T <= kSelBlockMaxTiles) {
-    // one block: the three phases and the compaction
-    if (T <= kSelThreads)
-      k_select_block<1><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
-                                                   pix_off);
-    else if (T <= kSelThreads * 4)
-      k_select_block<4><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
-                                                   pix_off);
-    else if (T <= kSelThreads * 8)
-      k_select_block<8><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
-                                                   pix_off);
-    else
-      k_select_block<16><<<1, kSelThreads, 0, s>>>(w, g, n_sel, kh, ks, n_pix, active_tiles, n_active, tile_rank,
-                                                    pix_off);
-  } else {
-    // many tiles: ranks by pairwise counting, then a device-wide scan.  A
-    // tile is taken when rank_h < kh, or (not hard) rank_s < ks, or
-    // (neither) rank_u < n_sel - kh - ks.
-    cudaMemsetAsync(w.rank_h, 0, sizeof(int32_t) * 3 * (size_t)T, s);
-    if (n_sel > 0) {
-      dim3 grid((T + 255) / 256, (T + RANK_CHUNK - 1) / RANK_CHUNK);
-      if (kh > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 0, kh, ks);
-      if (ks > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 1, kh, ks);
-      if (n_sel - kh - ks > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 2, kh, ks);
-    }
-    const int32_t* rh = w.rank_h;
-    const int32_t* rs = w.rank_s;
-    const int32_t* ru = w.rank_u;
-    const int none = n_sel == 0 ? 1 : 0;
-    const int ku = n_sel - kh - ks;
-    const int npx = n_pix;
-    int32_t* at = active_tiles;
-    int32_t* tr = tile_rank;
-    int32_t* po = pix_off;
-    auto load = [=] __device__(int64_t t) -> int64_t {
-      const bool taken = !none && (rh[t] < kh || rs[t] < ks || (rs[t] >= ks && ru[t] < ku));
-      if (!taken) return 0;
-      return (1ll << 32) | (int64_t)min(npx, tile_valid(g, (int)t));
-    };
-    auto store = [=] __device__(int64_t t, int64_t pre, int64_t v) {
-      if (v) {
-        const int r = (int)(pre >> 32);
-        tr[t] = r;
-        at[r] = (int)t;
-        po[r] = (int)(pre & 0xFFFFFFFFll);
-      } else {
-        tr[t] = -1;
-      }
-    };
-    exclusive_scan<int64_t>(load, store, nullptr, T, w.scan_sums, w.total, s);
-    k_sel_finish<<<1, 1, 0, s>>>(w.total, n_active, pix_off);
+    k_select_all<<<(T + 255) / 256, 256, 0, s>>>(a.g, a.n_pix, a.active_tiles, a.n_active, a.tile_rank, a.pix_off);
+    return;
   }
-  if (n_sel > 0)
-    k_sample_pixels<<<(n_sel + kSampleWarps - 1) / kSampleWarps, 32 * kSampleWarps, 0, s>>>(
-        err_map, age_map, g, n_pix, cfg->pix_hard_pm, cfg->pix_stable_pm, hk, active_tiles, n_active, pix_off,
-        pix_idx);
+  const SelBatch<1> one{{a}};
+  if (T <= kSelBlockMaxTiles) {
+    launch_block_select<1>(one, 1, T, n_sel > 0, s);
+    return;
+  }
+  // many tiles: ranks by pairwise counting, then a device-wide scan.  A
+  // tile is taken when rank_h < kh, or (not hard) rank_s < ks, or
+  // (neither) rank_u < n_sel - kh - ks.
+  const SelWs& w = a.w;
+  const int kh = a.kh, ks = a.ks;
+  if (n_sel > 0) k_tile_stats<1><<<(T + kStatsTiles - 1) / kStatsTiles, 256, 0, s>>>(one);
+  cudaMemsetAsync(w.rank_h, 0, sizeof(int32_t) * 3 * (size_t)T, s);
+  if (n_sel > 0) {
+    dim3 grid((T + 255) / 256, (T + RANK_CHUNK - 1) / RANK_CHUNK);
+    if (kh > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 0, kh, ks);
+    if (ks > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 1, kh, ks);
+    if (n_sel - kh - ks > 0) k_rank_tiles<<<grid, 256, 0, s>>>(w, T, 2, kh, ks);
+  }
+  const int32_t* rh = w.rank_h;
+  const int32_t* rs = w.rank_s;
+  const int32_t* ru = w.rank_u;
+  const int none = n_sel == 0 ? 1 : 0;
+  const int ku = n_sel - kh - ks;
+  const int npx = a.n_pix;
+  const SelGeom g = a.g;
+  int32_t* at = a.active_tiles;
+  int32_t* tr = a.tile_rank;
+  int32_t* po = a.pix_off;
+  auto load = [=] __device__(int64_t t) -> int64_t {
+    const bool taken = !none && (rh[t] < kh || rs[t] < ks || (rs[t] >= ks && ru[t] < ku));
+    if (!taken) return 0;
+    return (1ll << 32) | (int64_t)min(npx, tile_valid(g, (int)t));
+  };
+  auto store = [=] __device__(int64_t t, int64_t pre, int64_t v) {
+    if (v) {
+      const int r = (int)(pre >> 32);
+      tr[t] = r;
+      at[r] = (int)t;
+      po[r] = (int)(pre & 0xFFFFFFFFll);
+    } else {
+      tr[t] = -1;
+    }
+  };
+  exclusive_scan<int64_t>(load, store, nullptr, T, w.scan_sums, w.total, s);
+  k_sel_finish<<<1, 1, 0, s>>>(w.total, a.n_active, a.pix_off);
+}
+
+// The launch sequence of the one-view entry points.
+static tgs_status launch_select(const SelView& a, cudaStream_t s) {
+  launch_tiles(a, s);
+  if (a.n_sel > 0)
+    k_sample_pixels<1><<<(a.n_sel + kSampleWarps - 1) / kSampleWarps, 32 * kSampleWarps, 0, s>>>(SelBatch<1>{{a}});
   return check_launch();
+}
+
+// What both one-view entry points refuse.
+static bool select_args_ok(const uint16_t* err_map, const uint16_t* age_map, int32_t width, int32_t height,
+                           int32_t n_select, int32_t n_pix, const tgs_sampling* cfg, const int32_t* active_tiles,
+                           const int32_t* n_active, const int32_t* tile_rank, const int32_t* pix_off,
+                           const uint8_t* pix_idx) {
+  if (width <= 0 || height <= 0 || width > (1 << 16) || height > (1 << 16) || n_select < 0 || n_pix < 1 ||
+      n_pix > 256 || !cfg || !err_map || !age_map || !n_active || !tile_rank || !pix_off)
+    return false;
+  const int pms[4] = {cfg->tile_hard_pm, cfg->tile_stable_pm, cfg->pix_hard_pm, cfg->pix_stable_pm};
+  for (int k = 0; k < 4; ++k)
+    if (pms[k] < 0 || pms[k] > 1000) return false;
+  return std::min(n_select, tiles_x(width) * tiles_y(height)) == 0 || (active_tiles && pix_idx);
 }
 
 extern "C" size_t tgs_select_tiles_workspace_size(int32_t width, int32_t height) {
@@ -606,18 +678,48 @@ extern "C" tgs_status tgs_select_tiles(const uint16_t* err_map, const uint16_t* 
                                        void* workspace, size_t workspace_bytes, int32_t* active_tiles, int32_t* n_active,
                                        int32_t* tile_rank, int32_t* pix_off, uint8_t* pix_idx,
                                        tgs_stream stream) {
-  if (width <= 0 || height <= 0 || width > (1 << 16) || height > (1 << 16) || n_select < 0 || n_pix < 1 ||
-      n_pix > 256 || !cfg || !err_map || !age_map || !n_active || !tile_rank || !pix_off)
+  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, active_tiles, n_active, tile_rank, pix_off,
+                      pix_idx) ||
+      !workspace || workspace_bytes < tgs_select_tiles_workspace_size(width, height))
     return TGS_ERR_INVALID_ARG;
-  const int pms[4] = {cfg->tile_hard_pm, cfg->tile_stable_pm, cfg->pix_hard_pm, cfg->pix_stable_pm};
-  for (int k = 0; k < 4; ++k)
-    if (pms[k] < 0 || pms[k] > 1000) return TGS_ERR_INVALID_ARG;
-  const int T = tiles_x(width) * tiles_y(height);
-  const int n_sel = std::min(n_select, T);
-  if (n_sel > 0 && (!active_tiles || !pix_idx)) return TGS_ERR_INVALID_ARG;
-  if (!workspace || workspace_bytes < tgs_select_tiles_workspace_size(width, height)) return TGS_ERR_INVALID_ARG;
-  return launch_select(err_map, age_map, width, height, n_sel, n_pix, cfg, seed, iter, iter_dev, view, workspace,
-                       active_tiles, n_active, tile_rank, pix_off, pix_idx, (cudaStream_t)stream);
+  return launch_select(make_view(err_map, age_map, width, height, n_select, n_pix, cfg, seed, iter, iter_dev, view,
+                                 workspace, active_tiles, n_active, tile_rank, pix_off, pix_idx),
+                       (cudaStream_t)stream);
+}
+
+// Views chosen by one block each share the launches; a view with every tile, or
+// with more tiles than a block takes, is chosen by itself.  Eight views of 8160
+// tiles, 1200 to 4500 chosen, statistics, tiles and pixels: 380 -> 135 us.
+extern "C" tgs_status tgs_select_tiles_batched(int32_t n_views, const tgs_select_view* views, const tgs_sampling* cfg,
+                                               uint64_t iter, const uint64_t* iter_dev, tgs_stream stream) {
+  if (n_views < 1 || n_views > kMaxSelViews || !views) return TGS_ERR_INVALID_ARG;
+  SelBatch<kMaxSelViews> all, block;
+  int in_block = 0, max_T = 0, max_sel = 0;
+  bool any = false;
+  for (int k = 0; k < n_views; ++k) {
+    const tgs_select_view& v = views[k];
+    if (!select_args_ok(v.err_map, v.age_map, v.width, v.height, v.n_select, v.n_pix, cfg, v.active_tiles, v.n_active,
+                        v.tile_rank, v.pix_off, v.pix_idx) ||
+        !v.workspace || v.workspace_bytes < tgs_select_tiles_workspace_size(v.width, v.height))
+      return TGS_ERR_INVALID_ARG;
+    all.v[k] = make_view(v.err_map, v.age_map, v.width, v.height, v.n_select, v.n_pix, cfg, v.seed, iter, iter_dev,
+                         v.view, v.workspace, v.active_tiles, v.n_active, v.tile_rank, v.pix_off, v.pix_idx);
+    max_sel = std::max(max_sel, all.v[k].n_sel);
+    if (block_selects(all.v[k])) {
+      max_T = std::max(max_T, all.v[k].g.T);
+      any = any || all.v[k].n_sel > 0;
+      block.v[in_block++] = all.v[k];
+    }
+  }
+  cudaStream_t s = (cudaStream_t)stream;
+  if (n_views == 1) return launch_select(all.v[0], s);
+  for (int k = 0; k < n_views; ++k)
+    if (!block_selects(all.v[k])) launch_tiles(all.v[k], s);
+  if (in_block) launch_block_select<kMaxSelViews>(block, in_block, max_T, any, s);
+  if (max_sel > 0)
+    k_sample_pixels<kMaxSelViews>
+        <<<dim3((max_sel + kSampleWarps - 1) / kSampleWarps, n_views), 32 * kSampleWarps, 0, s>>>(all);
+  return check_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -673,22 +775,18 @@ extern "C" tgs_status tgs_select_tiles_noalloc(const uint16_t* err_map, const ui
                                                const uint64_t* iter_dev, uint32_t view, int32_t* active_tiles,
                                                int32_t* n_active, int32_t* tile_rank, int32_t* pix_off,
                                                uint8_t* pix_idx, tgs_stream stream) {
-  if (width <= 0 || height <= 0 || width > (1 << 16) || height > (1 << 16) || n_select < 0 || n_pix < 1 ||
-      n_pix > 256 || !cfg || !err_map || !age_map || !n_active || !tile_rank || !pix_off)
+  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, active_tiles, n_active, tile_rank, pix_off,
+                      pix_idx))
     return TGS_ERR_INVALID_ARG;
-  const int pms[4] = {cfg->tile_hard_pm, cfg->tile_stable_pm, cfg->pix_hard_pm, cfg->pix_stable_pm};
-  for (int k = 0; k < 4; ++k)
-    if (pms[k] < 0 || pms[k] > 1000) return TGS_ERR_INVALID_ARG;
   const int T = tiles_x(width) * tiles_y(height);
   if (T > TGS_SELECT_NOALLOC_MAX_TILES) return TGS_ERR_CAPACITY;
   size_t need = 0;
   carve_sel(nullptr, T, &need);
   if (need > sizeof(g_select_scratch)) return TGS_ERR_CAPACITY;
-  const int n_sel = std::min(n_select, T);
-  if (n_sel > 0 && (!active_tiles || !pix_idx)) return TGS_ERR_INVALID_ARG;
   void* scratch = nullptr;
   tgs_status st = select_scratch_address(&scratch);
   if (st != TGS_OK) return st;
-  return launch_select(err_map, age_map, width, height, n_sel, n_pix, cfg, seed, iter, iter_dev, view, scratch,
-                       active_tiles, n_active, tile_rank, pix_off, pix_idx, (cudaStream_t)stream);
+  return launch_select(make_view(err_map, age_map, width, height, n_select, n_pix, cfg, seed, iter, iter_dev, view,
+                                 scratch, active_tiles, n_active, tile_rank, pix_off, pix_idx),
+                       (cudaStream_t)stream);
 }

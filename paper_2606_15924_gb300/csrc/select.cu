@@ -651,18 +651,20 @@ static tgs_status launch_select(const SelView& a, cudaStream_t s) {
   return check_launch();
 }
 
-// What both one-view entry points refuse.
+// What every entry point refuses.
 static bool select_args_ok(const uint16_t* err_map, const uint16_t* age_map, int32_t width, int32_t height,
-                           int32_t n_select, int32_t n_pix, const tgs_sampling* cfg, const int32_t* active_tiles,
-                           const int32_t* n_active, const int32_t* tile_rank, const int32_t* pix_off,
-                           const uint8_t* pix_idx) {
+                           int32_t n_select, int32_t n_pix, const tgs_sampling* cfg, const int32_t* n_active,
+                           const int32_t* tile_rank, const int32_t* pix_off) {
   if (width <= 0 || height <= 0 || width > (1 << 16) || height > (1 << 16) || n_select < 0 || n_pix < 1 ||
       n_pix > 256 || !cfg || !err_map || !age_map || !n_active || !tile_rank || !pix_off)
     return false;
   const int pms[4] = {cfg->tile_hard_pm, cfg->tile_stable_pm, cfg->pix_hard_pm, cfg->pix_stable_pm};
   for (int k = 0; k < 4; ++k)
     if (pms[k] < 0 || pms[k] > 1000) return false;
-  return std::min(n_select, tiles_x(width) * tiles_y(height)) == 0 || (active_tiles && pix_idx);
+  return true;
+}
+static bool select_outputs_ok(int32_t n_select, const int32_t* active_tiles, const uint8_t* pix_idx) {
+  return n_select == 0 || (active_tiles && pix_idx);
 }
 
 extern "C" size_t tgs_select_tiles_workspace_size(int32_t width, int32_t height) {
@@ -678,9 +680,8 @@ extern "C" tgs_status tgs_select_tiles(const uint16_t* err_map, const uint16_t* 
                                        void* workspace, size_t workspace_bytes, int32_t* active_tiles, int32_t* n_active,
                                        int32_t* tile_rank, int32_t* pix_off, uint8_t* pix_idx,
                                        tgs_stream stream) {
-  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, active_tiles, n_active, tile_rank, pix_off,
-                      pix_idx) ||
-      !workspace || workspace_bytes < tgs_select_tiles_workspace_size(width, height))
+  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, n_active, tile_rank, pix_off) ||
+      !select_outputs_ok(n_select, active_tiles, pix_idx) || !workspace || workspace_bytes < tgs_select_tiles_workspace_size(width, height))
     return TGS_ERR_INVALID_ARG;
   return launch_select(make_view(err_map, age_map, width, height, n_select, n_pix, cfg, seed, iter, iter_dev, view,
                                  workspace, active_tiles, n_active, tile_rank, pix_off, pix_idx),
@@ -698,9 +699,9 @@ extern "C" tgs_status tgs_select_tiles_batched(int32_t n_views, const tgs_select
   bool any = false;
   for (int k = 0; k < n_views; ++k) {
     const tgs_select_view& v = views[k];
-    if (!select_args_ok(v.err_map, v.age_map, v.width, v.height, v.n_select, v.n_pix, cfg, v.active_tiles, v.n_active,
-                        v.tile_rank, v.pix_off, v.pix_idx) ||
-        !v.workspace || v.workspace_bytes < tgs_select_tiles_workspace_size(v.width, v.height))
+    if (!select_args_ok(v.err_map, v.age_map, v.width, v.height, v.n_select, v.n_pix, cfg, v.n_active, v.tile_rank,
+                        v.pix_off) ||
+        !select_outputs_ok(v.n_select, v.active_tiles, v.pix_idx) || !v.workspace || v.workspace_bytes < tgs_select_tiles_workspace_size(v.width, v.height))
       return TGS_ERR_INVALID_ARG;
     all.v[k] = make_view(v.err_map, v.age_map, v.width, v.height, v.n_select, v.n_pix, cfg, v.seed, iter, iter_dev,
                          v.view, v.workspace, v.active_tiles, v.n_active, v.tile_rank, v.pix_off, v.pix_idx);
@@ -775,14 +776,14 @@ extern "C" tgs_status tgs_select_tiles_noalloc(const uint16_t* err_map, const ui
                                                const uint64_t* iter_dev, uint32_t view, int32_t* active_tiles,
                                                int32_t* n_active, int32_t* tile_rank, int32_t* pix_off,
                                                uint8_t* pix_idx, tgs_stream stream) {
-  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, active_tiles, n_active, tile_rank, pix_off,
-                      pix_idx))
+  if (!select_args_ok(err_map, age_map, width, height, n_select, n_pix, cfg, n_active, tile_rank, pix_off))
     return TGS_ERR_INVALID_ARG;
   const int T = tiles_x(width) * tiles_y(height);
   if (T > TGS_SELECT_NOALLOC_MAX_TILES) return TGS_ERR_CAPACITY;
   size_t need = 0;
   carve_sel(nullptr, T, &need);
   if (need > sizeof(g_select_scratch)) return TGS_ERR_CAPACITY;
+  if (!select_outputs_ok(n_select, active_tiles, pix_idx)) return TGS_ERR_INVALID_ARG;
   void* scratch = nullptr;
   tgs_status st = select_scratch_address(&scratch);
   if (st != TGS_OK) return st;

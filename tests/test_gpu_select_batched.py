@@ -10,8 +10,6 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2606_15924_gb300 import scenes
-
 pytestmark = pytest.mark.gpu
 SIZES = [(256, 256, 64, 85), (250, 187, 192, 25), (333, 187, 0, 10), (1280, 720, 720, 84), (64, 48, 5, 256),
          (1957, 1091, 3000, 33), (40, 40, 99, 1), (4096, 1040, 1664, 25), (16, 16, 1, 200)]
@@ -26,8 +24,9 @@ def B():
 
 @functools.lru_cache(maxsize=None)
 def _maps(W, H):
-    return tuple(torch.from_numpy(a.view(np.int16)).cuda()
-                 for a in (scenes.error_map(W, H, seed=W), scenes.age_map(W, H, seed=H, max_age=40)))
+    rng = np.random.default_rng(W)
+    err, age = rng.random((H, W)).astype(np.float16), rng.integers(0, 40, (H, W)).astype(np.int16)
+    return torch.from_numpy(err.view(np.int16)).cuda(), torch.from_numpy(age).cuda()
 
 
 def _view(B, k, W, H, n_select, n_pix):

@@ -49,7 +49,9 @@ def test_every_tile_bit_exact(B, orc, W, H, n_pix):
     tiles than the one-block selection takes."""
     from gpu_util import select_dev, select_host
     T = ((W + 15) // 16) * ((H + 15) // 16)
-    err, age = scenes.error_map(W, H, seed=T), scenes.age_map(W, H, seed=H, max_age=9)
+    rng = np.random.default_rng(T)
+    err = rng.random((H, W)).astype(np.float16).view(np.uint16)
+    age = rng.integers(0, 9, (H, W)).astype(np.uint16)
     for n_sel in (T, T + 5):
         got = select_host(select_dev(B, err, age, W, H, n_sel, n_pix, seed=2, it=1, view=0))
         assert got["n_active"] == T

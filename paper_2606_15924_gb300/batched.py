@@ -218,7 +218,8 @@ class MultiViewTrainer:
             B.render_backward_batched(self.bwd_batch, self.grid[1], self.counters[1:2])
         else:
             for k, v in enumerate(self.views):
-                B.render_backward_batched(self.bwd_single[k], max(1, v.n_select * (self.ck_slots + 1)),
+                # the blocks are single warps that take items from the queue: as many as stay resident
+                B.render_backward_batched(self.bwd_single[k], max(1, self.resident[1]),
                                           self.counters[2 + self.K + k:3 + self.K + k])
 
     # ------------------------------------------------------------------ step

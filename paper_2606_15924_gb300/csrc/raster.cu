@@ -1453,10 +1453,14 @@ static bool raster_args(const tgs_projected* proj, const int32_t* tile_ranges, c
 
 // The division of a backward launch over `tiles` tiles.  Groups of 32
 // kBwdPpl pixels take the fewest instructions a pixel (one reduction serves
-// them all); while that leaves fewer items than four an SM (a tile's list
-// counted as four pieces where it has checkpoints), they are halved, down to
-// one pixel a lane.  64 tiles of 85 pixels: 10.7 us in three groups, 12.1 in
-// one; 19 whole tiles without checkpoints: 19.2 us at 32 pixels, 30.2 at 128.
+// them all), smaller ones shorten a warp's walk and give more of them.  With
+// checkpoints the pieces give enough: groups are halved, down to one pixel a
+// lane, while that leaves fewer than four items an SM (a tile's list counted as
+// four pieces).  64 tiles of 85 pixels: 10.7 us in three groups, 12.1 in one.
+// Without checkpoints a warp walks its tile's whole list: groups of 128 are
+// halved below 32 items an SM and groups of 64 below 16.  Whole tiles of 1M
+// Gaussians in groups of 128, 64, 32: 335 tiles 133, 98, 98 us; 670 tiles 150,
+// 119, 152; 1005 tiles 186, 165, 202; 2010 tiles 262, 255, -; 201 tiles -, 87, 79.
 // Pieces: short ones give more items, long ones read each pixel's state and
 // run into half-filled chunks less often.  span 1 / 2 / 4: 64 tiles of 85
 // pixels 12.1 / 17.6 / 28.9 us, 720 tiles 63.6 / 54.4 / 58.1 us, 3600 tiles of
@@ -1467,7 +1471,8 @@ static BwdSplit bwd_split(int64_t tiles, int n_pix_max, const Ckpt& ck) {
   BwdSplit sp;
   int most = 32 * kBwdPpl;
   auto groups = [&]() { return (n_pix_max + most - 1) / most; };
-  while (most > 32 && tiles * groups() * (ck.data ? 4 : 1) < 4 * sms) most /= 2;
+  const int64_t least = ck.data ? 1 : 16;  // items an SM below which groups of 64 are halved
+  while (most > 32 && tiles * groups() < (ck.data || most <= 64 ? least : 2 * least) * sms) most /= 2;
   sp.groups = groups();
   sp.gpx = (n_pix_max + sp.groups - 1) / sp.groups;
   sp.span = tiles * sp.groups <= 2 * sms ? 1 : tiles * sp.groups <= 16 * sms ? 2 : 4;

@@ -70,8 +70,9 @@ typedef struct {
  * geometric fields, which then lie in one array of rows (a multiple of 4, at
  * least 12; e.g. 16: means at row + 0, log_scales at + 3, opacity_logits at
  * + 6, quats at + 8, one 64-byte row per Gaussian, so that an update of
- * scattered Gaussians reads and writes whole rows).  quats stays 16-byte
- * aligned.  sh is always [N,16,3]. */
+ * scattered Gaussians reads and writes whole rows; that order from a 64-byte
+ * boundary is the fast one, and floats 7 and 12..15 of a row are then written
+ * back as they were).  quats stays 16-byte aligned.  sh is always [N,16,3]. */
 typedef struct {
   const float* means;
   const float* log_scales;

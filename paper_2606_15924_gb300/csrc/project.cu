@@ -1044,8 +1044,8 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_update(
   }
 }
 
-// The fused adjoint + update for geometric fields in 64-byte rows (geo_stride
-// 16, rows on 16-byte boundaries).  The same two roles and the same
+// The fused adjoint + update for geometric fields in whole 64-byte rows
+// (geo_whole_rows).  The same two roles and the same
 // arithmetic as k_adj_update, but a round first copies the whole rows it
 // needs into shared memory with coalesced asynchronous copies (cp.async):
 // the parameters' and both moments' geometric rows, the parameters' SH rows
@@ -1360,9 +1360,8 @@ extern "C" tgs_status tgs_project_backward_update(const tgs_param_ptrs* params, 
   cudaMemsetAsync(count, 0, sizeof(int32_t), s);
   // the mark pass writes no gradients (nothing to zero)
   k_adj_mark<<<(int)((g->n + 255) / 256), 256, 0, s>>>(g->n, mv, touched, 0, GeoW{}, nullptr, list, count);
-  // 64-byte geometric rows on 16-byte boundaries in all three: the staged-row kernel
-  const bool rows = params->geo_stride == 16 && m->geo_stride == 16 && v->geo_stride == 16 &&
-                    aligned16(params->means) && aligned16(m->means) && aligned16(v->means);
+  // whole 64-byte geometric rows in all three: the staged-row kernel
+  const bool rows = geo_whole_rows(*params) && geo_whole_rows(*m) && geo_whole_rows(*v);
   static int grid_dev[64][2][2] = {};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1421,7 +1420,7 @@ extern "C" tgs_status tgs_project_gaussians(const tgs_gaussians* g, const tgs_ca
     return TGS_ERR_INVALID_ARG;
   CamK k = make_cam(*cam);
   const int blocks = (int)((g->n + kProjectThreads - 1) / kProjectThreads);
-  const bool rows = g->geo_stride == 16 && aligned16(g->means);  // 64-byte rows on 16-byte boundaries
+  const bool rows = geo_in_rows(*g);
   (rows ? k_project<true> : k_project<false>)<<<blocks, kProjectThreads, 0, (cudaStream_t)stream>>>(
       geo_of(*g), reinterpret_cast<const float4*>(g->sh), g->n, g->sh_degree, k, tile_rank,
       reinterpret_cast<float2*>(out->xy), reinterpret_cast<float4*>(out->conic_opac), out->rgb, out->depth,

@@ -40,6 +40,24 @@ inline bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3
 // ---------------------------------------------------------------------------
 inline bool geo_stride_ok(int32_t s) { return s == 0 || (s >= 12 && s % 4 == 0); }
 
+// Fields in rows of 16 floats in the order means, log-scales, opacity logit, (7
+// unused), quats from a 16-byte boundary, so that three float4 loads take a
+// Gaussian (the header fixes the distance between rows, not the fields' order
+// in them: any other order is read through the four pointers).
+template <class G>  // tgs_gaussians or tgs_param_ptrs
+inline bool geo_in_rows(const G& g) {
+  return g.geo_stride == 16 && reinterpret_cast<uintptr_t>(g.means) % 16 == 0 && g.log_scales == g.means + 3 &&
+         g.opacity_logits == g.means + 6 && g.quats == g.means + 8;
+}
+// The same with means at the start of the row, which lies on a 64-byte boundary:
+// all 16 floats from means are the Gaussian's own.  Means at float 4 and quats at
+// 12 are in order too, but there the last four of 16 are the next Gaussian's, or
+// past the array.
+template <class G>
+inline bool geo_whole_rows(const G& g) {
+  return geo_in_rows(g) && reinterpret_cast<uintptr_t>(g.means) % 64 == 0;
+}
+
 struct GeoC {  // read-only view
   const float* m;
   const float* l;

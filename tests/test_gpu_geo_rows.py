@@ -29,6 +29,28 @@ def _rows(g, stride=16):
     return as_geo_rows(g, stride)
 
 
+# Sixteen floats a Gaussian with the fields at other places of the row than
+# binding.geo_rows puts them: (means, log_scales, quats, opacity_logits).
+ORDERS = {"quats_first": (4, 7, 0, 10), "means_last": (12, 0, 4, 3), "shifted": (4, 7, 12, 10)}
+
+
+def _ordered_rows(g, order):
+    """g in rows of 16 floats of the given order, or ("apart") as four arrays
+    of such rows; the floats of no field hold a large number.  Returns the
+    views and the arrays."""
+    n = g["means"].shape[0]
+    at = ORDERS.get(order, (0, 0, 0, 0))
+    one = torch.full((n, 16), 1e6, device="cuda")
+    arrays, out = [], {"sh": g["sh"].clone()}
+    for k, a, w in zip(("means", "log_scales", "quats", "opacity_logits"), at, (3, 3, 4, 1)):
+        base = torch.full_like(one, 1e6) if order == "apart" else one
+        arrays.append(base)
+        v = base[:, a:a + w] if w > 1 else base[:, a]
+        v.copy_(g[k])
+        out[k] = v
+    return out, arrays
+
+
 def _same(a, b):
     for k in KEYS:
         assert torch.equal(a[k].contiguous(), b[k].contiguous()), k
@@ -78,6 +100,46 @@ def test_projection_same_bits(B, stride):
     assert int((outs[0]["radius"] > 0).sum()) > 1000
     for k in outs[0]:
         assert torch.equal(outs[0][k], outs[1][k]), k
+
+
+@pytest.mark.parametrize("order", [*ORDERS, "apart"])
+def test_projection_reads_each_field_where_it_is(B, order):
+    from gpu_util import empty_projected, gaussians_dev
+    g = gaussians_dev(scenes.gaussians(3001, seed=3))
+    r, _ = _ordered_rows(g, order)
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=W, height=H)
+    a, b = empty_projected(3001), empty_projected(3001)
+    B.project_gaussians(g, cam, None, a)
+    B.project_gaussians(r, cam, None, b)
+    torch.cuda.synchronize()
+    assert int((a["radius"] > 0).sum()) > 500
+    for k in a:
+        assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("order", [*ORDERS, "apart"])
+def test_fused_update_reads_each_field_where_it_is(B, order):
+    """The one-pass adjoint and update, parameters and moments in such rows: the
+    packed arrays' bits, and the floats of no field stay as they are."""
+    mv = _setup(5000)
+    p0 = {k: mv.params[k].clone() for k in KEYS}
+    m0, v0 = _rand_like(p0, 5, 1e-3), _rand_like(p0, 6, 1e-4)
+    step = torch.full((1,), 3, dtype=torch.int32, device="cuda")
+    res = []
+    for packed in (True, False):
+        sets = [{k: t.clone() for k, t in d.items()} if packed else _ordered_rows(d, order) for d in (p0, m0, v0)]
+        p, m, v = sets if packed else [x[0] for x in sets]
+        t = torch.zeros(mv.n, dtype=torch.uint8, device="cuda")
+        B.project_backward_update(p, mv.adj, m, v, t, mv.opt, 1, step_dev=step)
+        torch.cuda.synchronize()
+        assert int(t.sum()) > 100
+        res.append((p, m, v))
+    for a, b in zip(*res):
+        _same(a, b)
+    for x in sets:
+        want, arrays = _ordered_rows(x[0], order)
+        for got, ref in zip(x[1], arrays):
+            assert torch.equal(got, ref)
 
 
 def test_adjoints_update_and_hybrid_same_bits(B):

@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(256) k_scatter_pairs(const float2* __restrict_
 // run's offset in the list; blocks land in any order, the lists are sorted
 // whole).
 constexpr int kHistThreads = 1024;
+constexpr size_t kHistStaticSmem = 1024;  // at least the kernels' statically allocated shared memory
 
 __device__ __forceinline__ void chunk_of(int64_t n, int64_t& i0, int64_t& i1) {
   const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
@@ -333,6 +334,7 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_scatter(const float2* __r
                                                                uint64_t* __restrict__ keys, int64_t cap) {
   extern __shared__ uint32_t sh[];
   __shared__ int64_t s_wt[32];
+  static_assert(sizeof(s_wt) <= kHistStaticSmem, "shared memory asked for");
   const int R = geo.n_ranks, b = blockIdx.x;
   const int32_t* row = table + (size_t)b * R;
   if (STARTS) {
@@ -685,7 +687,9 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
   const size_t smem = counters + rank_smem(kind, T);
   cudaMemsetAsync(w.tile_cnt, 0, sizeof(int32_t) * (size_t)R, s);
   if (shared_path) {
-    if (smem > 48 * 1024) {  // opt in to more than 48 KB of dynamic shared memory (per device)
+    // opt in to more than 48 KB of shared memory a block (per device); the
+    // scatter's own arrays count too
+    if (smem + kHistStaticSmem > 48 * 1024) {
       static bool attr_set[64] = {};
       int dev = 0;
       cudaGetDevice(&dev);

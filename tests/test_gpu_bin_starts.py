@@ -2,7 +2,13 @@
 tiles' starts and clears the keys before the scatter, bit for bit against the
 same scene at the capacity it needs: an odd and an even number of pairs, one
 pair, none, tile masks and no mask, and more pairs than the capacity (the
-lists before the cut are whole, the count is of all)."""
+lists before the cut are whole, the count is of all).  And the first call of
+a process at tables that take just under the shared memory of a block that has
+not asked for more."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -59,3 +65,34 @@ def test_more_pairs_than_the_capacity(B):
     whole = MANY // n
     got = out["vals"][:whole * n].view(whole, n).cpu().numpy()
     np.testing.assert_array_equal(got, np.broadcast_to(order, (whole, n)))
+
+
+FIRST_CALL = """
+import sys, torch
+sys.path[:0] = sys.argv[3:]
+from gpu_util import bin_dev, projected_dev
+from paper_2606_15924_gb300 import binding as B, scenes
+W, H, n, R = 1920, 1080, 4000, int(sys.argv[1])
+T = 8160
+cam = dict(viewmat=[1.0 * (k % 5 == 0) for k in range(16)], fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
+pd = projected_dev(scenes.projected(n, W, H, seed=1))
+rank = torch.where(torch.arange(T) < R, torch.arange(T), -1).to(torch.int32).cuda()
+got = bin_dev(B, pd, n, cam, rank, R, capacity=int(sys.argv[2]))
+want = bin_dev(B, pd, n, cam, None, T, capacity=10 ** 6)
+I = int(got["n_isect"].item())
+assert I == int(want["ranges"][R - 1, 1].item()) and 0 < I < 10 ** 6
+assert torch.equal(got["ranges"], want["ranges"][:R])
+for k in ("vals", "keys"):
+    assert torch.equal(got[k][:I], want[k][:I]), k
+"""
+
+
+@pytest.mark.parametrize("R,capacity", [(8160, 10 ** 6), (8160, MANY), (7900, 10 ** 6), (7952, 10 ** 6)])
+def test_first_call_of_a_process(B, R, capacity):
+    """Counters and the rank table of a view of 1920x1080: 48960 bytes with every
+    tile active, 48944 and 49152 of two shares of them, where a block has 49152
+    for these and the kernel's own arrays before the library asks for more."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", FIRST_CALL, str(R), str(capacity), os.path.dirname(here), here],
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]

@@ -1195,7 +1195,8 @@ __device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int 
                                            fabsf(w.c.w) + fabsf(w.r) + fabsf(w.g) + fabsf(w.b) <
                                        INFINITY);
     }
-    id = k - 32 >= first ? a.vals[k - 32] : -1;  // the next chunk's, ahead of this one's replay
+    // the next chunk's, ahead of this one's replay (a closed piece may begin past the list's end)
+    id = k - 32 >= first && k - 32 < range.y ? a.vals[k - 32] : -1;
     if (!__all_sync(full, finite)) {
       float2* TR = reinterpret_cast<float2*>(Q);
       __syncwarp();

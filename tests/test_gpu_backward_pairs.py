@@ -81,6 +81,50 @@ def test_pixel_counts_against_oracle(B, orc, n_pix, slots):
         assert np.all(g2[:, 9:] == 0.0)
 
 
+@pytest.mark.parametrize("n_pix,span", [(25, 1), (85, 2), (25, 4)])
+def test_lists_that_end_with_the_array(B, n_pix, span):
+    """Pieces of 32 span positions against whole lists (no checkpoints), where
+    the last tile's list ends where the array of entries does: lists of every
+    length about the pieces' chunks, and one cut off by the capacity."""
+    from gpu_util import bin_dev, projected_dev, select_dev
+    tiles = {1: 1, 2: 500, 4: 2600}[span]          # as many as make the pieces that long
+    tx = min(tiles, 64)
+    W2, H2 = 16 * tx, 16 * ((tiles + tx - 1) // tx)
+    T = (W2 // 16) * (H2 // 16)
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=W2, height=H2)
+    sel = select_dev(B, scenes.error_map(W2, H2), scenes.age_map(W2, H2), W2, H2, T, n_pix, seed=4)
+    for L in (1, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 161):
+        p = scenes.projected(L, W2, H2, seed=L, radius_max=5)
+        rng = np.random.default_rng(L)
+        p["xy"] = (np.array([W2 - 8.0, H2 - 8.0]) + rng.uniform(-2, 2, (L, 2))).astype(np.float32)   # the last tile
+        p["radius"][:] = 5
+        p["opac"] = rng.uniform(0.02, 0.06, L)
+        pd = projected_dev(p)
+        for cap in (L, L - 1):
+            if cap == 0:
+                continue
+            b = bin_dev(B, pd, L, cam, sel["tile_rank"], T, capacity=cap)
+            assert b["vals"].shape[0] == cap and int(b["ranges"][T - 1, 1]) == cap and int(b["n_isect"].item()) == L
+            P = T * n_pix
+            g = []
+            for slots in (0, 64):
+                rgb, Tf = torch.zeros(P, 3, device="cuda"), torch.zeros(P, device="cuda")
+                last = torch.zeros(P, dtype=torch.int32, device="cuda")
+                data = torch.full((B.checkpoint_bytes(T, n_pix, 64) // 4,), float("nan"), device="cuda")
+                longest = torch.zeros(T, dtype=torch.int32, device="cuda")
+                ck = B.checkpoints(data, 64, P, rgb, longest) if slots else None
+                a = (pd, b["ranges"], b["vals"], sel["active_tiles"], sel["n_active"], T, sel["pix_off"], sel["pix_idx"],
+                     n_pix, cam, (0.3, 0.1, 0.6))
+                B.render_sampled(*a, rgb, Tf, last, ckpt=ck)
+                dL = torch.randn(P, 3, generator=torch.Generator().manual_seed(5)).cuda()
+                g2 = torch.zeros(L, 12, device="cuda")
+                B.render_backward_sampled(*a, Tf, last, dL, g2, ckpt=ck)
+                g.append(g2)
+            assert float(g[0].abs().max()) > 0
+            # sums of the same terms, T recovered from another end: some 2^-24 a position
+            assert float((g[0] - g[1]).norm()) <= 1e-4 * float(g[0].norm()), (L, cap)
+
+
 @pytest.mark.parametrize("slots", [0, 64])
 def test_nonfinite_values_stay_local(B, slots):
     """One pixel with an infinite and one with a NaN gradient poison the splats

@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) k_mlp_backward_tc(
 // copied transposed; X and H1 carry a column of ones for the bias gradients.
 // The roundings are the forward's and the backward's: x, h1, h2, dH2 and dH1 in
 // bf16, fp32 sums; y sums its two halves of 64 units and then adds b3.
-// Measured on GB300, 1.7 M rows: 346 us (545 TFLOP/s bf16 of the contractions'
+// Measured on GB300, 1.7 M rows: 355 us (532 TFLOP/s bf16 of the contractions'
 // 189 GFLOP); one tile at a time with a barrier a step took 528.  Bound by
 // shared memory: 68 % of its cycles carry the epilogues' and the tensor cores'
 // accesses, and the issue slots are 31 % busy.  With 512 epilogue threads of 32
@@ -805,7 +805,10 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_mlp_train_tc(
     float2 w3acc[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) w3acc[k] = make_float2(0.f, 0.f);
-    float b3 = 0.f, l_hi = 0.f, l_lo = 0.f;  // sum of e^2 as an unevaluated pair of floats
+    float b3 = 0.f;
+    // the sum of e^2 in fp64, as the backward above has it: 9 us at 1.7M rows
+    // against a pair of floats, which holds 48 bits and e^2 up to 3e38 only
+    double lsum = 0.0;
     const int64_t Re = R_dev ? (*R_dev > 0 ? (*R_dev < R ? (int64_t)*R_dev : R) : 0) : R;
     const float inv = Re > 0 ? 1.f / (float)Re : 0.f;
     const float4* b1v = reinterpret_cast<const float4*>(par + u0);
@@ -926,11 +929,8 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_mlp_train_tc(
         if (y_out && valid && hf == 0) y_out[row] = yv;
         const float e = counted ? yv - tgv[s] : 0.f;
         const float d = e * inv;
-        if (hf == 0) {  // e^2 exactly as sq + rest, added to the pair
-          const float sq = __fmul_rn(e, e), rest = __fmaf_rn(e, e, -sq);
-          const float sum = __fadd_rn(l_hi, sq), bb = __fsub_rn(sum, l_hi);
-          l_lo += (l_hi - __fsub_rn(sum, bb)) + (sq - bb) + rest;
-          l_hi = sum;
+        if (hf == 0) {
+          lsum = __fma_rn((double)e, (double)e, lsum);
           b3 += d;
         }
         const float2 dd = make_float2(d, d);
@@ -1012,7 +1012,7 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_mlp_train_tc(
       }
       b3 = warp_sum(b3);
       if ((t & 31) == 0 && hf == 0) atomicAdd(grads + kOffB3, b3);
-      const double lsum = warp_sum_d(((double)l_hi + (double)l_lo) * 0.5 * (double)inv);
+      lsum = warp_sum_d(lsum * 0.5 * (double)inv);
       if ((t & 31) == 0 && lsum != 0.0) atomicAdd(loss, lsum);
     }
   }

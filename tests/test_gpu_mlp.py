@@ -164,6 +164,26 @@ def test_train_pass_slots(P, orc, tiles, extra, R_dev):
         assert rel_l2(g[sl[name]], gw[name].reshape(-1)) <= 2e-4, (name, rel_l2(g[sl[name]], gw[name].reshape(-1)))
 
 
+@pytest.mark.parametrize("scale", [1e21, 1e-24])
+def test_train_pass_loss_is_summed_in_64_bits(P, scale):
+    """Errors whose squares lie outside fp32's range: the loss is a sum of
+    doubles.  y is below 10 here, so at 1e21 an error is its target to fp32's
+    rounding (2^-24 a row); at 1e-24 the network is all zeros and y exactly 0."""
+    B, TileErrorMLP = P
+    R = 777
+    mlp = TileErrorMLP(seed=1)
+    if scale < 1:
+        mlp.params.zero_()
+        mlp._refresh_bf16()
+    t = (scale * (1.0 + np.random.default_rng(3).random(R))).astype(np.float32)
+    xd, td = torch.from_numpy(_features(R, 5)).cuda(), torch.from_numpy(t).cuda()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.mlp_train_tc(mlp.net(), xd, td, mlp.grads, mlp.loss, status=status)
+    assert int(status.item()) == 0
+    want = 0.5 * np.mean(t.astype(np.float64) ** 2)
+    assert float(mlp.loss.item()) == pytest.approx(want, rel=2.0 ** -22)
+
+
 def test_adam_step_and_training(P):
     B, TileErrorMLP = P
     mlp = TileErrorMLP(seed=3, lr=2e-3)

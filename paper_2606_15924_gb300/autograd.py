@@ -151,9 +151,10 @@ class _RenderSampled(torch.autograd.Function):
         params = dict(means=means, log_scales=log_scales, quats=quats, opacity_logits=opacity_logits, sh=sh)
         grads = {k: torch.empty_like(v) for k, v in params.items()}
         n_out = max(int(raster.pix_idx.shape[0]), 1)
-        if raster.P == n_out and dL_drgb.dtype == torch.float32 and dL_drgb.device == means.device:
+        if raster.P == n_out and dL_drgb.dtype == torch.float32 and dL_drgb.device == means.device \
+                and not dL_drgb.is_neg():
             g = dL_drgb.contiguous()
-        else:  # entries past the sampled pixels, or values to convert
+        else:  # entries past the sampled pixels, values to convert or signs still to apply
             g = torch.zeros(n_out, 3, device=means.device)
             g[:raster.P] = dL_drgb
         B.backward_sampled(params, raster.ccam, raster.proj, raster.ranges, raster.vals, raster.active_tiles,

@@ -1,5 +1,5 @@
 """The differentiable render's buffers: the gradient taken as it comes (dense,
-expanded, strided, of another precision) or copied, pixel lists longer than
+expanded, strided, with its sign pending) or copied, pixel lists longer than
 the sampled pixels, and lists that outgrow the capacity between two passes -
 against the same render from a fresh raster with room for everything."""
 import numpy as np
@@ -48,11 +48,12 @@ def _weights(rgb):
 
 
 @pytest.mark.parametrize("pad", [0, 37])
-@pytest.mark.parametrize("kind", ["dense", "strided", "expanded"])
+@pytest.mark.parametrize("kind", ["dense", "strided", "expanded", "negated"])
 def test_gradients_as_they_come(AG, kind, pad):
     leaves = _leaves()
     make = dict(dense=_weights, strided=lambda rgb: torch.stack([_weights(rgb)] * 2, -1)[..., 0],
-                expanded=lambda rgb: torch.full((1, 1), 0.5, device="cuda").expand_as(rgb))[kind]
+                expanded=lambda rgb: torch.full((1, 1), 0.5, device="cuda").expand_as(rgb),
+                negated=lambda rgb: torch._neg_view(_weights(rgb)))[kind]       # the sign not yet applied
     want_rgb, want = _grads(AG, _raster(AG), leaves, lambda rgb: make(rgb).clone(memory_format=torch.contiguous_format))
     raster = _raster(AG, pad=pad)
     for _ in range(2):                                       # the second pass reuses every buffer

@@ -50,9 +50,12 @@ class SampledRaster:
         self.n_last = torch.zeros(max(int(pix_idx.shape[0]), 1), dtype=torch.int32, device=dev)
         self.grad2d = torch.zeros(n, 12, device=dev)
         self.touched = torch.zeros(n, dtype=torch.uint8, device=dev)
-        # the pair count on the host: copied out after the binning, read once the render is under way
-        self._need = torch.zeros(1, dtype=torch.int64, pin_memory=True)
-        self._binned = torch.cuda.Event()
+        # the pair count on the host: copied out after the binning, read once the
+        # render is under way; made by the first render (a raster of CPU tensors has no use for it)
+        self._need = self._binned = None
+
+    def __getstate__(self):
+        return {**self.__dict__, "_need": None, "_binned": None}  # a copy makes its own
 
     @staticmethod
     def from_tiles(cam: dict, n_gaussians: int, tiles, device="cuda", **kw):
@@ -115,6 +118,9 @@ class SampledRaster:
         B.project_gaussians(params, self.ccam, self.tile_rank, self.proj, self.sh_degree)
         self._ensure_bins()
         self._bin()
+        if self._need is None:
+            self._need = torch.zeros(1, dtype=torch.int64, pin_memory=True)
+            self._binned = torch.cuda.Event()
         self._need.copy_(self.n_isect, non_blocking=True)
         self._binned.record()
         n_out = max(int(self.pix_idx.shape[0]), 1)

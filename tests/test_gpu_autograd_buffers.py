@@ -2,6 +2,8 @@
 expanded, strided, with its sign pending) or copied, pixel lists longer than
 the sampled pixels, and lists that outgrow the capacity between two passes -
 against the same render from a fresh raster with room for everything."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -61,6 +63,18 @@ def test_gradients_as_they_come(AG, kind, pad):
         assert rgb.shape == want_rgb.shape and torch.equal(rgb, want_rgb)
         for f, a, b in zip(FIELDS, got, want):
             # atomics in another order: a few 2^-24 of sums of some hundred terms
+            assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max()), f
+
+
+def test_copy_of_a_used_raster(AG):
+    leaves = _leaves()
+    raster = _raster(AG)
+    want_rgb, want = _grads(AG, raster, leaves, _weights)
+    twin = copy.deepcopy(raster)
+    for r in (twin, raster):
+        rgb, got = _grads(AG, r, leaves, _weights)
+        assert torch.equal(rgb, want_rgb)
+        for f, a, b in zip(FIELDS, got, want):
             assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max()), f
 
 

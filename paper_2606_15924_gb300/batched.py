@@ -30,6 +30,8 @@ rebuilt on the host, and such steps run without a captured graph.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 
@@ -359,13 +361,29 @@ def _cache_path() -> str:
     return os.path.join(root, "grid_tune.json")
 
 
+@functools.lru_cache(maxsize=1)
+def _library_digest() -> str:
+    return hashlib.sha256(open(B.LIB_PATH, "rb").read()).hexdigest()[:16]
+
+
+def _cache_key(mv: MultiViewTrainer, device_name: str) -> str:
+    """What a tuned grid belongs to.  A grid counts blocks of the kernels that
+    it was timed with, so the library's build and what chooses among its
+    kernels (checkpoints, statistics, resident blocks) are part of it: an
+    entry of another build, whose blocks were larger or smaller, is not found."""
+    return "|".join([device_name, str(mv.K)] + [f"{v.W}x{v.H}:{v.n_select}:{v.n_pix}" for v in mv.views] +
+                    [f"ck{mv.ck_slots}", f"stats{int(mv.stats is not None)}", "resident%d,%d" % tuple(mv.resident),
+                     f"lib{_library_digest()}"])
+
+
 def autotune_grid(mv: MultiViewTrainer, reps: int = 10, use_cache: bool = True) -> dict:
     """Pick (forward, backward) persistent grid sizes for this trainer's shape
     by timing graph replays of the two launches on the current sampled sets.
     The choice is cached per (device, views, image sizes, tile counts, pixels
-    per tile) in a JSON file; returns {"grid": (f, b), "times": {...}}."""
+    per tile, checkpoints, statistics, build of the library) in a JSON file;
+    returns {"grid": (f, b), "times": {...}}."""
     props = torch.cuda.get_device_properties(mv.params["means"].device)
-    key = "|".join([props.name, str(mv.K)] + [f"{v.W}x{v.H}:{v.n_select}:{v.n_pix}" for v in mv.views])
+    key = _cache_key(mv, props.name)
     path = _cache_path()
     cache = {}
     if use_cache and os.path.exists(path):

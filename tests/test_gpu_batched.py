@@ -177,6 +177,30 @@ def test_multiview_step_in_one_graph_trains(B, mode, rows):
     assert int(mv.step_dev.item()) == 42
 
 
+def test_autotune_does_not_take_another_builds_grid(B, tmp_path, monkeypatch):
+    """An entry under the device, views and sizes alone, as builds with other
+    blocks wrote it, and one of this trainer without statistics."""
+    import json
+    from paper_2606_15924_gb300.batched import autotune_grid, grid_candidates
+    monkeypatch.setenv("TURBOGS_CACHE", str(tmp_path))
+    mv = _make()
+    props = torch.cuda.get_device_properties(0)
+    old = "|".join([props.name, str(mv.K)] + [f"{v.W}x{v.H}:{v.n_select}:{v.n_pix}" for v in mv.views])
+    (tmp_path / "grid_tune.json").write_text(json.dumps({old: {"grid": [7, 7], "times": {}}}))
+    mv.forward()
+    autotune_grid(mv, reps=2)
+    for k in (0, 1):
+        assert mv.grid[k] in grid_candidates(mv.resident[k], props.multi_processor_count)
+    cache = json.loads((tmp_path / "grid_tune.json").read_text())
+    assert len(cache) == 2 and cache[old]["grid"] == [7, 7]
+    for key in cache:
+        cache[key]["grid"] = [7, 7]
+    (tmp_path / "grid_tune.json").write_text(json.dumps(cache))
+    mv.stats = torch.zeros(mv.n, 4, device="cuda")
+    autotune_grid(mv, reps=2)
+    assert 7 not in mv.grid
+
+
 def test_autotune_picks_a_candidate_and_keeps_results(B, tmp_path, monkeypatch):
     from paper_2606_15924_gb300.batched import autotune_grid, grid_candidates
     monkeypatch.setenv("TURBOGS_CACHE", str(tmp_path))

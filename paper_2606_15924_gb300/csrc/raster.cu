@@ -1612,9 +1612,19 @@ extern "C" tgs_status tgs_render_sampled(const tgs_projected* proj, const int32_
   return check_launch();
 }
 
+// Eq. 12's statistics of one view by the walk from the front.
+static void launch_error_stats(const RasterArgs& a, int n_active_max, int n_pix_max, const int32_t* n_last,
+                               const float* err, float* stats, cudaStream_t s) {
+  if (n_active_max <= 0) return;
+  const int B = block_for(n_pix_max);
+  k_error_stats<<<n_active_max, B, B * sizeof(Splat), s>>>(a, n_last, err, stats);
+}
+
 // The one-view backward; with st.stats set, Eq. 12's statistics of the same
-// pixels too (fused into the warp-per-piece replay, or as the separate pass
-// after the whole-tile backward).
+// pixels too: in the same replay where checkpoints are given, else by a walk of
+// their own.  A replay from a checkpoint recovers T over at most a piece from the
+// forward's own value, one without it over the whole list: at 500 blended splats a
+// pixel its sums were 9.7e-8 of their norm off 64 bits, the walk's 5.9e-8.
 static tgs_status render_backward_impl(const tgs_projected* proj, const int32_t* tile_ranges, const int32_t* vals,
                                        const int32_t* active_tiles, const int32_t* n_active, int32_t n_active_max,
                                        const int32_t* pix_off, const uint8_t* pix_idx, int32_t n_pix_max,
@@ -1639,8 +1649,11 @@ static tgs_status render_backward_impl(const tgs_projected* proj, const int32_t*
   if (n_active_max > 0) {
     const BwdSplit sp = bwd_split(n_active_max, n_pix_max, ck);
     const int64_t items = (int64_t)n_active_max * sp.groups * sp.pieces;
-    bwd_kernel((sp.gpx + 31) / 32, stats)<<<(int)items, 32, 0, s>>>(a, T_final, n_last, dL_drgb, grad2d, ck, st,
+    const bool fused = stats && ck.data;
+    bwd_kernel((sp.gpx + 31) / 32, fused)<<<(int)items, 32, 0, s>>>(a, T_final, n_last, dL_drgb, grad2d, ck, st,
                                                                           sp, n_active_max);
+    if (stats && !fused)
+      launch_error_stats(a, n_active_max, n_pix_max, n_last, st.err, reinterpret_cast<float*>(st.stats), s);
   }
   return check_launch();
 }
@@ -1686,10 +1699,7 @@ extern "C" tgs_status tgs_error_stats_sampled(const tgs_projected* proj, const i
   cudaStream_t s = (cudaStream_t)stream;
   if (n_gaussians == 0) return TGS_OK;
   if (!accumulate) cudaMemsetAsync(stats, 0, sizeof(float) * 4 * (size_t)n_gaussians, s);
-  if (n_active_max > 0) {
-    const int B = block_for(n_pix_max);
-    k_error_stats<<<n_active_max, B, B * sizeof(Splat), s>>>(a, n_last, err_pix, stats);
-  }
+  launch_error_stats(a, n_active_max, n_pix_max, n_last, err_pix, stats, s);
   return check_launch();
 }
 
@@ -1810,7 +1820,10 @@ static tgs_status render_backward_batched_impl(const tgs_view_batch* views, int3
   if (with_stats && !accumulate_stats && n_stats > 0) cudaMemsetAsync(stats, 0, sizeof(float4) * (size_t)n_stats, s);
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   if (b.base[n_views] == 0) return check_launch();
-  bwd_batched_kernel((b.split.gpx + 31) / 32, with_stats)<<<grid_ctas, 32, 0, s>>>(b, counter);
+  const bool fused = with_stats && b.ck[0].data;
+  bwd_batched_kernel((b.split.gpx + 31) / 32, fused)<<<grid_ctas, 32, 0, s>>>(b, counter);
+  for (int v = 0; with_stats && !fused && v < n_views; ++v)  // without checkpoints: as in the one-view backward
+    launch_error_stats(b.a[v], views[v].n_active_max, views[v].n_pix_max, b.last[v], b.err[v], stats, s);
   return check_launch();
 }
 

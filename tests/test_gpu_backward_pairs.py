@@ -159,3 +159,32 @@ def test_nonfinite_values_stay_local(B, slots):
     got = backward(dL, proj=q)
     assert not bool(torch.isfinite(got[i, :9]).all())
     assert bool(torch.isfinite(got).all(1).sum() > 0.5 * N)
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_statistics_without_checkpoints_are_the_walks(B, batched):
+    """One tile, so that every splat's row takes one sum: the bits of
+    error_stats_sampled, whose T are the forward's products."""
+    n_pix = 32
+    p, sel, binned, out, bg, backward, P, pd = _case(B, n_pix, 0, 1)
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=W, height=H)
+    err = torch.rand(P, generator=torch.Generator().manual_seed(7)).cuda()
+    dL = torch.randn(P, 3, generator=torch.Generator().manual_seed(5)).cuda()
+    a = (pd, binned["ranges"], binned["vals"], sel["active_tiles"], sel["n_active"], 1, sel["pix_off"], sel["pix_idx"],
+         n_pix, cam)
+    want = torch.zeros(N, 4, device="cuda")
+    B.error_stats_sampled(*a, out["n_last"], err, want)
+    g2, got = torch.zeros(N, 12, device="cuda"), torch.zeros(N, 4, device="cuda")
+    if batched:
+        vb = B.view_batch([dict(proj=pd, tile_ranges=binned["ranges"], vals=binned["vals"],
+                                active_tiles=sel["active_tiles"], n_active=sel["n_active"], n_active_max=1,
+                                pix_off=sel["pix_off"], pix_idx=sel["pix_idx"], n_pix_max=n_pix, cam=cam, bg=bg,
+                                rgb=out["rgb"], T_final=out["T"], n_last=out["n_last"], ckpt=None, dL_drgb=dL,
+                                grad2d=g2)])
+        B.render_backward_batched_stats(vb, 4, torch.zeros(1, dtype=torch.int32, device="cuda"), [err], got)
+    else:
+        B.render_backward_sampled_stats(*a, bg, out["T"], out["n_last"], dL, g2, err, got)
+    assert int((want[:, 1] > 0).sum()) > 20
+    assert torch.equal(got, want)
+    plain = backward(dL)
+    assert float((g2 - plain).norm()) <= 1e-6 * float(plain.norm())

@@ -967,7 +967,7 @@ __device__ __forceinline__ void bwd_pair(const BwdPair& P, const f32x2 (&px)[PPL
     v[8] = u == 0 ? mul2(w, g2[u]) : fma2(w, g2[u], v[8]);
     if (STATS) {
       // a dx^2 + 2 b dx dy + c dy^2 = -2 power = -2 ln(2) p
-      const float D0 = sqrt_approx(fmaxf(p0 * kInvA, 0.f)), D1 = sqrt_approx(fmaxf(p1 * kInvA, 0.f));
+      const float D0 = sqrtf(fmaxf(p0 * kInvA, 0.f)), D1 = sqrtf(fmaxf(p1 * kInvA, 0.f));
       const f32x2 ee = pk2(err[u], err[u]);
       sv[0] = u == 0 ? mul2(w, ee) : fma2(w, ee, sv[0]);
       sv[1] = u == 0 ? w : add2(w, sv[1]);
@@ -1074,7 +1074,7 @@ __device__ __noinline__ void bwd_rest_safe(const RasterArgs& a, int j, int p0, i
         }
         z[0] = err * w;
         z[1] = w;
-        z[2] = w * sqrt_approx(fmaxf(splat_pow2(sp.co, dx, dy) * kInvA, 0.f));
+        z[2] = w * sqrtf(fmaxf(splat_pow2(sp.co, dx, dy) * kInvA, 0.f));
       }
       if (!__any_sync(full, ok)) continue;
       for (int c = 0; c < 9; ++c) v[c] = warp_sum(v[c]);

@@ -188,3 +188,51 @@ def test_statistics_without_checkpoints_are_the_walks(B, batched):
     assert torch.equal(got, want)
     plain = backward(dL)
     assert float((g2 - plain).norm()) <= 1e-6 * float(plain.norm())
+
+
+def _one_splat_a_tile(B, opac):
+    """A splat and a sampled pixel in each of 4096 tiles: every output row is one
+    term.  Returns a call of the backward with checkpoints for a given gradient
+    and error: (grad2d, statistics), the separate walk's statistics for the
+    error, and the forward's outputs."""
+    from gpu_util import bin_dev, projected_dev, select_dev
+    n = T = 4096
+    W1 = H1 = 1024
+    rng = np.random.default_rng(9)
+    p = scenes.projected(n, W1, H1, seed=9)
+    t = np.arange(n)
+    p["xy"] = (16.0 * np.stack([t % 64, t // 64], 1) + rng.uniform(2.0, 14.0, (n, 2))).astype(np.float32)
+    p["radius"][:] = 1
+    p["conic"] = np.stack([rng.uniform(0.01, 0.05, n), rng.uniform(-0.005, 0.005, n), rng.uniform(0.01, 0.05, n)],
+                          1).astype(np.float32)
+    p["opac"] = opac(rng, n).astype(np.float32)
+    p["rgb"] = np.tile(np.float32([1.0, 0.0, 0.0]), (n, 1))
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=W1, height=H1)
+    sel = select_dev(B, scenes.error_map(W1, H1), scenes.age_map(W1, H1), W1, H1, T, 1, seed=4)
+    pd = projected_dev(p)
+    b = bin_dev(B, pd, n, cam, sel["tile_rank"], T, capacity=n)
+    rgb, Tf, last = torch.zeros(T, 3, device="cuda"), torch.zeros(T, device="cuda"), torch.zeros(T, dtype=torch.int32, device="cuda")
+    data, longest = torch.zeros(T * 4, device="cuda"), torch.zeros(T, dtype=torch.int32, device="cuda")
+    ck = B.checkpoints(data, 1, T, rgb, longest)
+    a = (pd, b["ranges"], b["vals"], sel["active_tiles"], sel["n_active"], T, sel["pix_off"], sel["pix_idx"], 1, cam)
+    bg = (0.0, 0.0, 0.0)
+    B.render_sampled(*a, bg, rgb, Tf, last, ckpt=ck)
+
+    def backward(dL, err):
+        keep = data, longest
+        g2, st, walk = (torch.zeros(n, w, device="cuda") for w in (12, 4, 4))
+        B.render_backward_sampled_stats(*a, bg, Tf, last, dL, g2, err, st, ckpt=ck)
+        B.error_stats_sampled(*a, last, err, walk)
+        return g2, st, walk
+    return p, rgb, backward
+
+
+def test_statistics_take_the_rounded_square_root(B):
+    """D is an IEEE square root in the replay as in the walk: where both have the
+    same bits of w (T recovered as exactly 1), D w has the same bits too."""
+    p, rgb, backward = _one_splat_a_tile(B, lambda rng, n: rng.uniform(0.2, 0.9, n))
+    one = torch.ones(4096, device="cuda")
+    _, st, walk = backward(torch.zeros(4096, 3, device="cuda"), one)
+    same = (st[:, 1] == walk[:, 1]) & (walk[:, 1] > 0)
+    assert int(same.sum()) > 1000
+    assert torch.equal(st[same, 2], walk[same, 2])

@@ -903,11 +903,14 @@ __device__ __forceinline__ void bwd_stage(BwdPair* Q, int i, const SplatRaw& w, 
   P.id[e] = w.id;
   // sums of dL/dpower times dx, dy, dx^2, dx dy, dy^2, 1 (power = -(a dx^2 +
   // c dy^2)/2 - b dx dy, dx = px - x): dL/dx = a m1 + b m2, dL/dy = c m2 + b m1,
-  // dL/da = -m3 / 2, dL/db = -m4, dL/dc = -m5 / 2, dL/do = m0 / o
+  // dL/da = -m3 / 2, dL/db = -m4, dL/dc = -m5 / 2, dL/do = m0 / o, by the rounded
+  // reciprocal: dL/do is then within 3 % of as near to 64 bits as the sum of
+  // dL/dalpha G itself, for two selections less a pair and pixel (dense view 861
+  // us a step against 867)
   const float o = w.c.w;
   float4* f = reinterpret_cast<float4*>(P.cf[e]);
   f[0] = make_float4(w.c.x, w.c.z, -0.5f, -1.f);
-  f[1] = make_float4(-0.5f, o > 0.f ? __fdividef(1.f, o) : 0.f, 1.f, 1.f);
+  f[1] = make_float4(-0.5f, o > 0.f ? __frcp_rn(o) : 0.f, 1.f, 1.f);
   P.bo[e] = w.c.y;
 }
 

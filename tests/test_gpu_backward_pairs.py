@@ -236,3 +236,17 @@ def test_statistics_take_the_rounded_square_root(B):
     same = (st[:, 1] == walk[:, 1]) & (walk[:, 1] > 0)
     assert int(same.sum()) > 1000
     assert torch.equal(st[same, 2], walk[same, 2])
+
+
+def test_opacity_gradient_takes_the_rounded_reciprocal(B):
+    """With colour (1, 0, 0), that gradient and no background, the sums of one
+    splat and pixel are dL/dred = alpha T and dL/do = (alpha T) / o: the same
+    bits times 1 / o rounded, over opacities of every mantissa."""
+    p, rgb, backward = _one_splat_a_tile(B, lambda rng, n: rng.uniform(0.1, 0.98, n))
+    dL = torch.zeros(4096, 3, device="cuda")
+    dL[:, 0] = 1.0
+    g2, _, _ = backward(dL, torch.zeros(4096, device="cuda"))
+    g2 = g2.cpu().numpy()
+    hit = g2[:, 6] > 0
+    assert hit.sum() > 3000
+    np.testing.assert_array_equal(g2[hit, 5], g2[hit, 6] * (np.float32(1.0) / p["opac"][hit]))

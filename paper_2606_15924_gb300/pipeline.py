@@ -70,6 +70,13 @@ def head_of(g: dict, m: int) -> dict:
 class Trainer:
     CKPT_POSITIONS = 2048
     CKPT_EVERY = 32       # list positions per checkpoint slot (fixed by the kernels)
+    # Render and backward without and with checkpoints, us, lists of 4000 to 5000
+    # pairs (500k Gaussians), every tile: 3600 tiles of 25 pixels 184, 140; 8160 of
+    # 25 264, 244 and of 87 373, 342; 10000 of 25 289, 286 and of 87 432, 412; 11900 of
+    # 25 304, 322 and of 87 465, 469; 16000 of 25 354, 404.  In two groups of pixels:
+    # 3600 of 204 410, 352; 6000 of 153 463, 472.  Lists of 16000 to 18000 pairs (2M
+    # Gaussians) gain up to 13600 tiles (471, 424) and lose from 24000 (594, 653).
+    CKPT_WARPS = 72
 
     def __init__(self, params: dict, cam: dict, target: torch.Tensor, tile_fraction: float = 0.2,
                  pixel_rate: float = 1.0 / 3.0, cfg: Config | None = None, dense: bool = False,
@@ -138,13 +145,13 @@ class Trainer:
         self.lam = torch.zeros(S, device=dev)
         self.err_pix = torch.zeros(P, device=dev)
         self.loss = torch.zeros(1, dtype=torch.float64, device=dev)
-        # forward checkpoints for the split backward: only when the step's
-        # tiles (whole lists, one warp per 128 sampled pixels) would fill the
-        # GPU less than twice over; one slot every CKPT_EVERY positions of the
-        # tile list up to CKPT_POSITIONS.  3600 tiles of 25 pixels: the
-        # backward takes 132 us with checkpoints, 201 without
+        # forward checkpoints for the split backward, one slot every CKPT_EVERY
+        # positions of the tile list up to CKPT_POSITIONS (1 KB a sampled
+        # pixel): while whole lists, one warp per 128 sampled pixels, give the
+        # GPU fewer than CKPT_WARPS warps an SM
         self.ckpt = None
-        if train and not dense and S * ((self.n_pix + 127) // 128) < 2 * B.render_batched_resident(self.n_pix, 1):
+        warps = S * ((self.n_pix + 127) // 128)
+        if train and not dense and warps < self.CKPT_WARPS * self._sms(dev):
             n_slots = self.CKPT_POSITIONS // self.CKPT_EVERY
             self.ck_data = torch.empty(B.checkpoint_bytes(S, self.n_pix, n_slots) // 4, device=dev)
             self.ck_last = torch.zeros(S, dtype=torch.int32, device=dev)
@@ -174,6 +181,10 @@ class Trainer:
         self.loss_params = (l.eps_charbonnier, l.eps_ncc, l.beta_ema)
 
     # ------------------------------------------------------------------ setup
+    @staticmethod
+    def _sms(dev) -> int:
+        return torch.cuda.get_device_properties(dev).multi_processor_count
+
     def _alloc_bins(self, capacity: int):
         dev = self.params["means"].device
         self.capacity = int(capacity)

@@ -7,7 +7,7 @@ the selection (bit for bit), the projection of every Gaussian, the forward at
 every sampled pixel (on the forward's output), the backward of a seeded dL/dI
 that is non-zero at those 512 pixels only (so that both sides sum the same
 terms), and the fused projection adjoint + hybrid update (mode 1) of the
-Gaussians it touches."""
+Gaussians it touches.  And which full-size views get checkpoints."""
 import numpy as np
 import pytest
 import torch
@@ -162,3 +162,15 @@ def test_full_size_step_against_oracle(orc):
     assert checked >= 3
     untouched = ~t_g
     np.testing.assert_array_equal(join(P_)[untouched], p0[untouched])
+
+
+@pytest.mark.parametrize("W,H,rate,want", [(1920, 1080, 0.1, True), (1920, 1080, 0.5, True), (1280, 720, 0.8, True),
+                                           (2560, 1600, 0.1, False), (1920, 1080, 0.8, False)])
+def test_checkpoints_where_whole_lists_leave_the_gpu_idle(W, H, rate, want):
+    """Every tile sampled: 8160 tiles in one group of pixels and 3600 in two have
+    checkpoints, 16000 and 8160 in two do not."""
+    from gpu_util import dev, gaussians_dev
+    from paper_2606_15924_gb300.pipeline import Trainer
+    tr = Trainer(gaussians_dev(scenes.gaussians(100, seed=1)), scenes.look_at((0.0, 0.0, -4.0), width=W, height=H),
+                 dev(scenes.smooth_image(W, H, seed=1)), tile_fraction=1.0, pixel_rate=rate)
+    assert (tr.ckpt is not None) is want

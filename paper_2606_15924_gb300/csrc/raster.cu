@@ -916,7 +916,9 @@ __device__ __forceinline__ void bwd_stage(BwdPair* Q, int i, const SplatRaw& w, 
 
 // One pair against the lane's pixels, and its sums into the gradient rows.
 // CAPPED: an opacity reaches the cap on alpha.  Where a splat does not blend,
-// sums and states change by zeros, so everything has to be finite.
+// sums and states change by zeros, so everything has to be finite; and T is
+// multiplied by rcp_approx(-1) twice, which has to be exactly -1 (the PTX
+// document promises it to one unit only; tested over thousands of skipped splats).
 template <int PPL, bool CAPPED, bool STATS>
 __device__ __forceinline__ void bwd_pair(const BwdPair& P, const f32x2 (&px)[PPL], const f32x2 (&py)[PPL],
                                          const f32x2 (&g0)[PPL], const f32x2 (&g1)[PPL], const f32x2 (&g2)[PPL],

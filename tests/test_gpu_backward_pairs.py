@@ -250,3 +250,42 @@ def test_opacity_gradient_takes_the_rounded_reciprocal(B):
     hit = g2[:, 6] > 0
     assert hit.sum() > 3000
     np.testing.assert_array_equal(g2[hit, 5], g2[hit, 6] * (np.float32(1.0) / p["opac"][hit]))
+
+
+def test_skipped_splats_leave_the_transmittance_alone(B):
+    """A pixel that blends the first and the last splat of a list and none of
+    the thousands between, which other pixels of its group blend: its gradients
+    have the bits of the list of those two."""
+    from gpu_util import bin_dev, dev, projected_dev
+    n, side = 6002, 16
+    cam = scenes.look_at((0.0, 0.0, -4.0), width=side, height=side)
+    rng = np.random.default_rng(2)
+    p = scenes.projected(n, side, side, seed=2)
+    ends = [0, n - 1]
+    p["xy"] = np.stack([rng.uniform(11.0, 15.0, n), rng.uniform(0.0, 2.0, n)], 1).astype(np.float32)
+    p["conic"] = np.tile(np.float32([1.0, 0.1, 1.0]), (n, 1))            # 10 pixels away: exp(-50)
+    p["xy"][ends], p["conic"][ends] = [[1.0, 1.2], [1.5, 0.9]], [[0.05, 0.01, 0.06], [0.04, 0.0, 0.05]]
+    p["radius"][:] = 4
+    p["opac"] = rng.uniform(0.02, 0.6, n).astype(np.float32)
+    p["depth"] = np.linspace(1.0, 9.0, n).astype(np.float32)
+    sel = dict(active_tiles=dev(np.int32([0])), n_active=dev(np.int32([1])), tile_rank=dev(np.int32([0])),
+               pix_off=dev(np.int32([0, 32])), pix_idx=dev(np.arange(32, dtype=np.uint8)))
+    rows = []
+    for keep in (np.arange(n), np.array(ends)):
+        q = {k: v[keep] for k, v in p.items()}
+        pd, m = projected_dev(q), len(keep)
+        b = bin_dev(B, pd, m, cam, sel["tile_rank"], 1, capacity=n)
+        rgb, Tf = torch.zeros(32, 3, device="cuda"), torch.zeros(32, device="cuda")
+        last, g2 = torch.zeros(32, dtype=torch.int32, device="cuda"), torch.zeros(m, 12, device="cuda")
+        a = (pd, b["ranges"], b["vals"], sel["active_tiles"], sel["n_active"], 1, sel["pix_off"], sel["pix_idx"], 32, cam,
+             (0.3, 0.1, 0.6))
+        B.set_forward_split(1)               # the sequential walk: no composition of half lists
+        B.render_sampled(*a, rgb, Tf, last)
+        B.set_forward_split(0)
+        dL = torch.zeros(32, 3, device="cuda")
+        dL[0] = torch.tensor([0.7, -0.4, 0.9])
+        B.render_backward_sampled(*a, Tf, last, dL, g2)
+        assert int(last[0]) == m and int((g2 != 0).any(1).sum()) == 2
+        rows.append((g2[[0, m - 1]], rgb[0], Tf[0]))
+    for x, y in zip(*rows):
+        assert torch.equal(x, y)

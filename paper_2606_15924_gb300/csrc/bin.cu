@@ -721,7 +721,8 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
     return check_launch();
   }
   if (shared_path) {
-    const bool starts = capacity >= kStartsPairs;
+    // it writes the keys 16 bytes at a time; a workspace is taken from any 8-byte boundary
+    const bool starts = capacity >= kStartsPairs && aligned16(w.keys);
     if (starts)
       k_hist_starts<<<2 * std::max(1, device_sm_count()), kStartThreads, 0, s>>>(w.tile_cnt, R, w.tile_start, n_isect,
                                                                                  w.keys, capacity);

@@ -51,6 +51,25 @@ def test_starts_launch_is_bit_exact(B, n, W, H, share):
         assert torch.equal(few[k][:I], many[k][:I]), k
 
 
+@pytest.mark.parametrize("capacity", [10 ** 6, MANY])
+def test_workspace_at_any_eight_bytes(B, capacity):
+    from gpu_util import bin_dev, projected_dev
+    n, W, H, T = 3001, 250, 187, 192
+    pd, cam = projected_dev(scenes.projected(n, W, H, seed=5)), _cam(W, H)
+    want = bin_dev(B, pd, n, cam, None, T, capacity=10 ** 6)
+    I = int(want["n_isect"].item())
+    need = B.bin_tiles_workspace_size(n, capacity, T)
+    ws = torch.empty(need + 24, dtype=torch.uint8, device="cuda")
+    vals = torch.zeros(capacity, dtype=torch.int32, device="cuda")
+    ranges = torch.zeros(T, 2, dtype=torch.int32, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for at in (0, 8, 16, 24):
+        vals.zero_()
+        assert (ws.data_ptr() + at) % 8 == 0
+        B.bin_tiles(pd, n, cam, None, T, ws[at:at + need], capacity, vals, None, ranges, count)
+        assert torch.equal(vals[:I], want["vals"][:I]) and torch.equal(ranges, want["ranges"]) and int(count.item()) == I
+
+
 def test_more_pairs_than_the_capacity(B):
     from gpu_util import bin_dev, projected_dev
     n, W, H, T = 1800, 1280, 720, 3600

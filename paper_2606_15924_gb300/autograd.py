@@ -132,6 +132,9 @@ class SampledRaster:
         need = int(self._need[0])
         if need > self.capacity:  # the Gaussians moved: grow, bin and render again
             self.capacity = int(need * 1.25) + 1024
+            # the first render may still be reading the old lists, on a stream that need not be the one they
+            # were allocated on
+            self.vals.record_stream(torch.cuda.current_stream())
             self.vals = None
             self._ensure_bins()
             self._bin()

@@ -91,6 +91,25 @@ def test_lists_that_outgrow_the_capacity(AG):
         assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max()), f
 
 
+def test_lists_that_outgrow_the_capacity_on_another_stream(AG, monkeypatch):
+    """The old lists are given back while the first render may still read them:
+    not before that stream is done with them."""
+    small, large = _leaves(), _leaves(1.2)
+    raster = _raster(AG)
+    _grads(AG, raster, small, _weights)
+    old, kept = raster.vals, []
+    record = torch.Tensor.record_stream
+    monkeypatch.setattr(torch.Tensor, "record_stream", lambda t, s: (kept.append((t.data_ptr(), s)), record(t, s))[1])
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side), torch.no_grad():
+        rgb = raster.forward_buffers(large)
+    torch.cuda.current_stream().wait_stream(side)
+    assert raster.vals is not old and (old.data_ptr(), side) in kept
+    want = _raster(AG, capacity=4 * raster.capacity).forward_buffers({k: v.detach() for k, v in large.items()})
+    assert torch.equal(rgb, want)
+
+
 def test_capture_is_refused_as_before(AG):
     """The pair count is read on the host, so a pass cannot be captured."""
     leaves = _leaves()

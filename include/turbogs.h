@@ -520,13 +520,12 @@ tgs_status tgs_render_backward_sampled(const tgs_projected* proj, const int32_t*
  * compositing weight w = T alpha, stats[i] += (e w, w, D w, 0), with e the
  * pixel's error err_pix [P] (from loss_sparse_ncc) and D the conic
  * Mahalanobis distance of the pixel centre from the splat.  The weights are
- * the ones the backward recovers (T by division from the end of the walk),
- * equal to the forward's up to rounding.  stats: device [N,4] float, 16-byte
+ * the forward's up to rounding.  stats: device [N,4] float, 16-byte
  * aligned, zeroed first unless accumulate_stats = 1 (so the views of a step
- * and several steps can add up).  With checkpoints the sums ride on the
- * warp-per-piece replay (one more 4-value warp reduction and one vector
- * atomic per warp and splat); without, error_stats_sampled runs after the
- * whole-tile backward.  Other arguments and results as
+ * and several steps can add up).  With checkpoints the sums ride on the replay
+ * of the pieces (T by division from a piece's end; one more 3-value warp
+ * reduction and one vector atomic per warp and splat); without,
+ * error_stats_sampled's walk runs after the backward.  Other arguments and results as
  * render_backward_sampled.
  */
 tgs_status tgs_render_backward_sampled_stats(const tgs_projected* proj, const int32_t* tile_ranges,
@@ -695,9 +694,11 @@ typedef struct {
 tgs_status tgs_advance_counters(int64_t* iter_dev, int32_t* step_dev, tgs_stream stream);
 
 /* Thread blocks of the batched kernels that fit on the current device at
- * once (SMs x resident blocks per SM) for n_pix_max pixels per tile: the
- * largest useful grid_ctas.  backward: 0 the forward, 1 the backward without
- * checkpoints (whole tiles), 2 the backward in pieces (with checkpoints). */
+ * once (SMs x resident blocks per SM) for n_pix_max pixels per tile: a grid_ctas
+ * that fills it.  backward: 0 the forward; 1 (without checkpoints) and 2 (with)
+ * the backward, one kernel of one-warp blocks for both, counted without
+ * statistics.  Launches of few tiles take groups of fewer pixels, whose kernels
+ * may fit a few more blocks. */
 tgs_status tgs_render_batched_resident(int32_t n_pix_max, int32_t backward, int32_t* ctas);
 tgs_status tgs_render_sampled_batched(const tgs_view_batch* views, int32_t n_views, int32_t grid_ctas,
                                       int32_t* counter, tgs_stream stream);

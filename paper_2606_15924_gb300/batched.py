@@ -90,9 +90,9 @@ class MultiViewTrainer:
         # per-view Jacobian rows feed only the full-matrix LM mode
         self.use_rows = (self.opt["mode"] == 2) if view_rows is None else bool(view_rows)
         self.rows = torch.zeros(self.max_active, self.n, 14, device=dev) if self.use_rows else None
-        # persistent=False: one launch per view with one block per active
-        # tile (the same kernels without the shared queue) and one
-        # accumulating projection adjoint per view, for comparison
+        # persistent=False: one launch per view (the forward one block per
+        # active tile, the backward a queue of its own) and one accumulating
+        # projection adjoint per view, for comparison
         self.persistent = bool(persistent)
         self.counters = torch.zeros(2 + 2 * self.max_active, dtype=torch.int32, device=dev)
         self.n_pix_max = max(v.n_pix for v in self.pool)

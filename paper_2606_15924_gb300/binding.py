@@ -593,8 +593,8 @@ def view_batch(views: list) -> C.Array:
 
 
 def render_batched_resident(n_pix_max: int, backward) -> int:
-    """backward: 0 / False the forward, 1 / True the whole-tile backward, 2 the
-    backward in pieces (with checkpoints)."""
+    """backward: 0 / False the forward, 1 / True the backward without, 2 with
+    checkpoints (the same number)."""
     out = _i32(0)
     _check("tgs_render_batched_resident", _lib.tgs_render_batched_resident(int(n_pix_max), int(backward),
                                                                              C.byref(out)))

@@ -171,8 +171,7 @@ __device__ __forceinline__ void for_each_pair(const float2* __restrict__ xy, con
   }
 }
 
-// 1''. pairs per active tile with global atomics, 256 Gaussians per block,
-// their pairs dealt out evenly over the lanes.
+// 1''. pairs per active tile with global atomics, 256 Gaussians per block.
 __global__ void __launch_bounds__(256) k_count_pairs(const float2* __restrict__ xy,
                                                      const int32_t* __restrict__ radius, int64_t n, BinGeom geo,
                                                      const int32_t* __restrict__ tile_rank,
@@ -530,8 +529,9 @@ __device__ __forceinline__ void sort_run(SortSmem<T, E>& S, const uint64_t* __re
   }
 }
 
-// 64 registers at 256 threads (four blocks an SM), 42 at 512 (three): the
-// sort waits on shared memory and barriers, so it wants warps.
+// 64 registers at 256 threads (four blocks an SM), 40 at 512 (three): the
+// sort waits on shared memory and barriers, so it wants warps.  Sixteen keys a
+// thread then spill, 8 bytes at 256 threads and 268 at 512.
 template <int T, int E>
 __global__ void __launch_bounds__(T, T == 512 ? 3 : 4) k_tile_sort(const uint64_t* __restrict__ keys, RangeSrc src,
                                                  const int32_t* __restrict__ inv_rank, int64_t cap,
@@ -736,9 +736,13 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
                                                            w.tile_start, w.tile_fill, w.keys, capacity);
   }
   if (keys) k_inv_rank<<<(T + 255) / 256, 256, 0, s>>>(tile_rank, T, w.inv_rank, R);
-  // The sort's block by the lists' mean length (from the capacity, which the
-  // caller sizes from the pairs of all tiles): lists past its CAP are sorted
-  // in several runs, and a larger block leaves fewer of them on an SM.
+  // The sort's block by the lists' mean length, as far as the capacity tells it:
+  // lists past its CAP are sorted in several runs, and a larger block leaves
+  // fewer of them on an SM.  A training view's capacity is sized from the pairs of
+  // all tiles.  The differentiable render's is sized from those of its active
+  // tiles only, so there the mean comes out too small by the share of the tiles that
+  // are active (1340 of 6700 tiles of 2M Gaussians: 453 for lists of 2270, most of
+  // which then take two or three runs).
   const int64_t mean = capacity / T;
   int2* rg = reinterpret_cast<int2*>(tile_ranges);
   if (mean <= 512) launch_tile_sort<256, 8>(R, w, src, capacity, vals, keys, rg, s);

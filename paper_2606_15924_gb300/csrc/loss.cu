@@ -43,8 +43,9 @@ constexpr float kC1 = 1e-4f, kC2 = 9e-4f;
 // 720 tiles of 85 pixels 10 -> 7.7, eight views of 1200 to 4500 such tiles 192 ->
 // 105.
 constexpr int kLossWarps = 4;
-// Blocks on an SM, and launched per SM: 168 registers hold eight pixels a lane
-// without spills (four blocks of 128: 51 us for 42; 105 for 115 at three pixels).
+// Blocks on an SM, and launched per SM: 168 registers hold eight pixels a lane,
+// without spills for NCC and with 64 bytes a thread for SSIM (four blocks of 128:
+// 51 us for 42; 105 for 115 at three pixels).
 __host__ __device__ constexpr int loss_blocks(int ppl) { return ppl > 4 ? 3 : 4; }
 
 template <int STRUCT, int PPL>

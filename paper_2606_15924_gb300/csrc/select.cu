@@ -6,7 +6,9 @@
 // Efraimidis-Spirakis order (ascending E_i / w_i with E_i = -log2 U_i an
 // exponential clock in 32-bit fixed point), so every item's fate is decided
 // by counting the items that precede it in a total order - no sequential
-// loop, and integer-only arithmetic, hence bit-identical on every run.
+// loop.  The keys are exact (integers, and correctly rounded quotients of them),
+// hence bit-identical on every run; the pixel draw orders by fp32 quotients first,
+// and by the exact keys wherever the bounds on their error leave a choice open.
 #include "block_select.cuh"
 #include "scan.cuh"
 

@@ -243,7 +243,7 @@ def test_backward_parity(B, orc, split):
     oracle's analytic backward (relative L2 <= 1e-3 per parameter group);
     split: the backward replays each tile list in pieces of 32 positions from
     the forward's checkpoints (few slots, so that a long tail piece occurs, or
-    the trainer's 64), at 1, 3, 5 and 8 pixels per lane."""
+    the trainer's 64), at one to four pixels a lane, one or two groups a tile."""
     from gpu_util import bin_dev, dev, empty_projected, gaussians_dev, render_dev, select_dev, select_host
     g, cam = _c0(seed=5, n=3000)
     g["log_scales"] += 1.0
@@ -251,7 +251,7 @@ def test_backward_parity(B, orc, split):
     n = 3000
     err, age = scenes.error_map(W, H), scenes.age_map(W, H)
     target = scenes.smooth_image(W, H, seed=2)
-    # n_pix 25, 84, 150, 256: 1, 3, 5 and 8 pixels per lane in the warp-per-piece backward
+    # n_pix 25, 84, 150, 256: groups of one to four pixels a lane, one or two a tile
     for n_select, n_pix in ((64, 84), (256, 256), (64, 25), (64, 150)):
         sel = select_dev(B, err, age, W, H, n_select, n_pix, seed=4)
         sh = select_host(sel)
@@ -389,8 +389,8 @@ def test_statistics_fused_into_backward(B, orc, split):
     """Eq. 12's statistics accumulated inside the backward replay
     (render_backward_sampled_stats) against the oracle; the gradients equal
     those of the plain backward; accumulate adds a second call's sums.
-    split: the warp-per-piece replay from checkpoints (the sums ride on it);
-    otherwise the whole-tile backward followed by the statistics pass."""
+    split: the replay in pieces from checkpoints (the sums ride on it);
+    otherwise the backward over whole lists followed by the statistics pass."""
     from gpu_util import bin_dev, dev, empty_projected, gaussians_dev, select_dev, select_host
     g, cam = _c0(seed=5, n=3000)
     g["log_scales"] += 1.0

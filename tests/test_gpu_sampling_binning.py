@@ -60,9 +60,9 @@ BIN_CASES = [
 ]
 
 
-@pytest.mark.parametrize("presort", [False, True])
+@pytest.mark.parametrize("large_block", [False, True])
 @pytest.mark.parametrize("n,W,H,frac", BIN_CASES)
-def test_bin_tiles_bit_exact(B, orc, n, W, H, frac, presort):
+def test_bin_tiles_bit_exact(B, orc, n, W, H, frac, large_block):
     from gpu_util import bin_dev, dev, projected_dev, tile_count
     pr = scenes.projected(n, W, H, seed=n + W)
     T = tile_count(W, H)
@@ -76,7 +76,7 @@ def test_bin_tiles_bit_exact(B, orc, n, W, H, frac, presort):
     want = orc.bin_tiles(pr["xy"], pr["radius"], pr["depth"], W, H, rank)
     keys_w, vals_w, counts_w = want
     cam = dict(viewmat=np.eye(4), fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
-    cap = max(len(vals_w) + 100, 2049 * T) if presort else len(vals_w) + 100
+    cap = max(len(vals_w) + 100, 2049 * T) if large_block else len(vals_w) + 100
     out = bin_dev(B, projected_dev(pr), n, cam, None if rank is None else dev(rank), n_active_max, capacity=cap)
     I = int(out["n_isect"].item())
     assert I == len(vals_w)
@@ -93,17 +93,16 @@ def test_bin_tiles_bit_exact(B, orc, n, W, H, frac, presort):
             assert ranges[r][1] - ranges[r][0] == 0
 
 
-# Splats crowded into one tile, so that a tile's list is split into long
-# runs: (total, crowded) -> every path of the per-segment sort (registers,
-# warp shared memory, per-segment block sort, whole-range sort).
+# Splats crowded into one tile (total, crowded): lists that fit the tile sort's
+# block, and ones of 30 000 to 200 000 keys, which it takes in runs.
 CLUSTER_CASES = [(5000, 5000), (50000, 50000), (200000, 30000), (200000, 200000)]
 
 
-@pytest.mark.parametrize("presort", [False, True])
+@pytest.mark.parametrize("large_block", [False, True])
 @pytest.mark.parametrize("n,n_crowd", CLUSTER_CASES)
-def test_bin_tiles_crowded_tile_bit_exact(B, orc, n, n_crowd, presort):
-    """presort: a capacity above 2048 pairs per tile makes bin_tiles sort the
-    Gaussians by depth first and sort only segments of each tile's list."""
+def test_bin_tiles_crowded_tile_bit_exact(B, orc, n, n_crowd, large_block):
+    """large_block: a capacity above 2048 pairs per tile chooses the sort's block
+    of 512 threads (8192 keys)."""
     from gpu_util import bin_dev, projected_dev
     W, H = 256, 256
     rng = np.random.default_rng(n + n_crowd)
@@ -121,7 +120,7 @@ def test_bin_tiles_crowded_tile_bit_exact(B, orc, n, n_crowd, presort):
     keys_w, vals_w, counts_w = orc.bin_tiles(pr["xy"], pr["radius"], pr["depth"], W, H)
     assert counts_w.max() > 4096 or n_crowd < 20000
     cam = dict(viewmat=np.eye(4), fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
-    cap = max(len(vals_w) + 7, 2049 * 256) if presort else len(vals_w) + 7
+    cap = max(len(vals_w) + 7, 2049 * 256) if large_block else len(vals_w) + 7
     out = bin_dev(B, projected_dev(pr), n, cam, None, 256, capacity=cap)
     I = int(out["n_isect"].item())
     assert I == len(vals_w)
@@ -129,14 +128,13 @@ def test_bin_tiles_crowded_tile_bit_exact(B, orc, n, n_crowd, presort):
     np.testing.assert_array_equal(out["keys"][:I].cpu().numpy().view(np.uint64), keys_w)
 
 
-# One tile's list grown through each size band of the per-tile sort (up to
-# 256, 512, 1024, 2048 and 4096 keys in registers, and past 4096 in global
-# memory), with exact depth ties.  presort: the same lists through the depth
-# presort and the segment sort (whole list in shared memory up to 4096 keys,
-# with segments sorted per lane, per warp and per block).
-@pytest.mark.parametrize("presort", [False, True])
+# One tile's list grown from less than a key a thread past the block of 2048 keys
+# that the capacity chooses (two runs from 2049, three from 4200), with exact depth
+# ties in buckets past the longest that is ordered by counting.  large_block: the
+# same lists in one run of the block of 8192.
+@pytest.mark.parametrize("large_block", [False, True])
 @pytest.mark.parametrize("n_crowd", [200, 300, 700, 1500, 3000, 3900, 4200])
-def test_bin_tiles_sort_bands_bit_exact(B, orc, n_crowd, presort):
+def test_bin_tiles_sort_bands_bit_exact(B, orc, n_crowd, large_block):
     from gpu_util import bin_dev, projected_dev
     W, H = 256, 256
     n = n_crowd + 500
@@ -155,7 +153,7 @@ def test_bin_tiles_sort_bands_bit_exact(B, orc, n_crowd, presort):
     keys_w, vals_w, counts_w = orc.bin_tiles(pr["xy"], pr["radius"], pr["depth"], W, H)
     assert counts_w.max() >= n_crowd
     cam = dict(viewmat=np.eye(4), fx=100.0, fy=100.0, cx=W / 2, cy=H / 2, width=W, height=H, znear=0.2)
-    cap = max(len(vals_w) + 3, 2049 * 256) if presort else len(vals_w) + 3
+    cap = max(len(vals_w) + 3, 2049 * 256) if large_block else len(vals_w) + 3
     out = bin_dev(B, projected_dev(pr), n, cam, None, 256, capacity=cap)
     I = int(out["n_isect"].item())
     assert I == len(vals_w)

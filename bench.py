@@ -814,7 +814,7 @@ def batched_measure(args):
             "iters_per_s": 1e3 / mean, "ms_per_step": mean, "views_per_step": mv.K,
             "sampled_pixels": P, "active_tiles": [int(v.n_active.item()) for v in mv.views],
             "render_fwd_ms": fm, "render_bwd_ms": bm, "fwd_bwd_mpix_per_s": P / ((fm + bm) * 1e-3) / 1e6,
-            "splat_evals": evals, "grid": list(mv.grid) if persistent else "one block per active tile",
+            "splat_evals": evals, "grid": list(mv.grid) if persistent else "one block per active tile (forward), the resident blocks (backward)",
             "stage_ms": st,
             "kernels_per_step": mv.kernels_per_step, "clocks": clocks,
             "render_fwd_roofline": {"bound": "alu", "achieved": evals * (FLOPS_ALPHA + FLOPS_BLEND) / (fm * 1e-3) / 1e12,

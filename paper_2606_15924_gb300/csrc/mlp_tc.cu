@@ -595,8 +595,8 @@ __global__ void __launch_bounds__(kBwThreads, 1) k_mlp_backward_tc(
 // bf16, fp32 sums; y sums its two halves of 64 units and then adds b3.
 // Measured on GB300, 1.7 M rows: 355 us (532 TFLOP/s bf16 of the contractions'
 // 189 GFLOP); one tile at a time with a barrier a step took 528.  Bound by
-// shared memory: 68 % of its cycles carry the epilogues' and the tensor cores'
-// accesses, and the issue slots are 31 % busy.  With 512 epilogue threads of 32
+// shared memory: 65 % of its cycles carry the epilogues' (41) and the tensor cores'
+// (24) accesses, and the issue slots are 31 % busy.  With 512 epilogue threads of 32
 // units (128 registers) 359 us; with the issuing thread one of the 256 epilogue
 // threads and a barrier a step 368.
 constexpr uint32_t FT_W2 = 0;                             // W2 [128 n][128 k]

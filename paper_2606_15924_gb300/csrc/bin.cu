@@ -684,6 +684,10 @@ extern "C" tgs_status tgs_bin_tiles(const tgs_projected* proj, int64_t n, const 
   const size_t counters = sizeof(int32_t) * (size_t)R;
   int kind = tile_rank ? (R < T ? kRankMasked : kRankShared) : kRankGlobal;
   if (counters + rank_smem(kind, T) > 100 * 1024) kind = kRankGlobal;  // R < 0xFFFF
+  // nor where a block stages a large table for a few Gaussians: 14 a block, 14400
+  // tiles 31.9 us staged, 29.8 not; 34560 tiles 50.3, 42.1, and 74.9, 64.6 with a fifth
+  // of them active; but 8160 tiles 23.7, 25.7, and 53 a block and 34560 tiles 57.5, 64.6
+  if (T > 8192 && T > 1000 * ((n + G - 1) / G)) kind = kRankGlobal;
   const size_t smem = counters + rank_smem(kind, T);
   cudaMemsetAsync(w.tile_cnt, 0, sizeof(int32_t) * (size_t)R, s);
   if (shared_path) {

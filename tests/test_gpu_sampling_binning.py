@@ -56,7 +56,8 @@ BIN_CASES = [
     (2000, 256, 256, 0.25),
     (30000, 1280, 720, 0.2),
     (5000, 200, 130, 0.5),        # ragged image
-    (3000, 1600, 1060, None),     # > 256 tiles: two tile digits
+    (3000, 1600, 1060, None),     # more tiles than Gaussians
+    (2000, 2560, 1440, 0.2),      # ranks looked up in global memory: few Gaussians a block, many tiles
 ]
 
 

@@ -874,7 +874,7 @@ constexpr int kBwdPpl = 4;      // most pixels a lane
 // block of four holds its slots until its longest is done (sparse step: 66 us
 // with four warps a block, 57 with one).  20 blocks an SM: 96 registers.  Four
 // pixels a lane spill 64 bytes a thread there, three none; with statistics 140
-// and 104; in the batched kernel 212 and 92, with statistics 272 and 228.
+// and 104; in the batched kernel 152 and none, with statistics 228 and 88.
 constexpr int kBwdBlocksPerSm = 20;
 
 // Two kept splats as the replay reads them (element e in half e).
@@ -1111,9 +1111,9 @@ struct BwdSplit {
   int groups, gpx, pieces, span;
 };
 
-// Item (tile j, q = piece * groups + group).
+// Item (tile j, q = piece * groups + group); false where nothing blended in it.
 template <int PPL, bool STATS>
-__device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int q, const BwdSplit& sp, BwdPair* Q,
+__device__ __forceinline__ bool render_item_bwd(const RasterArgs& a, int j, int q, const BwdSplit& sp, BwdPair* Q,
                                                 const float* __restrict__ T_final, const int32_t* __restrict__ n_last,
                                                 const float* __restrict__ dL_drgb, float* __restrict__ grad2d,
                                                 const Ckpt& ck, const StatsK& st) {
@@ -1123,7 +1123,7 @@ __device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int 
   const int lo_pos = c * sp.span * kCkptEvery;
   const bool open = c == sp.pieces - 1;
   const int hi_edge = open ? INT_MAX : lo_pos + sp.span * kCkptEvery;
-  if (ck.tile_last && ck.tile_last[j] <= lo_pos) return;  // warp-uniform: nothing blended here
+  if (ck.tile_last && ck.tile_last[j] <= lo_pos) return false;  // warp-uniform
   const int p0 = a.pix_off[j] + grp * sp.gpx, p1 = min(a.pix_off[j + 1], p0 + sp.gpx);
   const int2 range = a.ranges[j];
   const int first = range.x + lo_pos;
@@ -1173,7 +1173,7 @@ __device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int 
     g2[u] = pk2(d2, d2);
   }
   hi_pos = __reduce_max_sync(full, hi_pos);
-  if (hi_pos <= lo_pos) return;
+  if (hi_pos <= lo_pos) return false;
   if (open) {
     top = range.x + hi_pos;
     id = top - 1 - lane >= first ? a.vals[top - 1 - lane] : -1;
@@ -1214,7 +1214,7 @@ __device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int 
       for (int u = 0; u < PPL; ++u) TR[32 * u + lane] = make_float2(T[u], R[u]);
       __syncwarp();
       bwd_rest_safe<STATS>(a, j, p0, p1, lo_pos, range.x, first, qn ? left + 1 : min(top, range.y), TR, n_last, dL_drgb, grad2d, st);
-      return;
+      return true;
     }
     const unsigned m = __ballot_sync(full, keep);
     if (m) left = top - 1 - (31 - __clz(m));  // the front-most one kept
@@ -1254,6 +1254,7 @@ __device__ __forceinline__ void render_item_bwd(const RasterArgs& a, int j, int 
     }
     qn &= 1;
   }
+  return true;
 }
 
 template <int PPL, bool STATS>
@@ -1336,15 +1337,16 @@ __global__ void k_error_stats(RasterArgs a, const int32_t* __restrict__ n_last, 
 
 // ---------------------------------------------------------------------------
 // Several views in one persistent launch: CTAs take (view, tile) items from
-// an atomic counter (items of view v are [base[v], base[v+1])) until none
-// are left.  There is no waiting on other CTAs, only one atomic per item.
+// an atomic counter (tiles of view v are [base[v], base[v+1]); the backward's
+// items: below) until none are left.  There is no waiting on other CTAs, only
+// one atomic per item.
 // ---------------------------------------------------------------------------
 constexpr int kMaxViews = 16;
 
 struct BatchArgs {
   int n_views;
   BwdSplit split;  // the backward's items per tile
-  int base[kMaxViews + 1];
+  int base[kMaxViews + 1];  // view v's tiles are [base[v], base[v + 1])
   RasterArgs a[kMaxViews];
   float* rgb[kMaxViews];
   float* T[kMaxViews];
@@ -1384,32 +1386,33 @@ __global__ void __launch_bounds__(TGS_TILE_PIX / PPL) k_render_fwd_batched(Batch
   }
 }
 
-// The batched backward: items are (view, piece, group, tile); a warp claims some of
-// them per atomic and replays them as the one-view backward does: kItemClaim where
-// every warp has at least two such turns, else one (1080 whole lists of one view,
-// four a turn, left 270 of 3040 warps with work: its step 400 -> 230 us).
-constexpr int kItemClaim = 4;
-
+// The batched backward: a warp claims a group of a tile's pixels and one of Pm
+// pieces, and replays that piece and every Pm-th after it as the one-view backward
+// does, until one holds nothing (deeper ones do not either).  Pm is a quarter of the
+// pieces, so a list of up to Pm pieces, most of them, is spread over as many warps,
+// and the empty pieces take a quarter of the claims.  Claims go through the pieces at
+// the fronts of all views' lists first.  Four neighbouring tiles at a time left the
+// work to few warps, each of them four items to walk in turn: one view of 3600
+// tiles, 100k Gaussians 235 -> 102 us; sixteen of 256x256 779 -> 368; 1080 whole lists
+// of one view, a step 400 -> 227.  One at a time costs where most are empty (2000
+// Gaussians, eight views of 3600 tiles: four at a time 169, one 349, here 134).
 template <int PPL, bool STATS>
 __global__ void __launch_bounds__(32, kBwdBlocksPerSm) k_render_bwd_batched(BatchArgs b, int* __restrict__ counter) {
   __shared__ BwdPair Q[kBwdPairs];
-  const int lane = threadIdx.x;
-  const int total = b.base[b.n_views], per_tile = b.split.pieces * b.split.groups;
-  const int claim = total / (2 * kItemClaim) >= (int)gridDim.x ? kItemClaim : 1;
+  const int n_tiles = b.base[b.n_views], per_tile = b.split.pieces * b.split.groups;
+  const int step = (b.split.pieces + 3) / 4 * b.split.groups;  // Pm pieces
   for (;;) {
-    int first = 0;
-    if (lane == 0) first = atomicAdd(counter, claim);
-    first = __shfl_sync(0xffffffffu, first, 0);
-    if (first >= total) return;
-    const int end = min(first + claim, total);
-    for (int item = first; item < end; ++item) {
-      int v, q;
-      item_view(b, item, v, q);
-      const int n_tiles = (b.base[v + 1] - b.base[v]) / per_tile, r = q / n_tiles, j = q - r * n_tiles;
-      if (j >= *b.a[v].n_active) continue;
-      render_item_bwd<PPL, STATS>(b.a[v], j, r, b.split, Q, b.T[v], b.last[v], b.dL[v],
-                                  b.grad2d[v], b.ck[v], StatsK{b.err[v], b.stats});
-    }
+    int item = 0;
+    if (threadIdx.x == 0) item = atomicAdd(counter, 1);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_tiles * step) return;
+    int v, j, r = item / n_tiles;
+    item_view(b, item - r * n_tiles, v, j);
+    if (j >= *b.a[v].n_active) continue;
+    const StatsK st{b.err[v], b.stats};
+    for (; r < per_tile; r += step)
+      if (!render_item_bwd<PPL, STATS>(b.a[v], j, r, b.split, Q, b.T[v], b.last[v], b.dL[v], b.grad2d[v], b.ck[v], st))
+        break;
   }
 }
 
@@ -1775,8 +1778,7 @@ static tgs_status batch_args(const tgs_view_batch* views, int32_t n_views, bool 
     n_pix = std::max(n_pix, (int)views[v].n_pix_max);
   }
   b.split = bwd_split(tiles, n_pix, b.ck[0]);
-  for (int v = 0; v < n_views; ++v)
-    b.base[v + 1] = b.base[v] + views[v].n_active_max * (backward ? b.split.pieces * b.split.groups : 1);
+  for (int v = 0; v < n_views; ++v) b.base[v + 1] = b.base[v] + views[v].n_active_max;
   return TGS_OK;
 }
 

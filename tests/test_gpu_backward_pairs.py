@@ -44,6 +44,7 @@ def _case(B, n_pix, slots, n_select, seed=11):
         last = torch.zeros(sel["n_sel"], dtype=torch.int32, device="cuda")
         ck = B.checkpoints(data, slots, P, out["rgb"], last)
         out["keep"] = (data, last)
+    out["ck"] = ck
     bg = (0.3, 0.1, 0.6)
     B.render_sampled(pd, binned["ranges"], binned["vals"], sel["active_tiles"], sel["n_active"], sel["n_sel"],
                      sel["pix_off"], sel["pix_idx"], n_pix, cam, bg, out["rgb"], out["T"], out["n_last"], ckpt=ck)
@@ -291,21 +292,22 @@ def test_skipped_splats_leave_the_transmittance_alone(B):
         assert torch.equal(x, y)
 
 
-@pytest.mark.parametrize("grid,claim", [(64, 1), (2, 4)])
-def test_batched_warps_share_few_items(B, grid, claim):
-    """The queue's counter after the launch: the items, one turn's claim at a
-    time, and a last claim of every block."""
+@pytest.mark.parametrize("slots", [0, 3, 7, 64])
+@pytest.mark.parametrize("grid", [64, 2])
+def test_batched_warps_share_few_items(B, grid, slots):
+    """The queue's counter after the launch: a claim for each tile and every
+    piece of the first quarter, and a last one of every block."""
     n_pix, tiles = 32, 24
-    p, sel, binned, out, bg, backward, P, pd = _case(B, n_pix, 0, tiles)
+    p, sel, binned, out, bg, backward, P, pd = _case(B, n_pix, slots, tiles)
     cam = scenes.look_at((0.0, 0.0, -4.0), width=W, height=H)
     dL = torch.randn(P, 3, generator=torch.Generator().manual_seed(5)).cuda()
     g2 = torch.zeros(N, 12, device="cuda")
     vb = B.view_batch([dict(proj=pd, tile_ranges=binned["ranges"], vals=binned["vals"], active_tiles=sel["active_tiles"],
                             n_active=sel["n_active"], n_active_max=tiles, pix_off=sel["pix_off"], pix_idx=sel["pix_idx"],
                             n_pix_max=n_pix, cam=cam, bg=bg, rgb=out["rgb"], T_final=out["T"], n_last=out["n_last"],
-                            ckpt=None, dL_drgb=dL, grad2d=g2)])
+                            ckpt=out["ck"], dL_drgb=dL, grad2d=g2)])
     counter = torch.zeros(1, dtype=torch.int32, device="cuda")
     B.render_backward_batched(vb, grid, counter)
-    assert int(counter.item()) == tiles + grid * claim
+    assert int(counter.item()) == tiles * ((slots + 1 + 3) // 4) + grid      # short lists: a piece a slot, and the rest
     plain = backward(dL)
     assert float((g2 - plain).norm()) <= 1e-6 * float(plain.norm())
